@@ -94,8 +94,8 @@ typedef struct {
 } gfm_phys;
 
 typedef enum {
-    GFM_FP64 = 0,  /* Jacobi-PCG entirely in FP64                                       */
-    GFM_MIXED = 1  /* FP32 inner Jacobi-PCG (FP64-accurate dot sums) inside FP64
+    GFM_FP64 = 0,  /* preconditioned CG entirely in FP64                                */
+    GFM_MIXED = 1  /* FP32 inner preconditioned CG (FP64-accurate dot sums) inside FP64
                       iterative refinement: true residual, correction and the jump
                       source stay FP64                                                  */
 } gfm_mode;
@@ -470,8 +470,10 @@ gfm_status gfm_set_table(gfm_handle h, int32_t compact, int32_t force_stream);
 gfm_status gfm_get_table(gfm_handle h, int32_t *compact_usable, int32_t *n_classes, int32_t *compact_valid);
 
 /* Launch shape of the persistent kernels (threads a multiple of 32, at most
- * 512) and the form of the mixed-precision iteration.  A zero field keeps
- * the current value.  Both forms run the same preconditioned CG recurrences
+ * 512) and the form of the mixed-precision Jacobi iteration (gfm_set_coarse(0)
+ * and unpinned systems; the multigrid solve has one form).  A zero field
+ * keeps the current value.  The default shape {512, 1} lets the multigrid
+ * solve take up to 1024 threads in its one CTA per SM.  Both forms run the same preconditioned CG recurrences
  * of the pinned system of Sec. 3.1 (the paper names no solver) with the same
  * FP64 residual replacement and stopping rules.  Form 1 applies each FP32
  * iteration as an operator pass (p = u + beta p, s = A p, p.s) and an update
@@ -491,10 +493,10 @@ gfm_status gfm_get_tuning(gfm_handle h, gfm_tuning *t);
  * Autotuner: on the assembled system, time `trials` solves (median, CUDA
  * events on `stream`) with opts for each launch shape of the persistent
  * kernel ({512,1}, {256,2}, {128,4}, {384,1}, {256,1} threads x CTAs per
- * SM, where co-resident), and for a single mesh in GFM_MIXED mode with both
- * iteration forms (gfm_set_tuning).  For a batched handle it also tries the tank->CTA
- * table weighted by the iterations each tank took (tanks that iterate longer
- * get more CTAs).  The fastest shape and table are kept for later solves and
+ * SM, where co-resident); with Jacobi iterations, for a single mesh in
+ * GFM_MIXED mode both forms (gfm_set_tuning), and for a batched handle also the
+ * tank->CTA table weighted by the iterations each tank took (tanks that
+ * iterate longer get more CTAs).  The fastest shape and table are kept for later solves and
  * returned in *chosen and *best_ms (either may be NULL).  The paper has no
  * counterpart; tuning changes how the work is split, not what is computed.
  * The trial solutions go to the handle's own workspace; synchronises
@@ -506,20 +508,21 @@ gfm_status gfm_autotune(gfm_handle h, const gfm_solve_opts *opts, int32_t trials
                         gfm_stream stream);
 
 /*
- * Two-level preconditioner.  With a density ratio of 1000 the ghost-fluid
- * Laplacian (Sec. 3.1) couples each connected region of one phase to the rest
- * only through its interface faces, and Jacobi-PCG stalls for thousands of
- * iterations on the near-constant modes of the large regions.  Every
- * assembly finds the connected regions of each phase (cells joined by
- * non-interface faces) and keeps the up-to-max_vectors largest with at least
- * min_size cells as coarse space Z; the preconditioner is then
- * D^{-1} + Z (Z^T A Z)^{-1} Z^T.  max_vectors = 0 gives plain Jacobi.
- * Defaults: 8 vectors, 64 cells.  Takes effect at the next gfm_assemble.
- * The coarse space needs a pin (ref_cell >= 0); unpinned systems use Jacobi.
- * On a batched handle each tank keeps up to min(max_vectors, 2) regions of
- * its own (default 2).  gfm_get_coarse reports (host pointers, synchronises
- * `stream`) the vectors in use (summed over the tanks of a batch), the
- * regions of at least min_size cells, and the sizes [8] of the first kept ones.
+ * Preconditioner.  With a density ratio of 1000 the ghost-fluid Laplacian
+ * (Sec. 3.1) couples each connected region of one phase to the rest only
+ * through its interface faces, and Jacobi-PCG takes thousands of iterations.
+ * Every pinned system (ref_cell >= 0) is preconditioned by one symmetric
+ * multigrid V-cycle: gfm_create merges cells into aggregates level by level
+ * from the geometry, every assembly forms the coarse operators from gamma_f.
+ * max_vectors = 0 gives plain Jacobi from the next gfm_assemble on, any other
+ * value multigrid (the default); unpinned systems take Jacobi.
+ * gfm_get_coarse reports (host pointers, synchronises `stream`) the connected
+ * one-phase regions of the last assembled system (cells joined by
+ * non-interface faces): how many of at least min_size cells there are, how
+ * many of them, the largest ones, are counted (up to max_vectors; up to
+ * min(max_vectors, 2) per tank of a batch, summed over the tanks; 0 with
+ * plain Jacobi), and the sizes [8] of the first of these.
+ * Defaults: 8 vectors, 64 cells.
  */
 gfm_status gfm_set_coarse(gfm_handle h, int32_t max_vectors, int32_t min_size);
 gfm_status gfm_get_coarse(gfm_handle h, int32_t *n_vectors, int32_t *n_regions, int32_t *sizes, gfm_stream stream);

@@ -448,11 +448,11 @@ class GFM:
         return t.threads, t.ctas_per_sm, float(ms.value)
 
     def set_coarse(self, max_vectors: int = 8, min_size: int = 64):
-        """Coarse space of the two-level preconditioner (0 vectors = Jacobi only); next assembly on."""
+        """0 vectors: plain Jacobi instead of multigrid, from the next assembly on (gfm_set_coarse)."""
         self._check(self.lib.gfm_set_coarse(self.h, int(max_vectors), int(min_size)), "gfm_set_coarse")
 
     def coarse_info(self, stream=None):
-        """(vectors in use, regions of at least min_size cells, sizes of the kept regions)."""
+        """(one-phase regions counted, regions of at least min_size cells, sizes of the counted ones)."""
         import numpy as np
         k, nr = ct.c_int32(), ct.c_int32()
         sizes = np.zeros(8, dtype=np.int32)

@@ -27,12 +27,14 @@ UNITS = {
     "gfm_solve.cu": ["-Xptxas", "-v"],
     "gfm_coarse.cu": [],
     "gfm_setup.cpp": [],
+    "gfm_mg.cu": ["-Xptxas", "-v"],
+    "gfm_mg_setup.cpp": [],
     "gfm_noalloc.cu": ["-Xptxas", "-v"],
     "gfm_shard.cpp": [],
     "gfm_gradient.cu": [],
     "gfm_iso.cu": [],
 }
-HEADERS = ["gfm_internal.h", "gfm_setup.h"]
+HEADERS = ["gfm_internal.h", "gfm_grid.cuh", "gfm_setup.h", "gfm_mg_setup.h"]
 
 
 def nvcc() -> str:

@@ -4,13 +4,27 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <exception>
+#include <future>
 #include <new>
 #include <string>
+#include <system_error>
 #include <unordered_map>
 #include <vector>
 
 #include "gfm_internal.h"
+#include "gfm_mg_setup.h"
 #include "gfm_setup.h"
+
+// One coarse multigrid level on the device.
+struct MgDev {
+    int n = 0, n_slices = 0;
+    int32_t *sp = nullptr, *col = nullptr, *face = nullptr, *cp = nullptr, *child = nullptr;
+    int32_t *mem_ptr = nullptr, *mem = nullptr;
+    double *scale = nullptr, *gamma = nullptr, *val64 = nullptr, *pin64 = nullptr, *dinv64 = nullptr;
+    float *val32 = nullptr, *pin32 = nullptr, *dinv32 = nullptr;
+    double *b = nullptr, *xa = nullptr, *xb = nullptr, *res = nullptr;  // vectors (FP64 or FP32)
+};
 
 struct gfm_ctx {
     int device = 0;
@@ -47,6 +61,10 @@ struct gfm_ctx {
     gfm::Coarse *coarse = nullptr;
     int max_cross = 0;
     int coarse_max = gfm::kMaxCoarse, coarse_min_size = 64;
+    int asm_max = 0, asm_min_size = 64;  // the same as the last assembly took them
+    // multigrid hierarchy; used by pinned systems unless gfm_set_coarse(0)
+    std::vector<MgDev> mg;
+    bool mg_valid = false;  // the last assembly formed the coarse levels
     // batch of tanks (gfm_create_batched)
     bool batched = false;
     int T = 0, cta_grid = 0;
@@ -139,6 +157,12 @@ void free_all(gfm_ctx *h)
                     h->grad_scr, h->ent, h->fcls, h->ctank, h->ccls, h->dict};
     for (void *p : ptrs)
         if (p) cudaFree(p);
+    for (MgDev &l : h->mg) {
+        void *lp[] = {l.sp, l.col, l.face, l.cp, l.child, l.mem_ptr, l.mem, l.scale, l.gamma, l.val64, l.pin64,
+                      l.dinv64, l.val32, l.pin32, l.dinv32, l.b, l.xa, l.xb, l.res};
+        for (void *p : lp)
+            if (p) cudaFree(p);
+    }
     void *hptrs[] = {h->hinfo, h->tphys_h, h->tprm_h, h->binfos_h};
     for (void *p : hptrs)
         if (p) cudaFreeHost(p);
@@ -306,6 +330,35 @@ float prof_elapsed(gfm_ctx *h, int a, int b)
 // outside the library so that it is not reported as this call's failure.
 void clear_stale_error() { (void)cudaGetLastError(); }
 
+// Launch shape of the multigrid solve.  The default tuning (512 x 1) takes
+// the most threads the kernel allows in one CTA per SM (1024 in FP32, 512 in
+// FP64): its passes are bound by gather latency.  Other tunings are taken as
+// they are.  A small mesh gets a CTA per 8 slices, since every CTA more makes
+// the grid barriers dearer.
+gfm_status plan_mg(gfm_ctx *h, gfm::Mode mode, const void **kernel, int *grid, int *threads)
+{
+    int most = 0;
+    *kernel = gfm::mg_kernel(mode == gfm::Mode::MIXED, h->ht.max_width, &most);
+    const bool standard = h->tuning.threads == 512 && h->tuning.ctas_per_sm == 1;
+    int t = standard ? most : std::min(h->tuning.threads, most), per = h->tuning.ctas_per_sm;
+    int occ = 0;
+    GFM_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, *kernel, t, 0));
+    if (occ < 1) return fail(h, GFM_ERR_ARG, "multigrid kernel cannot run with this many threads per CTA");
+    per = std::min(per, occ);
+    *grid = std::max(1, std::min(h->sm_count * per, (h->ht.n_slices + 7) / 8));
+    *threads = t;
+    return GFM_OK;
+}
+
+// Slices below which a level runs in CTA 0 alone.
+int mg_tail(const gfm_ctx *h, gfm::Mode mode)
+{
+    const int most = mode == gfm::Mode::MIXED ? 64 : 16;
+    int l = 0;
+    while (l < (int)h->mg.size() && h->mg[(size_t)l].n_slices > most) ++l;
+    return l + 1;
+}
+
 // Enqueue one persistent solve of A x = rhs (internal order) writing the
 // solution in caller order to out_user.  info_dev receives the result.
 gfm_status enqueue_solve(gfm_ctx *h, const gfm_solve_opts *o, const double *rhs, double *out_user, int use_x0,
@@ -313,9 +366,17 @@ gfm_status enqueue_solve(gfm_ctx *h, const gfm_solve_opts *o, const double *rhs,
 {
     const gfm::Mode mode = (o->mode == GFM_MIXED) ? gfm::Mode::MIXED : gfm::Mode::FP64;
     LaunchPlan lp;
-    gfm_status st = plan_launch(h, mode, &lp);
-    if (st != GFM_OK) return st;
-    const int grid = lp.grid, threads = lp.threads;
+    const void *mgk = nullptr;
+    int grid = 0, threads = 0;
+    if (h->mg_valid) {
+        gfm_status st = plan_mg(h, mode, &mgk, &grid, &threads);
+        if (st != GFM_OK) return st;
+    } else {
+        gfm_status st = plan_launch(h, mode, &lp);
+        if (st != GFM_OK) return st;
+        grid = lp.grid;
+        threads = lp.threads;
+    }
     GFM_CUDA(h, cudaMemsetAsync(h->bar, 0, sizeof(unsigned), s));
     GFM_CUDA(h, cudaMemsetAsync(h->err, 0, sizeof(int), s));
     GFM_CUDA(h, cudaMemsetAsync(info_dev, 0, sizeof(gfm_solve_info), s));
@@ -372,9 +433,57 @@ gfm_status enqueue_solve(gfm_ctx *h, const gfm_solve_opts *o, const double *rhs,
         kernel = gfm::batched_kernel(h->ht.max_width, lp.n_stages > 0, lp.ct);
         GFM_CUDA(h, cudaMemsetAsync(info_dev, 0, sizeof(gfm_solve_info) * h->T, s));
     }
-    void *args[] = {&a, &ba};
+    gfm::MgArgs m{};
+    if (h->mg_valid) {
+        m.s = a;
+        m.L = (int)h->mg.size() + 1;
+        m.tail = mg_tail(h, mode);
+        m.T = h->batched ? h->T : 1;
+        m.tank_off = h->tioff;
+        m.tprm = h->tprm;
+        const bool mixed = mode == gfm::Mode::MIXED;
+        const size_t np = (size_t)h->ht.n_pad;
+        auto second = [&](void *p) -> void * {  // the second of a buffer's two vectors
+            return mixed ? (void *)((float *)p + np) : (void *)((double *)p + np);
+        };
+        void *v0 = mixed ? (void *)h->UP0 : (void *)h->Q0, *v1 = mixed ? (void *)h->UP1 : (void *)h->Q1;
+        gfm::MgLevel &l0 = m.lv[0];
+        l0.n = h->n;
+        l0.n_slices = h->ht.n_slices;
+        l0.sp = h->slice_ptr;
+        l0.col = h->col;
+        l0.val = mixed ? (const void *)h->val32 : (const void *)h->val64;
+        l0.dinv = mixed ? (const void *)h->dinv32 : (const void *)h->dinv;
+        l0.b = mixed ? (void *)h->R32 : (void *)h->r64;
+        l0.xa = v0;
+        l0.xb = second(v0);
+        l0.res = v1;
+        m.z = second(v1);
+        m.p = mixed ? (void *)h->P32 : (void *)h->p64;
+        m.sv = mixed ? (void *)h->S32 : (void *)h->q64;
+        m.e = h->E;
+        for (size_t l = 0; l < h->mg.size(); ++l) {
+            const MgDev &d = h->mg[l];
+            gfm::MgLevel &lv = m.lv[l + 1];
+            lv.n = d.n;
+            lv.n_slices = d.n_slices;
+            lv.sp = d.sp;
+            lv.col = d.col;
+            lv.val = mixed ? (const void *)d.val32 : (const void *)d.val64;
+            lv.dinv = mixed ? (const void *)d.dinv32 : (const void *)d.dinv64;
+            lv.pin = mixed ? (const void *)d.pin32 : (const void *)d.pin64;
+            lv.cp = d.cp;
+            lv.child = d.child;
+            lv.b = d.b;
+            lv.xa = d.xa;
+            lv.xb = d.xb;
+            lv.res = d.res;
+        }
+        kernel = mgk;
+    }
+    void *jargs[] = {&a, &ba}, *margs[] = {&m};
     prof_record(h, 2, s);
-    GFM_CUDA(h, cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(threads), args, lp.dyn, s));
+    GFM_CUDA(h, cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(threads), h->mg_valid ? margs : jargs, lp.dyn, s));
     prof_record(h, 3, s);
     h->prof.grid = grid;
     h->prof.threads = threads;
@@ -568,6 +677,70 @@ gfm_status setup_compact(gfm_ctx *h, cudaStream_t s)
     return GFM_OK;
 }
 
+// The multigrid levels of a host mesh (caller order: owner, neighbour, Sf
+// [3][F], C [3][n]; its arrays outlive the result), built on a host thread
+// while the calling thread uploads the tables.
+using MgFuture = std::future<std::vector<gfm::MgLevelHost>>;
+MgFuture start_mg(const gfm_ctx *h, const std::vector<int32_t> &owner, const std::vector<int32_t> &nb,
+                  const std::vector<double> &Sf, const std::vector<double> &C)
+{
+    static_assert(gfm::kMgLevels == gfm::kMgMaxLevels, "level limits differ");
+    auto build = [h, &owner, &nb, &Sf, &C]() {
+        return gfm::build_mg_levels(h->n, h->ht.n_pad, h->F, owner.data(), nb.data(), Sf.data(), C.data(),
+                                    h->ht.perm.data());
+    };
+    try {
+        return std::async(std::launch::async, build);
+    } catch (const std::system_error &) {  // no thread to be had: built when asked for
+        return std::async(std::launch::deferred, build);
+    }
+}
+
+// Upload the levels with their workspace.
+gfm_status setup_mg(gfm_ctx *h, MgFuture &built, cudaStream_t s)
+{
+    std::vector<gfm::MgLevelHost> lv;
+    try {
+        lv = built.get();
+    } catch (const std::exception &) {
+        return fail(h, GFM_ERR_NOMEM, "multigrid hierarchy");
+    }
+    h->mg.resize(lv.size());
+    cudaError_t e = cudaSuccess;
+    auto up = [&](auto **dst, const auto &src) {
+        if (e == cudaSuccess) e = dalloc(dst, src.size());
+        if (e == cudaSuccess && !src.empty())
+            e = cudaMemcpyAsync(*dst, src.data(), sizeof(src[0]) * src.size(), cudaMemcpyHostToDevice, s);
+    };
+    for (size_t l = 0; l < lv.size(); ++l) {
+        const gfm::MgLevelHost &q = lv[l];
+        MgDev &d = h->mg[l];
+        d.n = q.n;
+        d.n_slices = q.n_slices;
+        up(&d.sp, q.slice_ptr);
+        up(&d.col, q.col);
+        up(&d.face, q.face);
+        up(&d.cp, q.child_ptr);
+        up(&d.child, q.child);
+        up(&d.mem_ptr, q.mem_ptr);
+        up(&d.mem, q.mem);
+        up(&d.scale, q.scale);
+        const size_t np = (size_t)q.n_pad, ns = (size_t)q.n_slots;
+#define A(ptr, cnt) \
+    if (e == cudaSuccess) e = dalloc(&d.ptr, (cnt))
+        A(gamma, (size_t)q.F); A(val64, ns); A(val32, ns); A(pin64, np); A(pin32, np); A(dinv64, np); A(dinv32, np);
+        A(b, np); A(xa, np); A(xb, np); A(res, np);
+#undef A
+        double *zero[] = {d.b, d.xa, d.xb, d.res};
+        for (double *z : zero)
+            if (e == cudaSuccess) e = cudaMemsetAsync(z, 0, sizeof(double) * np, s);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaErrorMemoryAllocation) return fail(h, GFM_ERR_NOMEM, "multigrid workspace");
+    if (e != cudaSuccess) return cuda_fail(h, e, "multigrid set-up");
+    return GFM_OK;
+}
+
 // Batch-only workspace: tank of every face and slice, per-tank physics,
 // pins, cell counts and results, CTA table.
 gfm_status alloc_batch(gfm_ctx *h, cudaStream_t s)
@@ -612,6 +785,43 @@ gfm_status plan_batch(gfm_ctx *h)
     if (e != cudaSuccess) return cuda_fail(h, e, "uploading the CTA table");
     h->cta_grid = grid;
     return GFM_OK;
+}
+
+gfm::CoarseArgs coarse_args(gfm_ctx *h)
+{
+    gfm::CoarseArgs co{};
+    co.n = h->n;
+    co.F = h->F;
+    co.n_pad = h->ht.n_pad;
+    co.owner = h->owner;
+    co.neighbour = h->neighbour;
+    co.perm = h->perm;
+    co.kind = h->kind;
+    co.gamma = h->gamma;
+    co.ref = h->ref_internal;
+    co.max_k = h->asm_max;
+    co.min_size = h->asm_min_size;
+    co.max_cross = h->max_cross;
+    co.prm = h->prm;
+    co.parent = h->cc_parent;
+    co.csize = h->cc_size;
+    co.cand = h->cc_cand;
+    co.counters = h->cc_counters;
+    co.bcount = h->cc_bcount;
+    co.boff = h->cc_boff;
+    co.epart = h->cc_epart;
+    co.comp = h->comp;
+    co.cross = h->cross;
+    co.coarse = h->coarse;
+    if (h->batched) {  // one coarse space per tank
+        co.T = h->T;
+        co.coff = h->tcoff;
+        co.ioff = h->tioff;
+        co.tprm = h->tprm;
+        co.tco = h->tco;
+        co.max_k = std::min(h->asm_max, gfm::kTankCoarse);
+    }
+    return co;
 }
 
 }  // namespace
@@ -668,32 +878,29 @@ gfm_status gfm_create(const gfm_mesh *mesh, int32_t renumber, gfm_stream stream,
     do {
         if (st != GFM_OK) break;
         std::vector<int32_t> ho((size_t)F), hn((size_t)F);
-        std::vector<double> hC;
+        std::vector<double> hC((size_t)3 * n), hS((size_t)3 * F);
         if (cudaMemcpyAsync(ho.data(), mesh->owner, sizeof(int32_t) * F, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaMemcpyAsync(hn.data(), mesh->neighbour, sizeof(int32_t) * F, cudaMemcpyDeviceToHost, s) !=
                 cudaSuccess) {
             st = fail(h, GFM_ERR_CUDA, "reading owner/neighbour (must be device pointers)");
             break;
         }
-        if (renumber == 2) {
-            hC.resize((size_t)3 * n);
-            if (cudaMemcpyAsync(hC.data(), mesh->C, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, s) !=
-                cudaSuccess) {
-                st = fail(h, GFM_ERR_CUDA, "reading cell centres");
-                break;
-            }
+        if (cudaMemcpyAsync(hC.data(), mesh->C, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+            cudaMemcpyAsync(hS.data(), mesh->Sf, sizeof(double) * 3 * F, cudaMemcpyDeviceToHost, s) != cudaSuccess) {
+            st = fail(h, GFM_ERR_CUDA, "reading the mesh geometry (must be device pointers)");
+            break;
         }
         if (cudaStreamSynchronize(s) != cudaSuccess) {
             st = fail(h, GFM_ERR_CUDA, "synchronising stream");
             break;
         }
         std::string err;
-        if (!gfm::build_host_tables(n, F, ho.data(), hn.data(), hC.empty() ? nullptr : hC.data(), renumber, h->ht,
-                                    err)) {
+        if (!gfm::build_host_tables(n, F, ho.data(), hn.data(), hC.data(), renumber, h->ht, err)) {
             st = fail(h, GFM_ERR_ARG, err);
             break;
         }
         h->ht.iperm.resize((size_t)h->ht.n_pad, -1);  // padding cells
+        MgFuture mg = start_mg(h, ho, hn, hS, hC);
         st = alloc_upload(h, s);
         if (st != GFM_OK) break;
         cudaError_t e = cudaMemcpyAsync(h->owner, mesh->owner, sizeof(int32_t) * F, cudaMemcpyDeviceToDevice, s);
@@ -706,6 +913,8 @@ gfm_status gfm_create(const gfm_mesh *mesh, int32_t renumber, gfm_stream stream,
             break;
         }
         st = setup_compact(h, s);
+        if (st != GFM_OK) break;
+        st = setup_mg(h, mg, s);
     } while (0);
     if (st != GFM_OK) {
         fprintf(stderr, "gfm_create: %s\n", h->last_error.c_str());
@@ -735,7 +944,7 @@ gfm_status gfm_create_batched(const gfm_mesh *meshes, int32_t n_tanks, int32_t r
     do {
         if (st != GFM_OK) break;
         std::vector<std::vector<int32_t>> ho((size_t)n_tanks), hn((size_t)n_tanks);
-        std::vector<std::vector<double>> hC((size_t)n_tanks);
+        std::vector<std::vector<double>> hC((size_t)n_tanks), hS((size_t)n_tanks);
         long long ncell = 0, nface = 0;
         for (int t = 0; t < n_tanks; ++t) {
             const gfm_mesh &m = meshes[t];
@@ -746,11 +955,14 @@ gfm_status gfm_create_batched(const gfm_mesh *meshes, int32_t n_tanks, int32_t r
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(hn[(size_t)t].data(), m.neighbour, sizeof(int32_t) * m.n_faces,
                                     cudaMemcpyDeviceToHost, s);
-            if (e == cudaSuccess && renumber == 2) {
-                hC[(size_t)t].resize((size_t)3 * m.n_cells);
+            hC[(size_t)t].resize((size_t)3 * m.n_cells);
+            hS[(size_t)t].resize((size_t)3 * m.n_faces);
+            if (e == cudaSuccess)
                 e = cudaMemcpyAsync(hC[(size_t)t].data(), m.C, sizeof(double) * 3 * m.n_cells, cudaMemcpyDeviceToHost,
                                     s);
-            }
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(hS[(size_t)t].data(), m.Sf, sizeof(double) * 3 * m.n_faces, cudaMemcpyDeviceToHost,
+                                    s);
             if (e != cudaSuccess) {
                 st = cuda_fail(h, e, "reading tank meshes (must be device pointers)");
                 break;
@@ -770,7 +982,7 @@ gfm_status gfm_create_batched(const gfm_mesh *meshes, int32_t n_tanks, int32_t r
         std::vector<gfm::TankMesh> tm((size_t)n_tanks);
         for (int t = 0; t < n_tanks; ++t)
             tm[(size_t)t] = gfm::TankMesh{meshes[t].n_cells, meshes[t].n_faces, ho[(size_t)t].data(),
-                                          hn[(size_t)t].data(), hC[(size_t)t].empty() ? nullptr : hC[(size_t)t].data()};
+                                          hn[(size_t)t].data(), hC[(size_t)t].data()};
         std::string err;
         if (!gfm::build_batch_tables(tm, renumber, h->ht, h->bt, err)) {
             st = fail(h, GFM_ERR_ARG, err);
@@ -781,10 +993,6 @@ gfm_status gfm_create_batched(const gfm_mesh *meshes, int32_t n_tanks, int32_t r
         h->batched = true;
         h->T = n_tanks;
         h->coarse_max = gfm::kTankCoarse;  // per tank: the water body and the air above it
-        st = alloc_upload(h, s);
-        if (st != GFM_OK) break;
-        st = alloc_batch(h, s);
-        if (st != GFM_OK) break;
         // caller-order concatenated mesh: indices offset by the tanks' cell offsets
         std::vector<int32_t> co((size_t)h->F), cn((size_t)h->F);
         for (int t = 0; t < n_tanks; ++t) {
@@ -794,6 +1002,18 @@ gfm_status gfm_create_batched(const gfm_mesh *meshes, int32_t n_tanks, int32_t r
                 cn[(size_t)f0 + f] = hn[(size_t)t][(size_t)f] + c0;
             }
         }
+        std::vector<double> cS((size_t)3 * h->F), cC((size_t)3 * h->n);
+        for (int t = 0; t < n_tanks; ++t)
+            for (int k = 0; k < 3; ++k) {
+                const int nt = meshes[t].n_cells, ft = meshes[t].n_faces;
+                std::copy_n(hS[(size_t)t].data() + (size_t)k * ft, ft, cS.data() + (size_t)k * h->F + h->bt.foff[(size_t)t]);
+                std::copy_n(hC[(size_t)t].data() + (size_t)k * nt, nt, cC.data() + (size_t)k * h->n + h->bt.coff[(size_t)t]);
+            }
+        MgFuture mg = start_mg(h, co, cn, cS, cC);
+        st = alloc_upload(h, s);
+        if (st != GFM_OK) break;
+        st = alloc_batch(h, s);
+        if (st != GFM_OK) break;
         cudaError_t e = cudaMemcpyAsync(h->owner, co.data(), sizeof(int32_t) * h->F, cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(h->neighbour, cn.data(), sizeof(int32_t) * h->F, cudaMemcpyHostToDevice, s);
         for (int t = 0; t < n_tanks && e == cudaSuccess; ++t) {
@@ -812,6 +1032,8 @@ gfm_status gfm_create_batched(const gfm_mesh *meshes, int32_t n_tanks, int32_t r
             break;
         }
         st = setup_compact(h, s);
+        if (st != GFM_OK) break;
+        st = setup_mg(h, mg, s);
         if (st != GFM_OK) break;
         st = plan_batch(h);
     } while (0);
@@ -934,40 +1156,44 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
     ca.pad_code = 2 * h->n_cls;
     GFM_CUDA(h, gfm::launch_cells(ca, s));
     h->ent_valid = use_ct;
-    {
-        gfm::CoarseArgs co{};
-        co.n = h->n;
-        co.F = h->F;
-        co.n_pad = h->ht.n_pad;
-        co.owner = h->owner;
-        co.neighbour = h->neighbour;
-        co.perm = h->perm;
-        co.kind = h->kind;
-        co.gamma = h->gamma;
-        co.ref = h->ref_internal;
-        co.max_k = h->coarse_max;
-        co.min_size = h->coarse_min_size;
-        co.max_cross = h->max_cross;
-        co.prm = h->prm;
-        co.parent = h->cc_parent;
-        co.csize = h->cc_size;
-        co.cand = h->cc_cand;
-        co.counters = h->cc_counters;
-        co.bcount = h->cc_bcount;
-        co.boff = h->cc_boff;
-        co.epart = h->cc_epart;
-        co.comp = h->comp;
-        co.cross = h->cross;
-        co.coarse = h->coarse;
-        if (h->batched) {  // one coarse space per tank
-            co.T = h->T;
-            co.coff = h->tcoff;
-            co.ioff = h->tioff;
-            co.tprm = h->tprm;
-            co.tco = h->tco;
-            co.max_k = std::min(h->coarse_max, gfm::kTankCoarse);
+    // A pinned system is preconditioned by multigrid, whose coarse levels
+    // follow from gamma; the one-phase regions are then only reported
+    // (gfm_get_coarse finds them).  Unpinned systems and gfm_set_coarse(0)
+    // take the Jacobi forms.
+    h->mg_valid = false;
+    h->asm_max = h->coarse_max;
+    h->asm_min_size = h->coarse_min_size;
+    if (h->ref_internal >= 0 && h->coarse_max > 0) {
+        for (size_t l = 0; l < h->mg.size(); ++l) {
+            const MgDev &d = h->mg[l];
+            gfm::MgLevelArgs ma{};
+            ma.n_slices = d.n_slices;
+            ma.sp = d.sp;
+            ma.col = d.col;
+            ma.face = d.face;
+            ma.cp = d.cp;
+            ma.child = d.child;
+            ma.mem_ptr = d.mem_ptr;
+            ma.mem = d.mem;
+            ma.scale = d.scale;
+            ma.fine_gamma = l == 0 ? h->gamma : h->mg[l - 1].gamma;
+            ma.fine_pin = l == 0 ? nullptr : h->mg[l - 1].pin64;
+            ma.prm = h->prm;
+            ma.stank = h->batched ? h->stank : nullptr;
+            ma.tprm = h->tprm;
+            ma.gamma = d.gamma;
+            ma.val64 = d.val64;
+            ma.pin64 = d.pin64;
+            ma.dinv64 = d.dinv64;
+            ma.val32 = d.val32;
+            ma.pin32 = d.pin32;
+            ma.dinv32 = d.dinv32;
+            GFM_CUDA(h, gfm::launch_mg_level(ma, s));
+            ++launched;
         }
-        GFM_CUDA(h, gfm::launch_coarse(co, s, &launched));
+        h->mg_valid = true;
+    } else {
+        GFM_CUDA(h, gfm::launch_coarse(coarse_args(h), s, &launched));
     }
     if (h->ref_internal < 0) {  // only an unpinned system needs sum(b) for its compatibility test
         GFM_CUDA(h, gfm::launch_bsums(h->b, h->n, h->prm, s));
@@ -1455,7 +1681,7 @@ gfm_status gfm_autotune(gfm_handle h, const gfm_solve_opts *opts, int32_t trials
     const int shapes[][2] = {{512, 1}, {256, 2}, {128, 4}, {384, 1}, {256, 1}};
     std::vector<gfm_tuning> cands;
     // a single mesh in MIXED mode also tries the fused form with every shape
-    const int n_forms = (!h->batched && opts->mode == GFM_MIXED) ? 2 : 1;
+    const int n_forms = (!h->batched && !h->mg_valid && opts->mode == GFM_MIXED) ? 2 : 1;
     for (int f = 1; f <= n_forms; ++f)
         for (const auto &sh : shapes) cands.push_back(gfm_tuning{sh[0], sh[1], f});
     gfm_tuning best = start;
@@ -1474,7 +1700,7 @@ gfm_status gfm_autotune(gfm_handle h, const gfm_solve_opts *opts, int32_t trials
             best_iters = it;
         }
     }
-    if (st == GFM_OK && h->batched && best_t > 0.0f && gfm_set_tuning(h, &best) == GFM_OK) {
+    if (st == GFM_OK && h->batched && !h->mg_valid && best_t > 0.0f && gfm_set_tuning(h, &best) == GFM_OK) {
         // the tank table weighted by the iterations each tank took
         h->bweight.assign(best_iters.begin(), best_iters.end());
         float ms = 0.0f;
@@ -1519,6 +1745,8 @@ gfm_status gfm_get_coarse(gfm_handle h, int32_t *n_vectors, int32_t *n_regions, 
     if (!h) return GFM_ERR_ARG;
     gfm::Coarse co;
     cudaStream_t s = (cudaStream_t)stream;
+    // a multigrid solve does not need the regions: find those of the last assembly
+    if (h->mg_valid) GFM_CUDA(h, gfm::launch_coarse(coarse_args(h), s, nullptr));
     GFM_CUDA(h, cudaMemcpyAsync(&co, h->coarse, sizeof co, cudaMemcpyDeviceToHost, s));
     if (h->batched) {  // vectors summed over the tanks; sizes of the first tanks' vectors
         std::vector<gfm::TankCoarse> tc((size_t)h->T);

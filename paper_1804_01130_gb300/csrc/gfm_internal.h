@@ -305,6 +305,45 @@ struct BatchArgs {
 };
 const void *batched_kernel(int max_width, bool streamed = false, bool compact = false);
 
+// ---- multigrid (gfm_mg.cu) -------------------------------------------------
+constexpr int kMgLevels = 24;  // levels of a hierarchy, the mesh included
+
+// One level as the V-cycle sees it; the typed pointers are float or double
+// with the solve's precision.  Level 0 is the mesh.
+struct MgLevel {
+    int32_t n, n_slices;
+    const int32_t *sp, *col;    // sliced-ELL graph
+    const void *val, *dinv;     // coefficients per slot, 1 / diagonal
+    const void *pin;            // pin per node (coarse levels)
+    const int32_t *cp, *child;  // children in the next finer level (coarse levels)
+    void *b, *xa, *xb, *res;    // right-hand side, iterates, residual
+};
+
+struct MgArgs {
+    SolveArgs s;
+    int32_t L;       // levels
+    int32_t tail;    // levels from this one on run in CTA 0 alone
+    int32_t T;       // tanks (1: a single mesh)
+    const int32_t *tank_off;  // batched: [T+1] internal cell offsets
+    const DevParams *tprm;    // batched: pin of each tank
+    void *z, *p, *sv, *e;     // z = M^{-1} r, direction, A p, FP32 correction
+    MgLevel lv[kMgLevels];
+};
+const void *mg_kernel(bool mixed, int max_width, int *max_threads);
+
+struct MgLevelArgs {
+    int32_t n_slices;
+    const int32_t *sp, *col, *face, *cp, *child, *mem_ptr, *mem;
+    const double *scale, *fine_gamma;
+    const double *fine_pin;   // nullptr on the first coarse level: the pinned cell of prm / tprm
+    const DevParams *prm;
+    const int32_t *stank;     // batched: tank of each mesh slice (else nullptr)
+    const DevParams *tprm;
+    double *gamma, *val64, *pin64, *dinv64;
+    float *val32, *pin32, *dinv32;
+};
+cudaError_t launch_mg_level(const MgLevelArgs &a, cudaStream_t s);
+
 enum class Mode { FP64 = 0, MIXED = 1 };
 const void *solver_kernel(Mode m, int max_width, int threads, bool streamed = false, bool compact = false,
                           bool fused = false);

@@ -1,0 +1,972 @@
+// Multigrid-preconditioned conjugate gradients for the pinned GFM pressure
+// system (Sec. 3.1; the paper names no solver), one persistent cooperative
+// kernel per solve, for one mesh or a batch of tanks.
+//
+// Preconditioner: one symmetric V-cycle over the aggregates of
+// gfm_mg_setup.cpp.  On each level two damped Jacobi sweeps before and after
+// the coarse correction, with the two weights of the degree-2 Chebyshev
+// polynomial on [0.35, 2] (the spectrum of D^{-1} A is in [0, 2]) in mirrored
+// order, piecewise constant transfers, and the coarse operator formed by
+// every assembly from the assembled face coefficients (k_mg_level).  The
+// iteration count hardly depends on the mesh size: 20-40 V-cycles for a
+// relative residual of 1e-12 where Jacobi with the deflated one-phase
+// regions took 270 (64x32 tank) to 4300 (1024x512 tank).
+//
+// A V-cycle on the mesh level is five passes over the rows (two sweeps, the
+// residual, two sweeps), all of them gathers of ONE vector, against the one
+// pass of a Jacobi iteration; the coarse levels add a third (2D) or a
+// seventh (3D).  A is applied in difference form, sum_f gamma_f (x_i - x_j) +
+// pin_i x_i, which keeps the zero row sums of the GFM Laplacian exact.  The
+// CG direction needs no pass of its own gathers: s = A p is updated as
+// s = A z + beta s.
+//
+// Precision.  GFM_FP64 (T = double): everything FP64; the result is accepted
+// on the true residual b - A x.  GFM_MIXED (T = float): FP32 iterations with
+// double-float dot products inside FP64 residual replacement, as the Jacobi
+// forms: when the FP32 residual has dropped by three decades (or claims
+// convergence) e is folded into x in FP64 and r becomes the true FP64
+// residual; the direction is kept.
+//
+// Levels too small to share between CTAs run in CTA 0 alone with CTA
+// barriers while the others wait at the grid barrier (from MgArgs::tail on).
+//
+// Batches: rows of all tanks form one block-diagonal system, so the V-cycle
+// needs no tank bookkeeping; only the dot products, alpha, beta and the
+// stopping tests are per tank.  CTAs own equal contiguous stretches of slices
+// across tank borders; a CTA writes one partial sum per (CTA, tank) segment,
+// to slot CTA + tank, and every CTA adds each tank's segments in the same
+// order, so all CTAs take identical decisions and results are
+// bit-reproducible.
+#include "gfm_grid.cuh"
+
+namespace gfm {
+
+namespace {
+
+constexpr int kMgNR = 2;       // most values one all-reduce sums
+constexpr float kOm1 = 0.56418f;  // Chebyshev degree 2 on [0.35, 2]: 1 / (1.175 +- 0.825 cos(pi/4))
+constexpr float kOm2 = 1.69016f;
+constexpr int kSegLane = 8;    // tanks with more segments are summed by a warp
+
+enum MgAct : int { kMgGo = 0, kMgConverged = 1, kMgNotConverged = 2, kMgBreakdown = 3 };
+enum MgFlag : int { kFlagNone = 0, kFlagUpdate = 1, kFlagRestart = 2, kFlagCap = 3 };
+
+struct MgShared {
+    double2 warp_p[32][kMgNR];   // partial sums of the warps (double, or a double-float pair)
+    double bnorm[kMaxTanks], sc[kMaxTanks], isc[kMaxTanks], gam[kMaxTanks], rho_max[kMaxTanks], rho[kMaxTanks];
+    double best[kMaxTanks], rho_stop[kMaxTanks], xavg[kMaxTanks];
+    double tot[kMgNR][kMaxTanks];
+    float al32[kMaxTanks], be32[kMaxTanks];
+    double al64[kMaxTanks], be64[kMaxTanks];
+    int act[kMaxTanks], flag[kMaxTanks], wait[kMaxTanks], fresh[kMaxTanks];
+    int iters[kMaxTanks], updates[kMaxTanks], stall[kMaxTanks], last_rep[kMaxTanks], restarts[kMaxTanks];
+    int c0[kMaxTanks], c1[kMaxTanks];  // first and last CTA holding slices of the tank
+    int seg_s0[kMaxTanks + 1], seg_tank[kMaxTanks];
+    int wide[kMaxTanks];
+    int nseg, n_wide, any_active, any_flag, fail;
+};
+
+// ---- sums ------------------------------------------------------------------
+// Accumulators: double-float for the FP32 iterations' dot products, double otherwise.
+__device__ __forceinline__ void acc_add(FF &a, float x) { ff_add(a, x); }
+__device__ __forceinline__ void acc_add(double &a, double x) { a += x; }
+__device__ __forceinline__ FF acc_merge(FF a, FF b) { return ff_merge(a, b); }
+__device__ __forceinline__ double acc_merge(double a, double b) { return a + b; }
+__device__ __forceinline__ FF acc_shfl(FF v, int off)
+{
+    return FF{__shfl_xor_sync(0xffffffffu, v.hi, off), __shfl_xor_sync(0xffffffffu, v.lo, off)};
+}
+__device__ __forceinline__ double acc_shfl(double v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
+__device__ __forceinline__ double acc_value(FF v) { return (double)v.hi + (double)v.lo; }
+__device__ __forceinline__ double acc_value(double v) { return v; }
+template <typename A>
+__device__ __forceinline__ A acc_tree(A v)
+{
+#pragma unroll
+    for (int off = 16; off; off >>= 1) v = acc_merge(v, acc_shfl(v, off));
+    return v;
+}
+template <typename T>
+struct AccOf {
+    using type = double;
+};
+template <>
+struct AccOf<float> {
+    using type = FF;
+};
+
+struct Ctx {
+    Grid g;
+    MgShared *sh;
+    int T, lane, warp, nw;
+    int P;  // partial slots per value (grid + tanks)
+};
+
+// Plain grid barrier (an error raised elsewhere is seen at the next wait).
+__device__ __forceinline__ bool mg_sync(Ctx &c)
+{
+    __syncthreads();
+    c.g.epoch += 1u;
+    if (threadIdx.x == 0) c.sh->fail = grid_arrive_wait(c.g) ? 0 : 1;
+    __syncthreads();
+    return c.sh->fail == 0;
+}
+
+// Sum the CTA's per-thread values of one segment and write them to its slot.
+template <int NR, typename A>
+__device__ __forceinline__ void put_partials(Ctx &c, int tank, const A (&v)[NR])
+{
+    MgShared &sh = *c.sh;
+    A r[NR];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) r[k] = acc_tree(v[k]);
+    __syncthreads();
+    if (c.lane == 0) {
+#pragma unroll
+        for (int k = 0; k < NR; ++k) *reinterpret_cast<A *>(&sh.warp_p[c.warp][k]) = r[k];
+    }
+    __syncthreads();
+    if (c.warp == 0) {
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+            A t = c.lane < c.nw ? *reinterpret_cast<const A *>(&sh.warp_p[c.lane][k]) : A{};
+            t = acc_tree(t);
+            if (c.lane == 0)
+                reinterpret_cast<A *>(c.g.partials)[((size_t)c.g.parity * kMgNR + k) * c.P + blockIdx.x + tank] = t;
+        }
+    }
+}
+
+// After every segment's put_partials: grid barrier, then sh.tot[k][t] = the
+// sum of value k over tank t's segments, the same bits in every CTA.
+template <int NR, typename A>
+__device__ __forceinline__ bool mg_allreduce(Ctx &c)
+{
+    MgShared &sh = *c.sh;
+    if (!mg_sync(c)) return false;
+    const A *src = reinterpret_cast<const A *>(c.g.partials) + (size_t)c.g.parity * kMgNR * c.P;
+    auto get = [&](int k, int slot) {
+        if constexpr (sizeof(A) == sizeof(float2)) {
+            const float2 t = __ldcg(reinterpret_cast<const float2 *>(src + (size_t)k * c.P + slot));
+            A a;
+            memcpy(&a, &t, sizeof a);
+            return a;
+        }
+    };
+    if (sh.n_wide < c.T)
+        for (int q = threadIdx.x; q < NR * c.T; q += blockDim.x) {
+            const int k = q / c.T, t = q - k * c.T;
+            const int n = sh.c1[t] - sh.c0[t] + 1;
+            if (n > kSegLane) continue;
+            A v[kSegLane];
+#pragma unroll
+            for (int j = 0; j < kSegLane; ++j) v[j] = j < n ? get(k, sh.c0[t] + j + t) : A{};
+            sh.tot[k][t] = acc_value(acc_merge(acc_merge(acc_merge(v[0], v[1]), acc_merge(v[2], v[3])),
+                                               acc_merge(acc_merge(v[4], v[5]), acc_merge(v[6], v[7]))));
+        }
+    for (int q = c.warp; q < NR * sh.n_wide; q += c.nw) {
+        const int k = q / sh.n_wide, t = sh.wide[q - k * sh.n_wide];
+        A v[6];  // 192 segments with every load in flight
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            const int b = sh.c0[t] + c.lane + 32 * j;
+            v[j] = b <= sh.c1[t] ? get(k, b + t) : A{};
+        }
+        A acc = acc_merge(acc_merge(acc_merge(v[0], v[1]), acc_merge(v[2], v[3])), acc_merge(v[4], v[5]));
+        for (int b = sh.c0[t] + c.lane + 192; b <= sh.c1[t]; b += 32) acc = acc_merge(acc, get(k, b + t));
+        acc = acc_tree(acc);
+        if (c.lane == 0) sh.tot[k][t] = acc_value(acc);
+    }
+    c.g.parity ^= 1;
+    __syncthreads();
+    return true;
+}
+
+// ---- row passes --------------------------------------------------------------
+// acc_i = sum_k val (x_i - x_j) over the rows of slices s0 + w0, + nw, ...
+// below s1 (U of them in flight per warp, chunks of CH faces), then
+// op.post(i, x_i, acc_i, pre) with pre = op.pre(i) loaded before the gathers.
+template <typename T, int CH, int U, bool FINE, typename Op>
+__device__ __forceinline__ void row_pass(const MgLevel &lv, const T *X, int s0, int s1, int w0, int nw, int lane, int n,
+                                         Op &op)
+{
+    const T *__restrict__ val = static_cast<const T *>(lv.val);
+    const int32_t *__restrict__ col = lv.col;
+    for (int sb = s0 + w0; sb < s1; sb += U * nw) {
+        int base[U], w[U];
+        T xi[U], acc[U];
+        typename Op::Pre pr[U];
+        int wmax = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int s = sb + u * nw, i = s * kSlice + lane;
+            base[u] = 0;
+            w[u] = 0;
+            xi[u] = T(0);
+            acc[u] = T(0);
+            if (s < s1 && i < n) {
+                base[u] = __ldg(lv.sp + s);
+                w[u] = (__ldg(lv.sp + s + 1) - base[u]) >> 5;
+                xi[u] = X[i];
+                pr[u] = op.pre(i);
+            }
+            wmax = max(wmax, w[u]);
+        }
+        for (int k0 = 0; k0 < wmax; k0 += CH) {
+            int j[U][CH];
+            T gm[U][CH], xj[U][CH];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int q = 0; q < CH; ++q) {
+                    const bool ok = k0 + q < w[u];
+                    const int slot = base[u] + (k0 + q) * kSlice + lane;
+                    if constexpr (FINE) {  // read once per pass
+                        j[u][q] = ok ? __ldcs(col + slot) : 0;
+                        gm[u][q] = ok ? __ldcs(val + slot) : T(0);
+                    } else {
+                        j[u][q] = ok ? __ldg(col + slot) : 0;
+                        gm[u][q] = ok ? __ldg(val + slot) : T(0);
+                    }
+                }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int q = 0; q < CH; ++q) xj[u][q] = (k0 + q < w[u]) ? X[j[u][q]] : xi[u];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int q = 0; q < CH; ++q) acc[u] = fma(gm[u][q], xi[u] - xj[u][q], acc[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int s = sb + u * nw, i = s * kSlice + lane;
+            if (s < s1 && i < n) op.post(i, xi[u], acc[u], pr[u]);
+        }
+    }
+}
+
+// The pinned cell's extra diagonal: on the mesh one cell of the tank, on a
+// coarse level an array (zero but for the aggregate holding the pinned cell).
+template <typename T, bool FINE>
+struct Pin {
+    const T *a;
+    int ref;
+    T pin;
+    __device__ __forceinline__ T at(int i) const
+    {
+        if constexpr (FINE) return i == ref ? pin : T(0);
+        else return a[i];
+    }
+};
+
+// out = x + w D^{-1} (b - A x)
+template <typename T, bool FINE>
+struct SweepOp {
+    struct Pre {
+        T b, d, p;
+    };
+    const T *b, *dinv;
+    T *out;
+    T w;
+    Pin<T, FINE> pin;
+    __device__ __forceinline__ Pre pre(int i) const { return Pre{b[i], dinv[i], pin.at(i)}; }
+    __device__ __forceinline__ void post(int i, T x, T ax, const Pre &p)
+    {
+        out[i] = fma(w * p.d, p.b - fma(p.p, x, ax), x);
+    }
+};
+
+// out = b - A x
+template <typename T, bool FINE>
+struct ResidOp {
+    struct Pre {
+        T b, p;
+    };
+    const T *b;
+    T *out;
+    Pin<T, FINE> pin;
+    __device__ __forceinline__ Pre pre(int i) const { return Pre{b[i], pin.at(i)}; }
+    __device__ __forceinline__ void post(int i, T x, T ax, const Pre &p) { out[i] = p.b - fma(p.p, x, ax); }
+};
+
+// The last sweep on the mesh: z = x + w D^{-1} (r - A x), and r.z.
+template <typename T>
+struct LastOp {
+    struct Pre {
+        T b, d, p;
+    };
+    const T *b, *dinv;
+    T *out;
+    T w;
+    Pin<T, true> pin;
+    typename AccOf<T>::type acc;
+    __device__ __forceinline__ Pre pre(int i) const { return Pre{b[i], dinv[i], pin.at(i)}; }
+    __device__ __forceinline__ void post(int i, T x, T ax, const Pre &p)
+    {
+        const T z = fma(w * p.d, p.b - fma(p.p, x, ax), x);
+        out[i] = z;
+        acc_add(acc, p.b * z);
+    }
+};
+
+// The last sweep on a coarse level, its result added to the children.
+template <typename T>
+struct LastCoarseOp {
+    struct Pre {
+        T b, d, p;
+    };
+    const T *b, *dinv;
+    const int32_t *cp, *child;
+    T *fine;
+    T w;
+    Pin<T, false> pin;
+    __device__ __forceinline__ Pre pre(int i) const { return Pre{b[i], dinv[i], pin.at(i)}; }
+    __device__ __forceinline__ void post(int i, T x, T ax, const Pre &p)
+    {
+        const T z = fma(w * p.d, p.b - fma(p.p, x, ax), x);
+        const int s = i >> 5, lane = i & 31;
+        const int c0 = __ldg(cp + s), w0 = (__ldg(cp + s + 1) - c0) >> 5;
+        for (int k = 0; k < w0; k += 4) {
+            int ch[4];
+            T v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) ch[q] = k + q < w0 ? __ldg(child + c0 + (k + q) * kSlice + lane) : -1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = ch[q] >= 0 ? fine[ch[q]] : T(0);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (ch[q] >= 0) fine[ch[q]] = v[q] + z;
+        }
+    }
+};
+
+// s = A z + beta s, p = z + beta p (fresh: s = A z, p = z), and p.s.
+template <typename T>
+struct DirOp {
+    struct Pre {
+        T p, s, pin;
+    };
+    T *P, *S;
+    T be;
+    bool fresh;
+    Pin<T, true> pin;
+    typename AccOf<T>::type acc;
+    __device__ __forceinline__ Pre pre(int i) const
+    {
+        return fresh ? Pre{T(0), T(0), pin.at(i)} : Pre{P[i], S[i], pin.at(i)};
+    }
+    __device__ __forceinline__ void post(int i, T x, T ax, const Pre &p)
+    {
+        const T s = fma(be, p.s, fma(p.pin, x, ax));
+        const T d = fma(be, p.p, x);
+        S[i] = s;
+        P[i] = d;
+        acc_add(acc, d * s);
+    }
+};
+
+// b = the sum of the children's residuals, x = w D^{-1} b (the first sweep from zero).
+template <typename T>
+__device__ __forceinline__ void restrict_pass(const MgLevel &lv, const T *res, T w, int s0, int s1, int w0, int nw,
+                                              int lane)
+{
+    const T *dinv = static_cast<const T *>(lv.dinv);
+    T *b = static_cast<T *>(lv.b), *x = static_cast<T *>(lv.xa);
+    for (int s = s0 + w0; s < s1; s += nw) {
+        const int i = s * kSlice + lane;
+        const int c0 = __ldg(lv.cp + s), cw = (__ldg(lv.cp + s + 1) - c0) >> 5;
+        const T d = i < lv.n ? dinv[i] : T(0);
+        T sum = T(0);
+        for (int k = 0; k < cw; k += 4) {
+            int ch[4];
+            T v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) ch[q] = k + q < cw ? __ldg(lv.child + c0 + (k + q) * kSlice + lane) : -1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = ch[q] >= 0 ? res[ch[q]] : T(0);
+            sum += (v[0] + v[1]) + (v[2] + v[3]);
+        }
+        if (i < lv.n) {
+            b[i] = sum;
+            x[i] = w * d * sum;
+        }
+    }
+}
+
+__device__ __forceinline__ void split(int ns, int G, int b, int &s0, int &s1)
+{
+    s0 = (int)(((long long)ns * b) / G);
+    s1 = (int)(((long long)ns * (b + 1)) / G);
+}
+
+// Levels 1 .. L-1 of the V-cycle, from the mesh's residual (lv[0].res) to the
+// correction added to lv[0].xb.  Ends with a grid barrier.
+template <typename T, int CH>
+__device__ __forceinline__ bool coarse_cycle(const MgArgs &a, Ctx &c)
+{
+    const int L = a.L;
+    const T om1 = T(kOm1), om2 = T(kOm2);
+    auto down = [&](int l, int s0, int s1, auto sync) -> bool {
+        const MgLevel &lv = a.lv[l];
+        const Pin<T, false> pin{static_cast<const T *>(lv.pin), -1, T(0)};
+        restrict_pass<T>(lv, static_cast<const T *>(a.lv[l - 1].res), om1, s0, s1, c.warp, c.nw, c.lane);
+        if (!sync()) return false;
+        SweepOp<T, false> sw{static_cast<const T *>(lv.b), static_cast<const T *>(lv.dinv), static_cast<T *>(lv.xb), om2, pin};
+        row_pass<T, CH, 1, false>(lv, static_cast<const T *>(lv.xa), s0, s1, c.warp, c.nw, c.lane, lv.n, sw);
+        if (!sync()) return false;
+        if (l + 1 < L) {
+            ResidOp<T, false> rs{static_cast<const T *>(lv.b), static_cast<T *>(lv.res), pin};
+            row_pass<T, CH, 1, false>(lv, static_cast<const T *>(lv.xb), s0, s1, c.warp, c.nw, c.lane, lv.n, rs);
+            if (!sync()) return false;
+        }
+        return true;
+    };
+    auto up = [&](int l, int s0, int s1, auto sync) -> bool {
+        const MgLevel &lv = a.lv[l];
+        const Pin<T, false> pin{static_cast<const T *>(lv.pin), -1, T(0)};
+        SweepOp<T, false> sw{static_cast<const T *>(lv.b), static_cast<const T *>(lv.dinv), static_cast<T *>(lv.xa), om2, pin};
+        row_pass<T, CH, 1, false>(lv, static_cast<const T *>(lv.xb), s0, s1, c.warp, c.nw, c.lane, lv.n, sw);
+        if (!sync()) return false;
+        LastCoarseOp<T> lc{static_cast<const T *>(lv.b), static_cast<const T *>(lv.dinv), lv.cp, lv.child,
+                           static_cast<T *>(a.lv[l - 1].xb), om1, pin};
+        row_pass<T, CH, 1, false>(lv, static_cast<const T *>(lv.xa), s0, s1, c.warp, c.nw, c.lane, lv.n, lc);
+        return sync();
+    };
+    auto gsync = [&]() { return mg_sync(c); };
+    auto bsync = [&]() {
+        __syncthreads();
+        return true;
+    };
+    int s0, s1;
+    const int tail = a.tail < L ? a.tail : L;
+    for (int l = 1; l < tail; ++l) {
+        split(a.lv[l].n_slices, c.g.G, blockIdx.x, s0, s1);
+        if (!down(l, s0, s1, gsync)) return false;
+    }
+    if (tail < L) {
+        if (blockIdx.x == 0) {
+            for (int l = tail; l < L; ++l) down(l, 0, a.lv[l].n_slices, bsync);
+            for (int l = L - 1; l >= tail; --l) up(l, 0, a.lv[l].n_slices, bsync);
+        }
+        if (!mg_sync(c)) return false;
+    }
+    for (int l = tail - 1; l >= 1; --l) {
+        split(a.lv[l].n_slices, c.g.G, blockIdx.x, s0, s1);
+        if (!up(l, s0, s1, gsync)) return false;
+    }
+    return true;
+}
+
+// (A x)_i in FP64, difference form with the pin.
+template <int CH>
+__device__ __forceinline__ double row64(const SolveArgs &a, int s, int lane, double xi, double pin_i)
+{
+    const int base = __ldg(a.m.slice_ptr + s), w = (__ldg(a.m.slice_ptr + s + 1) - base) >> 5;
+    double acc = pin_i * xi;
+    for (int k0 = 0; k0 < w; k0 += CH) {
+        int j[CH];
+        double gm[CH], xj[CH];
+#pragma unroll
+        for (int q = 0; q < CH; ++q) {
+            const bool ok = k0 + q < w;
+            const int slot = base + (k0 + q) * kSlice + lane;
+            j[q] = ok ? __ldcs(a.m.col + slot) : 0;
+            gm[q] = ok ? __ldcs(a.m.val64 + slot) : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < CH; ++q) xj[q] = (k0 + q < w) ? a.x64[j[q]] : xi;
+#pragma unroll
+        for (int q = 0; q < CH; ++q) acc = fma(gm[q], xi - xj[q], acc);
+    }
+    return acc;
+}
+
+__device__ void mg_abort(const MgArgs &a)
+{
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const int e = ld_volatile_i32(a.s.err);
+        for (int t = 0; t < a.T; ++t) {
+            a.s.info[t].status = e;
+            a.s.info[t].rel_res_l2 = -1.0;
+            a.s.info[t].rel_res_l1 = -1.0;
+        }
+    }
+}
+
+}  // namespace
+
+template <typename T, int CH, int NT>
+__global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
+{
+    constexpr bool kMixed = sizeof(T) == 4;
+    constexpr int U = kMixed ? 2 : 1;  // slices in flight per warp in the row passes
+    constexpr int UB = kMixed ? 4 : 2;  // the same in the update pass
+    using A = typename AccOf<T>::type;
+    __shared__ MgShared sh;
+    Ctx c;
+    c.g = Grid{a.s.bar, a.s.err, a.s.partials, a.s.budget_ns, 0u, (int)gridDim.x, 0};
+    c.sh = &sh;
+    c.T = a.T;
+    c.lane = threadIdx.x & 31;
+    c.warp = threadIdx.x >> 5;
+    c.nw = blockDim.x >> 5;
+    c.P = (int)gridDim.x + a.T;
+    const int T_ = a.T, lane = c.lane, warp = c.warp, nw = c.nw;
+    const T om1 = T(kOm1), om2 = T(kOm2);
+    int s_lo, s_hi;
+    split(a.s.m.n_slices, c.g.G, blockIdx.x, s_lo, s_hi);
+    // this CTA's segments and every tank's CTAs
+    for (int t = threadIdx.x; t < T_; t += blockDim.x) {
+        const long long G = c.g.G, ns = a.s.m.n_slices;
+        const int f = T_ > 1 ? a.tank_off[t] >> 5 : 0, e = T_ > 1 ? a.tank_off[t + 1] >> 5 : (int)ns;
+        sh.c0[t] = (int)(((f + 1) * G - 1) / ns);
+        sh.c1[t] = (int)((e * G - 1) / ns);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int m = 0, nwd = 0;
+        for (int t = 0; t < T_; ++t) {
+            const int f = T_ > 1 ? a.tank_off[t] >> 5 : 0, e = T_ > 1 ? a.tank_off[t + 1] >> 5 : a.s.m.n_slices;
+            if (f < s_hi && e > s_lo) {
+                sh.seg_s0[m] = max(f, s_lo);
+                sh.seg_tank[m++] = t;
+            }
+            if (sh.c1[t] - sh.c0[t] + 1 > kSegLane) sh.wide[nwd++] = t;
+        }
+        sh.seg_s0[m] = s_hi;
+        sh.nseg = m;
+        sh.n_wide = nwd;
+    }
+    __syncthreads();
+    const int nseg = sh.nseg;
+    auto bail = [&]() { mg_abort(a); };
+
+    const MgLevel &l0 = a.lv[0];
+    T *R = static_cast<T *>(l0.b), *XA = static_cast<T *>(l0.xa), *XB = static_cast<T *>(l0.xb);
+    T *RES = static_cast<T *>(l0.res), *Z = static_cast<T *>(a.z), *P = static_cast<T *>(a.p), *S = static_cast<T *>(a.sv);
+    T *E = static_cast<T *>(a.e);  // FP32 correction (mixed); unused in FP64
+    const T *dinv = static_cast<const T *>(l0.dinv);
+    // pinned cell and end of the real cells of a tank
+    auto tank_end = [&](int t) { return T_ > 1 ? a.tank_off[t] + a.s.n_per_tank[t] : a.s.m.n; };
+    auto tank_pin = [&](int t) {
+        const DevParams *p = T_ > 1 ? a.tprm + t : a.s.prm;
+        return Pin<T, true>{nullptr, p->ref, T(p->pin64)};
+    };
+
+    // prologue: x0, ||b||
+    for (int q = 0; q < nseg; ++q) {
+        const int t = sh.seg_tank[q], end = tank_end(t);
+        double vb[1] = {0.0};
+        for (int s = sh.seg_s0[q] + warp; s < sh.seg_s0[q + 1]; s += nw) {
+            const int i = s * kSlice + lane;
+            if (i < end) {
+                a.s.x64[i] = a.s.use_x0 ? a.s.p_user[a.s.iperm[i]] : 0.0;
+                if constexpr (kMixed) E[i] = T(0);
+                const double bi = a.s.b[i];
+                vb[0] = fma(bi, bi, vb[0]);
+            }
+        }
+        put_partials<1, double>(c, t, vb);
+    }
+    if (!mg_allreduce<1, double>(c)) { bail(); return; }
+    for (int t = threadIdx.x; t < T_; t += blockDim.x) {
+        const double bb = sh.tot[0][t], bn = bb > 0.0 ? sqrt(bb) : 1.0;
+        sh.bnorm[t] = bn;
+        int ex = 0;
+        // FP32: one power-of-two scale for the whole solve, so residual
+        // entries start near 1 and shrink by at most the tolerance
+        if constexpr (kMixed) frexp(bn / sqrt((double)(a.s.n_per_tank ? a.s.n_per_tank[t] : a.s.m.n)), &ex);
+        sh.sc[t] = ldexp(1.0, -ex);
+        sh.isc[t] = ldexp(1.0, ex);
+        sh.rho_stop[t] = (a.s.rtol * bn * sh.sc[t]) * (a.s.rtol * bn * sh.sc[t]);
+        sh.gam[t] = 1.0;
+        sh.rho[t] = 0.0;
+        sh.act[t] = kMgGo;
+        sh.flag[t] = kFlagRestart;  // the first residual, no direction yet
+        sh.wait[t] = 0;
+        sh.fresh[t] = 1;
+        sh.iters[t] = sh.updates[t] = sh.stall[t] = sh.last_rep[t] = sh.restarts[t] = 0;
+        sh.best[t] = 1e300;
+    }
+    __syncthreads();
+    const int cap_updates = a.s.max_refine + 1 + (kMixed ? (int)(2.0 * log10(1.0 / a.s.rtol)) : 0);
+
+    // r = b - A x (FP64) for the flagged tanks, x += e first (mixed); also
+    // the V-cycle's first sweep from zero.  Then the tanks' decisions.
+    auto replace = [&](bool first) -> bool {
+        if (kMixed && !first) {
+            for (int q = 0; q < nseg; ++q) {
+                const int t = sh.seg_tank[q], end = tank_end(t);
+                if (sh.flag[t] == kFlagNone) continue;
+                const double isc = sh.isc[t];
+                for (int sb = sh.seg_s0[q] + warp; sb < sh.seg_s0[q + 1]; sb += 4 * nw) {
+                    T e[4];
+                    double x[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int i = (sb + u * nw) * kSlice + lane;
+                        const bool ok = sb + u * nw < sh.seg_s0[q + 1] && i < end;
+                        e[u] = ok ? E[i] : T(0);
+                        x[u] = ok ? a.s.x64[i] : 0.0;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int i = (sb + u * nw) * kSlice + lane;
+                        if (sb + u * nw < sh.seg_s0[q + 1] && i < end) {
+                            a.s.x64[i] = fma((double)e[u], isc, x[u]);
+                            E[i] = T(0);
+                        }
+                    }
+                }
+            }
+            if (!mg_sync(c)) return false;
+        }
+        for (int q = 0; q < nseg; ++q) {
+            const int t = sh.seg_tank[q], end = tank_end(t);
+            A v[1] = {A{}};
+            if (sh.flag[t] != kFlagNone) {
+                const double sc = sh.sc[t];
+                const DevParams *pp = T_ > 1 ? a.tprm + t : a.s.prm;
+                const int ref = pp->ref;
+                const double pin = pp->pin64;
+                const bool with_x = !first || a.s.use_x0;
+                for (int s = sh.seg_s0[q] + warp; s < sh.seg_s0[q + 1]; s += nw) {
+                    const int i = s * kSlice + lane;
+                    if (i < end) {
+                        const double bi = a.s.b[i];
+                        const T d = dinv[i];
+                        const double r = with_x ? bi - row64<CH>(a.s, s, lane, a.s.x64[i], i == ref ? pin : 0.0) : bi;
+                        const T rt = (T)(r * sc);
+                        R[i] = rt;
+                        XA[i] = om1 * d * rt;
+                        acc_add(v[0], rt * rt);
+                    }
+                }
+            }
+            put_partials<1, A>(c, t, v);
+        }
+        if (!mg_allreduce<1, A>(c)) return false;
+        if (threadIdx.x < 32) {
+            bool active = false;
+            for (int t = threadIdx.x; t < T_; t += 32) {
+                const int f = sh.flag[t];
+                if (sh.act[t] == kMgGo && f != kFlagNone) {
+                    sh.flag[t] = kFlagNone;
+                    sh.wait[t] = 0;
+                    sh.last_rep[t] = sh.iters[t];
+                    ++sh.updates[t];
+                    const double rr = sh.tot[0][t];
+                    const double rel2 = rr / (sh.bnorm[t] * sh.sc[t] * (sh.bnorm[t] * sh.sc[t]));
+                    // FP32 residual entries carry 6e-8 each: stay below the target by as much
+                    const double tol2 = a.s.rtol * a.s.rtol * (kMixed ? 1.0 - 1e-6 : 1.0);
+                    sh.fresh[t] |= (f == kFlagRestart) ? 1 : 0;
+                    // the recurrence had drifted from the true residual: its
+                    // direction is no longer conjugate to anything
+                    if (!(rr <= 4.0 * sh.rho[t])) sh.fresh[t] = 1;
+                    sh.rho_max[t] = rr;
+                    if (rel2 <= tol2) sh.act[t] = kMgConverged;
+                    else if (f == kFlagCap) sh.act[t] = kMgNotConverged;
+                    else if (!isfinite(rr)) sh.act[t] = kMgBreakdown;
+                    else if (!first) {
+                        if (f == kFlagRestart && ++sh.restarts[t] > 3) sh.act[t] = kMgBreakdown;
+                        if (rel2 < 0.25 * sh.best[t]) {
+                            sh.best[t] = rel2;
+                            sh.stall[t] = 0;
+                        } else {
+                            ++sh.stall[t];
+                        }
+                        if (sh.act[t] == kMgGo && (sh.stall[t] > (kMixed ? 8 : 2) || sh.updates[t] > cap_updates))
+                            sh.act[t] = kMgNotConverged;
+                    } else {
+                        sh.best[t] = rel2;
+                        if (a.s.max_iters <= 0) sh.act[t] = kMgNotConverged;
+                    }
+                }
+                active |= sh.act[t] == kMgGo;
+            }
+            active = __any_sync(0xffffffffu, active);
+            if (threadIdx.x == 0) sh.any_active = active;
+        }
+        __syncthreads();
+        return true;
+    };
+    if (!replace(true)) { bail(); return; }
+
+    auto working = [&](int t) { return sh.act[t] == kMgGo && sh.wait[t] == 0; };
+    auto fine_sweep = [&](const T *X, T *out, T w) {
+        for (int q = 0; q < nseg; ++q) {
+            const int t = sh.seg_tank[q];
+            if (!working(t)) continue;
+            SweepOp<T, true> op{R, dinv, out, w, tank_pin(t)};
+            row_pass<T, CH, U, true>(l0, X, sh.seg_s0[q], sh.seg_s0[q + 1], warp, nw, lane, tank_end(t), op);
+        }
+    };
+    while (sh.any_active) {
+        // z = V-cycle(r): XA holds the first sweep
+        fine_sweep(XA, XB, om2);
+        if (!mg_sync(c)) { bail(); return; }
+        if (a.L > 1) {
+            for (int q = 0; q < nseg; ++q) {
+                const int t = sh.seg_tank[q];
+                if (!working(t)) continue;
+                ResidOp<T, true> op{R, RES, tank_pin(t)};
+                row_pass<T, CH, U, true>(l0, XB, sh.seg_s0[q], sh.seg_s0[q + 1], warp, nw, lane, tank_end(t), op);
+            }
+            if (!mg_sync(c)) { bail(); return; }
+            if (!coarse_cycle<T, CH>(a, c)) { bail(); return; }
+        }
+        fine_sweep(XB, XA, om2);
+        if (!mg_sync(c)) { bail(); return; }
+        for (int q = 0; q < nseg; ++q) {
+            const int t = sh.seg_tank[q];
+            A v[1] = {A{}};
+            if (working(t)) {
+                LastOp<T> op{R, dinv, Z, om1, tank_pin(t), A{}};
+                row_pass<T, CH, U, true>(l0, XA, sh.seg_s0[q], sh.seg_s0[q + 1], warp, nw, lane, tank_end(t), op);
+                v[0] = op.acc;
+            }
+            put_partials<1, A>(c, t, v);
+        }
+        if (!mg_allreduce<1, A>(c)) { bail(); return; }
+        for (int t = threadIdx.x; t < T_; t += blockDim.x) {
+            if (!working(t)) continue;
+            const double gn = sh.tot[0][t];
+            const bool ok = gn > 0.0 && isfinite(gn);
+            if (!ok) sh.flag[t] = kFlagRestart;
+            const bool fresh = sh.fresh[t] || !ok;
+            if constexpr (kMixed) sh.be32[t] = fresh ? 0.0f : (float)gn / (float)sh.gam[t];
+            else sh.be64[t] = fresh ? 0.0 : gn / sh.gam[t];
+            sh.fresh[t] = fresh;
+            sh.gam[t] = gn;
+        }
+        __syncthreads();
+        // p = z + beta p, s = A p, p.s
+        for (int q = 0; q < nseg; ++q) {
+            const int t = sh.seg_tank[q];
+            A v[1] = {A{}};
+            if (working(t) && sh.flag[t] == kFlagNone) {
+                T be;
+                if constexpr (kMixed) be = sh.be32[t];
+                else be = sh.be64[t];
+                DirOp<T> op{P, S, be, sh.fresh[t] != 0, tank_pin(t), A{}};
+                row_pass<T, CH, U, true>(l0, Z, sh.seg_s0[q], sh.seg_s0[q + 1], warp, nw, lane, tank_end(t), op);
+                v[0] = op.acc;
+            }
+            put_partials<1, A>(c, t, v);
+        }
+        if (!mg_allreduce<1, A>(c)) { bail(); return; }
+        for (int t = threadIdx.x; t < T_; t += blockDim.x) {
+            if (!working(t) || sh.flag[t] != kFlagNone) continue;
+            const double ps = sh.tot[0][t];
+            const bool ok = ps > 0.0 && isfinite(ps);
+            if constexpr (kMixed) sh.al32[t] = ok ? (float)sh.gam[t] / (float)ps : 0.0f;
+            else sh.al64[t] = ok ? sh.gam[t] / ps : 0.0;
+            if (!ok) sh.flag[t] = kFlagRestart;
+            sh.fresh[t] = 0;
+        }
+        __syncthreads();
+        // e += alpha p (FP64: x), r -= alpha s, the next V-cycle's first sweep, r.r
+        for (int q = 0; q < nseg; ++q) {
+            const int t = sh.seg_tank[q], end = tank_end(t), e1 = sh.seg_s0[q + 1];
+            A v[1] = {A{}};
+            if (working(t) && sh.flag[t] == kFlagNone) {
+                T al;
+                if constexpr (kMixed) al = sh.al32[t];
+                else al = sh.al64[t];
+                T *X;
+                if constexpr (kMixed) X = E;
+                else X = a.s.x64;
+                for (int sb = sh.seg_s0[q] + warp; sb < e1; sb += UB * nw) {
+                    T p[UB], s[UB], r[UB], x[UB], d[UB];
+#pragma unroll
+                    for (int u = 0; u < UB; ++u) {
+                        const int i = (sb + u * nw) * kSlice + lane;
+                        const bool ok = sb + u * nw < e1 && i < end;
+                        p[u] = ok ? P[i] : T(0);
+                        s[u] = ok ? S[i] : T(0);
+                        r[u] = ok ? R[i] : T(0);
+                        x[u] = ok ? X[i] : T(0);
+                        d[u] = ok ? dinv[i] : T(0);
+                    }
+#pragma unroll
+                    for (int u = 0; u < UB; ++u) {
+                        const int i = (sb + u * nw) * kSlice + lane;
+                        if (sb + u * nw < e1 && i < end) {
+                            X[i] = fma(al, p[u], x[u]);
+                            const T rn = fma(-al, s[u], r[u]);
+                            R[i] = rn;
+                            XA[i] = om1 * d[u] * rn;
+                            acc_add(v[0], rn * rn);
+                        }
+                    }
+                }
+            }
+            put_partials<1, A>(c, t, v);
+        }
+        if (!mg_allreduce<1, A>(c)) { bail(); return; }
+        // A tank asks for a residual replacement when its residual claims
+        // convergence, can no longer be trusted in FP32 (three decades below
+        // the last true one) or cannot go on.  In a batch a tank that claims
+        // convergence idles until the round, which comes when no tank is left
+        // iterating or some tank must not wait.
+        if (threadIdx.x < 32) {
+            bool now = false, asked = false, going = false;
+            for (int t = threadIdx.x; t < T_; t += 32) {
+                if (sh.act[t] != kMgGo) continue;
+                if (sh.wait[t]) {
+                    asked = true;
+                    continue;
+                }
+                if (sh.flag[t] == kFlagRestart) {
+                    now = true;
+                    continue;
+                }
+                const int it = ++sh.iters[t];
+                const double rho = sh.tot[0][t];
+                sh.rho[t] = rho;
+                if (it >= a.s.max_iters) {
+                    sh.flag[t] = kFlagCap;
+                    now = true;
+                } else if (!(rho > 0.81 * sh.rho_stop[t])) {
+                    sh.flag[t] = kFlagUpdate;
+                    sh.wait[t] = 1;
+                    asked = true;
+                } else if (kMixed && (rho <= 1e-6 * sh.rho_max[t] || it - sh.last_rep[t] >= 40)) {
+                    sh.flag[t] = kFlagUpdate;
+                    sh.wait[t] = 1;
+                    asked = true;
+                } else {
+                    going = true;
+                }
+            }
+            now = __any_sync(0xffffffffu, now);
+            asked = __any_sync(0xffffffffu, asked);
+            going = __any_sync(0xffffffffu, going);
+            if (threadIdx.x == 0) sh.any_flag = now || (asked && !going);
+        }
+        __syncthreads();
+        if (sh.any_flag && !replace(false)) { bail(); return; }
+    }
+
+    // the record: true FP64 residual (r in r64), solution in caller order,
+    // normalised L1 residual sum|r| / (sum|A x - x_avg rowsum| + sum|b - x_avg rowsum|)
+    if (!mg_sync(c)) { bail(); return; }
+    for (int q = 0; q < nseg; ++q) {
+        const int t = sh.seg_tank[q], end = tank_end(t);
+        const DevParams *pp = T_ > 1 ? a.tprm + t : a.s.prm;
+        const int ref = pp->ref;
+        const double pin = pp->pin64;
+        double v[2] = {0.0, 0.0};
+        for (int s = sh.seg_s0[q] + warp; s < sh.seg_s0[q + 1]; s += nw) {
+            const int i = s * kSlice + lane;
+            if (i < end) {
+                const double xi = a.s.x64[i];
+                const double r = a.s.b[i] - row64<CH>(a.s, s, lane, xi, i == ref ? pin : 0.0);
+                a.s.r64[i] = r;
+                a.s.p_user[a.s.iperm[i]] = xi;
+                v[0] = fma(r, r, v[0]);
+                v[1] += xi;
+            }
+        }
+        put_partials<2, double>(c, t, v);
+    }
+    if (!mg_allreduce<2, double>(c)) { bail(); return; }
+    for (int t = threadIdx.x; t < T_; t += blockDim.x) {
+        sh.xavg[t] = sh.tot[1][t] / (double)(a.s.n_per_tank ? a.s.n_per_tank[t] : a.s.m.n);
+        sh.rho[t] = sh.tot[0][t];
+    }
+    __syncthreads();
+    for (int q = 0; q < nseg; ++q) {
+        const int t = sh.seg_tank[q], end = tank_end(t);
+        const DevParams *pp = T_ > 1 ? a.tprm + t : a.s.prm;
+        const int ref = pp->ref;
+        const double pin = pp->pin64, xavg = sh.xavg[t];
+        double v[2] = {0.0, 0.0};
+        for (int s = sh.seg_s0[q] + warp; s < sh.seg_s0[q + 1]; s += nw) {
+            const int i = s * kSlice + lane;
+            if (i < end) {
+                const double r = a.s.r64[i], bi = a.s.b[i], rs = i == ref ? pin : 0.0;
+                v[0] += fabs(r);
+                v[1] += fabs(bi - r - xavg * rs) + fabs(bi - xavg * rs);
+            }
+        }
+        put_partials<2, double>(c, t, v);
+    }
+    if (!mg_allreduce<2, double>(c)) { bail(); return; }
+    if (blockIdx.x == 0)
+        for (int t = threadIdx.x; t < T_; t += blockDim.x) {
+            const int e = ld_volatile_i32(a.s.err);
+            int st = GFM_OK;
+            if (sh.act[t] == kMgNotConverged) st = GFM_ERR_NOT_CONVERGED;
+            else if (sh.act[t] == kMgBreakdown) st = GFM_ERR_BREAKDOWN;
+            if (e != 0) st = e;
+            a.s.info[t].iters = sh.iters[t];
+            a.s.info[t].refinements = sh.updates[t];
+            a.s.info[t].status = st;
+            a.s.info[t].reserved = 0;
+            a.s.info[t].rel_res_l2 = sqrt(sh.rho[t]) / sh.bnorm[t];
+            a.s.info[t].rel_res_l1 = sh.tot[0][t] / (sh.tot[1][t] + 1e-300);
+        }
+}
+
+// ---- assembly of the coarse levels -------------------------------------------
+// One thread per coarse node: its faces' coefficients (scale x the sum of the
+// finer faces' in ascending order, the same bits from both sides), diagonal
+// and pin, in FP64 with FP32 copies.
+__global__ void __launch_bounds__(256) k_mg_level(MgLevelArgs a)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int s = i >> 5, lane = i & 31;
+    if (s >= a.n_slices) return;
+    const int base = a.sp[s], w = (a.sp[s + 1] - base) >> 5;
+    double diag = 0.0;
+    for (int k = 0; k < w; ++k) {
+        const int slot = base + k * kSlice + lane;
+        const int f = a.face[slot] - 1;
+        double g = 0.0;
+        if (f >= 0) {
+            for (int m = a.mem_ptr[f]; m < a.mem_ptr[f + 1]; ++m) g += a.fine_gamma[a.mem[m]];
+            g *= a.scale[f];
+            if (a.col[slot] > i) a.gamma[f] = g;
+        }
+        a.val64[slot] = g;
+        a.val32[slot] = (float)g;
+        diag += g;
+    }
+    // the pin: the sum over the children's
+    double pin = 0.0;
+    const int c0 = a.cp[s], cw = (a.cp[s + 1] - c0) >> 5;
+    for (int k = 0; k < cw; ++k) {
+        const int ch = a.child[c0 + k * kSlice + lane];
+        if (ch < 0) continue;
+        if (a.fine_pin) pin += a.fine_pin[ch];
+        else {
+            const DevParams *p = a.stank ? a.tprm + a.stank[ch >> 5] : a.prm;
+            if (ch == p->ref) pin += p->pin64;
+        }
+    }
+    diag += pin;
+    const double d = diag > 0.0 ? 1.0 / diag : 0.0;
+    a.pin64[i] = pin;
+    a.pin32[i] = (float)pin;
+    a.dinv64[i] = d;
+    a.dinv32[i] = (float)d;
+}
+
+cudaError_t launch_mg_level(const MgLevelArgs &a, cudaStream_t s)
+{
+    k_mg_level<<<(a.n_slices * kSlice + 255) / 256, 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+// Instantiations by faces per row chunk and by precision; *threads in: the
+// wanted threads per CTA, out: at most what the instantiation allows.
+const void *mg_kernel(bool mixed, int max_width, int *max_threads)
+{
+    *max_threads = mixed ? 1024 : 512;
+    if (mixed) return max_width <= 4 ? (const void *)k_solve_mg<float, 4, 1024> : (const void *)k_solve_mg<float, 6, 1024>;
+    return max_width <= 4 ? (const void *)k_solve_mg<double, 4, 512> : (const void *)k_solve_mg<double, 6, 512>;
+}
+
+}  // namespace gfm
