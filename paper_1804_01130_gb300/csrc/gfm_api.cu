@@ -6,6 +6,7 @@
 #include <cstring>
 #include <exception>
 #include <future>
+#include <iterator>
 #include <new>
 #include <string>
 #include <system_error>
@@ -18,10 +19,10 @@
 
 // One coarse multigrid level on the device.
 struct MgDev {
-    int n = 0, n_slices = 0;
+    int n = 0, n_slices = 0, max_width = 0, max_child = 0;
     int32_t *sp = nullptr, *col = nullptr, *face = nullptr, *cp = nullptr, *child = nullptr;
     int32_t *mem_ptr = nullptr, *mem = nullptr;
-    double *scale = nullptr, *gamma = nullptr, *val64 = nullptr, *pin64 = nullptr, *dinv64 = nullptr;
+    double *scale = nullptr, *gamma = nullptr, *val64 = nullptr, *pin64 = nullptr, *diag64 = nullptr, *dinv64 = nullptr;
     float *val32 = nullptr, *pin32 = nullptr, *dinv32 = nullptr;
     double *b = nullptr, *xa = nullptr, *xb = nullptr, *res = nullptr;  // vectors (FP64 or FP32)
 };
@@ -159,7 +160,7 @@ void free_all(gfm_ctx *h)
         if (p) cudaFree(p);
     for (MgDev &l : h->mg) {
         void *lp[] = {l.sp, l.col, l.face, l.cp, l.child, l.mem_ptr, l.mem, l.scale, l.gamma, l.val64, l.pin64,
-                      l.dinv64, l.val32, l.pin32, l.dinv32, l.b, l.xa, l.xb, l.res};
+                      l.diag64, l.dinv64, l.val32, l.pin32, l.dinv32, l.b, l.xa, l.xb, l.res};
         for (void *p : lp)
             if (p) cudaFree(p);
     }
@@ -335,28 +336,76 @@ void clear_stale_error() { (void)cudaGetLastError(); }
 // FP64): its passes are bound by gather latency.  Other tunings are taken as
 // they are.  A small mesh gets a CTA per 8 slices, since every CTA more makes
 // the grid barriers dearer.
-gfm_status plan_mg(gfm_ctx *h, gfm::Mode mode, const void **kernel, int *grid, int *threads)
+struct MgPlan {
+    const void *kernel = nullptr;
+    int grid = 0, threads = 0, tail = 0;
+    size_t dyn = 0;
+    gfm::MgTail tl[gfm::kMgTailMax] = {};
+};
+
+gfm_status plan_mg(gfm_ctx *h, gfm::Mode mode, MgPlan *mp)
 {
+    const bool mixed = mode == gfm::Mode::MIXED;
     int most = 0;
-    *kernel = gfm::mg_kernel(mode == gfm::Mode::MIXED, h->ht.max_width, &most);
+    mp->kernel = gfm::mg_kernel(mixed, h->ht.max_width, &most);
     const bool standard = h->tuning.threads == 512 && h->tuning.ctas_per_sm == 1;
-    int t = standard ? most : std::min(h->tuning.threads, most), per = h->tuning.ctas_per_sm;
-    int occ = 0;
-    GFM_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, *kernel, t, 0));
+    const int t = standard ? most : std::min(h->tuning.threads, most);
+    int per = h->tuning.ctas_per_sm, occ = 0;
+    GFM_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, mp->kernel, t, 0));
     if (occ < 1) return fail(h, GFM_ERR_ARG, "multigrid kernel cannot run with this many threads per CTA");
     per = std::min(per, occ);
-    *grid = std::max(1, std::min(h->sm_count * per, (h->ht.n_slices + 7) / 8));
-    *threads = t;
+    // The tail: the levels that CTA 0 holds in its shared memory, as many of
+    // the last ones as fit beside the other CTAs of the SM, up to 2048 nodes
+    // (two rows a thread) in FP32 and 512 in FP64, whose pipe takes a row's
+    // FP64 instructions at 1/64 of the FP32 rate.
+    cudaFuncAttributes fa;
+    GFM_CUDA(h, cudaFuncGetAttributes(&fa, mp->kernel));
+    const long long budget = std::min((long long)h->smem_per_sm / per - 1024, (long long)h->smem_optin) -
+                             (long long)fa.sharedSizeBytes;
+    const int most_nodes = mixed ? 2048 : 512, ts = mixed ? 4 : 8;
+    const int L = (int)h->mg.size() + 1;
+    // bytes of a level; the first tail level's children are 32-bit cell or node numbers
+    auto bytes = [&](const MgDev &d, bool first) {
+        const long long np = (long long)d.n_slices * 32;
+        return np * (ts * (d.max_width + 3) + 2 * d.max_width + (first ? 4 : 2) * d.max_child) + 2 * ts * (np + 2) + 16;
+    };
+    long long used = 0;
+    mp->tail = L;
+    while (mp->tail > 1 && L - mp->tail < gfm::kMgTailMax) {
+        const MgDev &d = h->mg[(size_t)mp->tail - 2];
+        const int rows = std::min(most_nodes, d.max_width <= 6 ? 2 * t : t);
+        if (d.n > rows || d.max_width > gfm::kMgTailWidth || used + bytes(d, true) > budget) break;
+        used += bytes(d, false);
+        --mp->tail;
+    }
+    int off = 0;
+    for (int l = mp->tail; l < L; ++l) {
+        const MgDev &d = h->mg[(size_t)l - 1];
+        gfm::MgTail &q = mp->tl[l - mp->tail];
+        q.n = d.n;
+        q.np = d.n_slices * 32;
+        q.w = d.max_width;
+        q.cw = d.max_child;
+        int32_t *v[] = {&q.dinv, &q.pin, &q.b, &q.xa, &q.xb};
+        for (int32_t *p : v) {
+            *p = off;
+            off += ts * (q.np + ((p == &q.xa || p == &q.xb) ? 2 : 0));  // an element for missing children
+        }
+        q.val = off;
+        off += ts * q.np * q.w;
+        q.child = off;
+        off += (l == mp->tail ? 4 : 2) * q.np * q.cw;
+        q.col = off;
+        off += 2 * q.np * q.w;
+        off = (off + 15) & ~15;
+    }
+    mp->dyn = (size_t)off;
+    GFM_CUDA(h, cudaFuncSetAttribute(mp->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, off));
+    GFM_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, mp->kernel, t, mp->dyn));
+    if (occ < per) return fail(h, GFM_ERR_ARG, "launch shape cannot be co-resident with its shared memory");
+    mp->grid = std::max(1, std::min(h->sm_count * per, (h->ht.n_slices + 7) / 8));
+    mp->threads = t;
     return GFM_OK;
-}
-
-// Slices below which a level runs in CTA 0 alone.
-int mg_tail(const gfm_ctx *h, gfm::Mode mode)
-{
-    const int most = mode == gfm::Mode::MIXED ? 64 : 16;
-    int l = 0;
-    while (l < (int)h->mg.size() && h->mg[(size_t)l].n_slices > most) ++l;
-    return l + 1;
 }
 
 // Enqueue one persistent solve of A x = rhs (internal order) writing the
@@ -366,11 +415,13 @@ gfm_status enqueue_solve(gfm_ctx *h, const gfm_solve_opts *o, const double *rhs,
 {
     const gfm::Mode mode = (o->mode == GFM_MIXED) ? gfm::Mode::MIXED : gfm::Mode::FP64;
     LaunchPlan lp;
-    const void *mgk = nullptr;
+    MgPlan mp;
     int grid = 0, threads = 0;
     if (h->mg_valid) {
-        gfm_status st = plan_mg(h, mode, &mgk, &grid, &threads);
+        gfm_status st = plan_mg(h, mode, &mp);
         if (st != GFM_OK) return st;
+        grid = mp.grid;
+        threads = mp.threads;
     } else {
         gfm_status st = plan_launch(h, mode, &lp);
         if (st != GFM_OK) return st;
@@ -437,7 +488,8 @@ gfm_status enqueue_solve(gfm_ctx *h, const gfm_solve_opts *o, const double *rhs,
     if (h->mg_valid) {
         m.s = a;
         m.L = (int)h->mg.size() + 1;
-        m.tail = mg_tail(h, mode);
+        m.tail = mp.tail;
+        std::copy(std::begin(mp.tl), std::end(mp.tl), std::begin(m.tl));
         m.T = h->batched ? h->T : 1;
         m.tank_off = h->tioff;
         m.tprm = h->tprm;
@@ -453,6 +505,7 @@ gfm_status enqueue_solve(gfm_ctx *h, const gfm_solve_opts *o, const double *rhs,
         l0.sp = h->slice_ptr;
         l0.col = h->col;
         l0.val = mixed ? (const void *)h->val32 : (const void *)h->val64;
+        l0.pin = mixed ? nullptr : (const void *)h->diag;
         l0.dinv = mixed ? (const void *)h->dinv32 : (const void *)h->dinv;
         l0.b = mixed ? (void *)h->R32 : (void *)h->r64;
         l0.xa = v0;
@@ -471,7 +524,7 @@ gfm_status enqueue_solve(gfm_ctx *h, const gfm_solve_opts *o, const double *rhs,
             lv.col = d.col;
             lv.val = mixed ? (const void *)d.val32 : (const void *)d.val64;
             lv.dinv = mixed ? (const void *)d.dinv32 : (const void *)d.dinv64;
-            lv.pin = mixed ? (const void *)d.pin32 : (const void *)d.pin64;
+            lv.pin = mixed ? (const void *)d.pin32 : (const void *)d.diag64;
             lv.cp = d.cp;
             lv.child = d.child;
             lv.b = d.b;
@@ -479,11 +532,12 @@ gfm_status enqueue_solve(gfm_ctx *h, const gfm_solve_opts *o, const double *rhs,
             lv.xb = d.xb;
             lv.res = d.res;
         }
-        kernel = mgk;
+        kernel = mp.kernel;
     }
     void *jargs[] = {&a, &ba}, *margs[] = {&m};
     prof_record(h, 2, s);
-    GFM_CUDA(h, cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(threads), h->mg_valid ? margs : jargs, lp.dyn, s));
+    GFM_CUDA(h, cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(threads), h->mg_valid ? margs : jargs,
+                                            h->mg_valid ? mp.dyn : lp.dyn, s));
     prof_record(h, 3, s);
     h->prof.grid = grid;
     h->prof.threads = threads;
@@ -717,6 +771,8 @@ gfm_status setup_mg(gfm_ctx *h, MgFuture &built, cudaStream_t s)
         MgDev &d = h->mg[l];
         d.n = q.n;
         d.n_slices = q.n_slices;
+        d.max_width = q.max_width;
+        d.max_child = q.max_child;
         up(&d.sp, q.slice_ptr);
         up(&d.col, q.col);
         up(&d.face, q.face);
@@ -728,7 +784,7 @@ gfm_status setup_mg(gfm_ctx *h, MgFuture &built, cudaStream_t s)
         const size_t np = (size_t)q.n_pad, ns = (size_t)q.n_slots;
 #define A(ptr, cnt) \
     if (e == cudaSuccess) e = dalloc(&d.ptr, (cnt))
-        A(gamma, (size_t)q.F); A(val64, ns); A(val32, ns); A(pin64, np); A(pin32, np); A(dinv64, np); A(dinv32, np);
+        A(gamma, (size_t)q.F); A(val64, ns); A(val32, ns); A(pin64, np); A(diag64, np); A(pin32, np); A(dinv64, np); A(dinv32, np);
         A(b, np); A(xa, np); A(xb, np); A(res, np);
 #undef A
         double *zero[] = {d.b, d.xa, d.xb, d.res};
@@ -1184,6 +1240,7 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
             ma.gamma = d.gamma;
             ma.val64 = d.val64;
             ma.pin64 = d.pin64;
+            ma.diag64 = d.diag64;
             ma.dinv64 = d.dinv64;
             ma.val32 = d.val32;
             ma.pin32 = d.pin32;

@@ -314,15 +314,25 @@ struct MgLevel {
     int32_t n, n_slices;
     const int32_t *sp, *col;    // sliced-ELL graph
     const void *val, *dinv;     // coefficients per slot, 1 / diagonal
-    const void *pin;            // pin per node (coarse levels)
+    const void *pin;            // float: pin per node (coarse levels); double: diagonal
     const int32_t *cp, *child;  // children in the next finer level (coarse levels)
     void *b, *xa, *xb, *res;    // right-hand side, iterates, residual
+};
+
+// Shared-memory layout of one tail level: byte offsets into the dynamic
+// shared memory, rows padded to np, w faces per row, cw children per node.
+constexpr int kMgTailMax = 14;    // a named barrier each
+constexpr int kMgTailWidth = 16;  // most faces of a row
+struct MgTail {
+    int32_t n, np, w, cw;
+    int32_t val, dinv, pin, b, xa, xb, col, child;
 };
 
 struct MgArgs {
     SolveArgs s;
     int32_t L;       // levels
-    int32_t tail;    // levels from this one on run in CTA 0 alone
+    int32_t tail;    // levels from this one on run in CTA 0 alone, in shared memory
+    MgTail tl[kMgTailMax];  // [L - tail]
     int32_t T;       // tanks (1: a single mesh)
     const int32_t *tank_off;  // batched: [T+1] internal cell offsets
     const DevParams *tprm;    // batched: pin of each tank
@@ -339,7 +349,7 @@ struct MgLevelArgs {
     const DevParams *prm;
     const int32_t *stank;     // batched: tank of each mesh slice (else nullptr)
     const DevParams *tprm;
-    double *gamma, *val64, *pin64, *dinv64;
+    double *gamma, *val64, *pin64, *diag64, *dinv64;
     float *val32, *pin32, *dinv32;
 };
 cudaError_t launch_mg_level(const MgLevelArgs &a, cudaStream_t s);

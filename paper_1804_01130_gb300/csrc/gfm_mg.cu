@@ -15,9 +15,9 @@
 // A V-cycle on the mesh level is five passes over the rows (two sweeps, the
 // residual, two sweeps), all of them gathers of ONE vector, against the one
 // pass of a Jacobi iteration; the coarse levels add a third (2D) or a
-// seventh (3D).  A is applied in difference form, sum_f gamma_f (x_i - x_j) +
-// pin_i x_i, which keeps the zero row sums of the GFM Laplacian exact.  The
-// CG direction needs no pass of its own gathers: s = A p is updated as
+// seventh (3D).  The FP32 operator is applied in difference form, sum_f
+// gamma_f (x_i - x_j) + pin_i x_i, which keeps the zero row sums of the GFM
+// Laplacian exact; the FP64 one in diagonal form.  The CG direction needs no pass of its own gathers: s = A p is updated as
 // s = A z + beta s.
 //
 // Precision.  GFM_FP64 (T = double): everything FP64; the result is accepted
@@ -27,8 +27,8 @@
 // convergence) e is folded into x in FP64 and r becomes the true FP64
 // residual; the direction is kept.
 //
-// Levels too small to share between CTAs run in CTA 0 alone with CTA
-// barriers while the others wait at the grid barrier (from MgArgs::tail on).
+// Levels too small to share between CTAs run in CTA 0 alone, in its shared
+// memory, while the others wait at the grid barrier (from MgArgs::tail on).
 //
 // Batches: rows of all tanks form one block-diagonal system, so the V-cycle
 // needs no tank bookkeeping; only the dot products, alpha, beta and the
@@ -183,9 +183,36 @@ __device__ __forceinline__ bool mg_allreduce(Ctx &c)
 }
 
 // ---- row passes --------------------------------------------------------------
-// acc_i = sum_k val (x_i - x_j) over the rows of slices s0 + w0, + nw, ...
-// below s1 (U of them in flight per warp, chunks of CH faces), then
-// op.post(i, x_i, acc_i, pre) with pre = op.pre(i) loaded before the gathers.
+// The rows' off-diagonal parts, in the form each precision can afford:
+//  float:  acc_i = sum_k val (x_i - x_j), which keeps the zero row sums exact
+//          under FP32 rounding; A x = acc + pin x.
+//  double: acc_i = sum_k val x_j, half the instructions of the FP64 pipe
+//          (64 cycles each per quarter SM); A x = diag x - acc, and a sweep
+//          x + w D^{-1} (b - A x) = (1 - w) x + w D^{-1} (b + acc).
+template <typename T>
+__device__ __forceinline__ T row_add(T acc, T g, T xi, T xj)
+{
+    if constexpr (sizeof(T) == 8) return fma(g, xj, acc);
+    else return fma(g, xi - xj, acc);
+}
+// A x of a row; p its pin (float) or diagonal (double)
+template <typename T>
+__device__ __forceinline__ T row_ax(T acc, T x, T p)
+{
+    if constexpr (sizeof(T) == 8) return fma(p, x, -acc);
+    else return fma(p, x, acc);
+}
+// x + w d (b - A x)
+template <typename T>
+__device__ __forceinline__ T row_sweep(T acc, T x, T b, T w, T d, T p)
+{
+    if constexpr (sizeof(T) == 8) return fma(w * d, b + acc, (T(1) - w) * x);
+    else return fma(w * d, b - fma(p, x, acc), x);
+}
+
+// Rows of slices s0 + w0, + nw, ... below s1 (U of them in flight per warp,
+// chunks of CH faces), then op.post(i, x_i, acc_i, pre) with pre = op.pre(i)
+// loaded before the gathers.
 template <typename T, int CH, int U, bool FINE, typename Op>
 __device__ __forceinline__ void row_pass(const MgLevel &lv, const T *X, int s0, int s1, int w0, int nw, int lane, int n,
                                          Op &op)
@@ -236,7 +263,7 @@ __device__ __forceinline__ void row_pass(const MgLevel &lv, const T *X, int s0, 
 #pragma unroll
             for (int u = 0; u < U; ++u)
 #pragma unroll
-                for (int q = 0; q < CH; ++q) acc[u] = fma(gm[u][q], xi[u] - xj[u][q], acc[u]);
+                for (int q = 0; q < CH; ++q) acc[u] = row_add(acc[u], gm[u][q], xi[u], xj[u][q]);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -246,8 +273,9 @@ __device__ __forceinline__ void row_pass(const MgLevel &lv, const T *X, int s0, 
     }
 }
 
-// The pinned cell's extra diagonal: on the mesh one cell of the tank, on a
-// coarse level an array (zero but for the aggregate holding the pinned cell).
+// What a row needs of its diagonal: the pin (float; on the mesh one cell of
+// the tank, on a coarse level an array that is zero but for the aggregate
+// holding the pinned cell), or the diagonal (double, an array).
 template <typename T, bool FINE>
 struct Pin {
     const T *a;
@@ -255,7 +283,7 @@ struct Pin {
     T pin;
     __device__ __forceinline__ T at(int i) const
     {
-        if constexpr (FINE) return i == ref ? pin : T(0);
+        if constexpr (FINE && sizeof(T) == 4) return i == ref ? pin : T(0);
         else return a[i];
     }
 };
@@ -270,10 +298,13 @@ struct SweepOp {
     T *out;
     T w;
     Pin<T, FINE> pin;
-    __device__ __forceinline__ Pre pre(int i) const { return Pre{b[i], dinv[i], pin.at(i)}; }
-    __device__ __forceinline__ void post(int i, T x, T ax, const Pre &p)
+    __device__ __forceinline__ Pre pre(int i) const
     {
-        out[i] = fma(w * p.d, p.b - fma(p.p, x, ax), x);
+        return Pre{b[i], dinv[i], sizeof(T) == 8 ? T(0) : pin.at(i)};
+    }
+    __device__ __forceinline__ void post(int i, T x, T acc, const Pre &p)
+    {
+        out[i] = row_sweep(acc, x, p.b, w, p.d, p.p);
     }
 };
 
@@ -287,7 +318,7 @@ struct ResidOp {
     T *out;
     Pin<T, FINE> pin;
     __device__ __forceinline__ Pre pre(int i) const { return Pre{b[i], pin.at(i)}; }
-    __device__ __forceinline__ void post(int i, T x, T ax, const Pre &p) { out[i] = p.b - fma(p.p, x, ax); }
+    __device__ __forceinline__ void post(int i, T x, T acc, const Pre &p) { out[i] = p.b - row_ax(acc, x, p.p); }
 };
 
 // The last sweep on the mesh: z = x + w D^{-1} (r - A x), and r.z.
@@ -300,15 +331,37 @@ struct LastOp {
     T *out;
     T w;
     Pin<T, true> pin;
-    typename AccOf<T>::type acc;
-    __device__ __forceinline__ Pre pre(int i) const { return Pre{b[i], dinv[i], pin.at(i)}; }
-    __device__ __forceinline__ void post(int i, T x, T ax, const Pre &p)
+    typename AccOf<T>::type sum;
+    __device__ __forceinline__ Pre pre(int i) const
     {
-        const T z = fma(w * p.d, p.b - fma(p.p, x, ax), x);
+        return Pre{b[i], dinv[i], sizeof(T) == 8 ? T(0) : pin.at(i)};
+    }
+    __device__ __forceinline__ void post(int i, T x, T acc, const Pre &p)
+    {
+        const T z = row_sweep(acc, x, p.b, w, p.d, p.p);
         out[i] = z;
-        acc_add(acc, p.b * z);
+        acc_add(sum, p.b * z);
     }
 };
+
+// fine[child] += z for the children of node i of a level.
+template <typename T>
+__device__ __forceinline__ void add_to_children(const MgLevel &lv, T *fine, int i, T z)
+{
+    const int s = i >> 5, lane = i & 31;
+    const int c0 = __ldg(lv.cp + s), w0 = (__ldg(lv.cp + s + 1) - c0) >> 5;
+    for (int k = 0; k < w0; k += 4) {
+        int ch[4];
+        T v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) ch[q] = k + q < w0 ? __ldg(lv.child + c0 + (k + q) * kSlice + lane) : -1;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = ch[q] >= 0 ? fine[ch[q]] : T(0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (ch[q] >= 0) fine[ch[q]] = v[q] + z;
+    }
+}
 
 // The last sweep on a coarse level, its result added to the children.
 template <typename T>
@@ -316,28 +369,18 @@ struct LastCoarseOp {
     struct Pre {
         T b, d, p;
     };
-    const T *b, *dinv;
-    const int32_t *cp, *child;
+    const MgLevel &lv;
     T *fine;
     T w;
     Pin<T, false> pin;
-    __device__ __forceinline__ Pre pre(int i) const { return Pre{b[i], dinv[i], pin.at(i)}; }
-    __device__ __forceinline__ void post(int i, T x, T ax, const Pre &p)
+    __device__ __forceinline__ Pre pre(int i) const
     {
-        const T z = fma(w * p.d, p.b - fma(p.p, x, ax), x);
-        const int s = i >> 5, lane = i & 31;
-        const int c0 = __ldg(cp + s), w0 = (__ldg(cp + s + 1) - c0) >> 5;
-        for (int k = 0; k < w0; k += 4) {
-            int ch[4];
-            T v[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) ch[q] = k + q < w0 ? __ldg(child + c0 + (k + q) * kSlice + lane) : -1;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) v[q] = ch[q] >= 0 ? fine[ch[q]] : T(0);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (ch[q] >= 0) fine[ch[q]] = v[q] + z;
-        }
+        return Pre{static_cast<const T *>(lv.b)[i], static_cast<const T *>(lv.dinv)[i],
+                   sizeof(T) == 8 ? T(0) : pin.at(i)};
+    }
+    __device__ __forceinline__ void post(int i, T x, T acc, const Pre &p)
+    {
+        add_to_children<T>(lv, fine, i, row_sweep(acc, x, p.b, w, p.d, p.p));
     }
 };
 
@@ -351,18 +394,18 @@ struct DirOp {
     T be;
     bool fresh;
     Pin<T, true> pin;
-    typename AccOf<T>::type acc;
+    typename AccOf<T>::type sum;
     __device__ __forceinline__ Pre pre(int i) const
     {
         return fresh ? Pre{T(0), T(0), pin.at(i)} : Pre{P[i], S[i], pin.at(i)};
     }
-    __device__ __forceinline__ void post(int i, T x, T ax, const Pre &p)
+    __device__ __forceinline__ void post(int i, T x, T acc, const Pre &p)
     {
-        const T s = fma(be, p.s, fma(p.pin, x, ax));
+        const T s = fma(be, p.s, row_ax(acc, x, p.pin));
         const T d = fma(be, p.p, x);
         S[i] = s;
         P[i] = d;
-        acc_add(acc, d * s);
+        acc_add(sum, d * s);
     }
 };
 
@@ -400,60 +443,300 @@ __device__ __forceinline__ void split(int ns, int G, int b, int &s0, int &s1)
     s1 = (int)(((long long)ns * (b + 1)) / G);
 }
 
+// ---- the tail: small levels in CTA 0's shared memory -------------------------
+template <int N>
+struct Int {
+    static constexpr int value = N;
+};
+
+// Barrier t + 1 over the first `nwarps` warps (one warp: a warp barrier).
+__device__ __forceinline__ void tail_bar(int t, int nwarps)
+{
+    if (nwarps == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(t + 1), "r"(nwarps * 32) : "memory");
+}
+
+// Stage the tail levels' tables (constant during a solve), all threads of CTA 0.
+// Padding slots point at the row itself with coefficient 0; a missing child at
+// the element after the finer vector's last, which xa keeps at 0.
+template <typename T>
+__device__ void tail_stage(const MgArgs &a, unsigned char *dsm)
+{
+    for (int l = a.tail; l < a.L; ++l) {
+        const MgTail &q = a.tl[l - a.tail];
+        const MgLevel &lv = a.lv[l];
+        T *val = reinterpret_cast<T *>(dsm + q.val), *dinv = reinterpret_cast<T *>(dsm + q.dinv);
+        T *pin = reinterpret_cast<T *>(dsm + q.pin), *xa = reinterpret_cast<T *>(dsm + q.xa);
+        uint16_t *col = reinterpret_cast<uint16_t *>(dsm + q.col), *child = reinterpret_cast<uint16_t *>(dsm + q.child);
+        int32_t *gchild = reinterpret_cast<int32_t *>(dsm + q.child);
+        if (threadIdx.x == 0) xa[q.np] = T(0);
+        for (int i = threadIdx.x; i < q.np; i += blockDim.x) {
+            const bool on = i < q.n;
+            dinv[i] = on ? static_cast<const T *>(lv.dinv)[i] : T(0);
+            pin[i] = on ? static_cast<const T *>(lv.pin)[i] : T(0);
+            const int s = i >> 5, lane = i & 31;
+            const int base = __ldg(lv.sp + s), w = (__ldg(lv.sp + s + 1) - base) >> 5;
+            for (int k = 0; k < q.w; ++k) {
+                const int slot = base + k * kSlice + lane;
+                val[k * q.np + i] = k < w ? __ldg(static_cast<const T *>(lv.val) + slot) : T(0);
+                col[k * q.np + i] = (uint16_t)(k < w ? __ldg(lv.col + slot) : i);
+            }
+            const int c0 = __ldg(lv.cp + s), cw = (__ldg(lv.cp + s + 1) - c0) >> 5;
+            for (int k = 0; k < q.cw; ++k) {
+                const int ch = k < cw ? __ldg(lv.child + c0 + k * kSlice + lane) : -1;
+                if (l == a.tail) gchild[k * q.np + i] = ch;
+                else child[k * q.np + i] = (uint16_t)(ch >= 0 ? ch : a.tl[l - a.tail - 1].np);
+            }
+        }
+    }
+    __syncthreads();
+}
+
+// The rows a thread holds of one tail level, W faces each (padded), in registers.
+template <typename T, int W, int R>
+struct TailRows {
+    T val[R][W], d[R], pin[R];
+    int col[R][W];
+    __device__ __forceinline__ TailRows(const MgTail &q, const unsigned char *dsm, int tid, int nth)
+    {
+        const T *v = reinterpret_cast<const T *>(dsm + q.val);
+        const uint16_t *cl = reinterpret_cast<const uint16_t *>(dsm + q.col);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int i = tid + r * nth;
+            const bool on = r == 0 || i < q.np;
+#pragma unroll
+            for (int k = 0; k < W; ++k) {
+                const bool ok = on && k < q.w;
+                val[r][k] = ok ? v[k * q.np + i] : T(0);
+                col[r][k] = ok ? (int)cl[k * q.np + i] : 0;
+            }
+            d[r] = on ? reinterpret_cast<const T *>(dsm + q.dinv)[i] : T(0);
+            pin[r] = on ? reinterpret_cast<const T *>(dsm + q.pin)[i] : T(0);
+        }
+    }
+    __device__ __forceinline__ T off_diagonal(int r, T xi, const T *x) const
+    {
+        T xj[W], acc = T(0);
+#pragma unroll
+        for (int k = 0; k < W; ++k) xj[k] = x[col[r][k]];
+#pragma unroll
+        for (int k = 0; k < W; ++k) acc = row_add(acc, val[r][k], xi, xj[k]);
+        return acc;
+    }
+    // b - A x of row r, xi its own value; and a sweep with weight w
+    __device__ __forceinline__ T resid(int r, T b, T xi, const T *x) const
+    {
+        return b - row_ax(off_diagonal(r, xi, x), xi, pin[r]);
+    }
+    __device__ __forceinline__ T sweep(int r, T b, T xi, T w, const T *x) const
+    {
+        return row_sweep(off_diagonal(r, xi, x), xi, b, w, d[r], pin[r]);
+    }
+};
+
+// One tail level of the V-cycle on the way down (restriction, two sweeps,
+// residual into xa) and on the way up (two sweeps, the result added to the
+// children).  t = 0: the children are in global memory.
+template <typename T, int W, int R>
+__device__ __forceinline__ void tail_down(const MgArgs &a, unsigned char *dsm, int t, bool last, int nwp)
+{
+    const MgTail &q = a.tl[t];
+    const int nth = nwp * 32, tid = threadIdx.x;
+    const T om1 = T(kOm1), om2 = T(kOm2);
+    auto vec = [&](int off) { return reinterpret_cast<T *>(dsm + off); };
+    T *b = vec(q.b), *xa = vec(q.xa), *xb = vec(q.xb);
+    T br[R], x[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) br[r] = T(0);
+    if (t == 0) {
+        const T *res = static_cast<const T *>(a.lv[a.tail - 1].res);
+        const int32_t *child = reinterpret_cast<const int32_t *>(dsm + q.child);
+        for (int k = 0; k < q.cw; k += 4) {
+            T v[R][4];
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int i = tid + r * nth;
+                    const int ch = (i < q.np && k + u < q.cw) ? child[(k + u) * q.np + i] : -1;
+                    v[r][u] = ch >= 0 ? res[ch] : T(0);
+                }
+#pragma unroll
+            for (int r = 0; r < R; ++r) br[r] += (v[r][0] + v[r][1]) + (v[r][2] + v[r][3]);
+        }
+    } else {
+        const T *res = vec(a.tl[t - 1].xa);
+        const uint16_t *child = reinterpret_cast<const uint16_t *>(dsm + q.child);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int i = tid + r * nth;
+            if (i < q.np)
+                for (int k = 0; k < q.cw; ++k) br[r] += res[child[k * q.np + i]];
+        }
+    }
+    const TailRows<T, W, R> row(q, dsm, tid, nth);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = tid + r * nth;
+        x[r] = om1 * row.d[r] * br[r];
+        if (i < q.np) {
+            b[i] = br[r];
+            xa[i] = x[r];
+        }
+    }
+    tail_bar(t, nwp);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = tid + r * nth;
+        x[r] = row.sweep(r, br[r], x[r], om2, xa);
+        if (i < q.np) xb[i] = x[r];
+    }
+    tail_bar(t, nwp);
+    if (last) return;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = tid + r * nth;
+        const T v = row.resid(r, br[r], x[r], xb);
+        if (i < q.np) xa[i] = v;
+    }
+    tail_bar(t, nwp);
+}
+
+template <typename T, int W, int R>
+__device__ __forceinline__ void tail_up(const MgArgs &a, unsigned char *dsm, int t, bool last, int nwp)
+{
+    const MgTail &q = a.tl[t];
+    const int nth = nwp * 32, tid = threadIdx.x;
+    const T om1 = T(kOm1), om2 = T(kOm2);
+    auto vec = [&](int off) { return reinterpret_cast<T *>(dsm + off); };
+    T *xa = vec(q.xa), *xb = vec(q.xb);
+    T br[R], x[R];
+    const TailRows<T, W, R> row(q, dsm, tid, nth);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = tid + r * nth;
+        br[r] = i < q.np ? vec(q.b)[i] : T(0);
+    }
+    if (!last) tail_bar(t, nwp);  // the coarser level's correction is in xb
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = tid + r * nth;
+        x[r] = i < q.np ? xb[i] : T(0);
+        x[r] = row.sweep(r, br[r], x[r], om2, xb);
+        if (i < q.np) xa[i] = x[r];
+    }
+    tail_bar(t, nwp);
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r] = row.sweep(r, br[r], x[r], om1, xa);
+    if (t == 0) {
+        T *fine = static_cast<T *>(a.lv[a.tail - 1].xb);
+        const int32_t *child = reinterpret_cast<const int32_t *>(dsm + q.child);
+        for (int k = 0; k < q.cw; k += 4) {
+            int ch[R][4];
+            T v[R][4];
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int i = tid + r * nth;
+                    ch[r][u] = (i < q.np && k + u < q.cw) ? child[(k + u) * q.np + i] : -1;
+                    v[r][u] = ch[r][u] >= 0 ? fine[ch[r][u]] : T(0);
+                }
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (ch[r][u] >= 0) fine[ch[r][u]] = v[r][u] + x[r];
+        }
+    } else {
+        T *fine = vec(a.tl[t - 1].xb);
+        const uint16_t *child = reinterpret_cast<const uint16_t *>(dsm + q.child);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int i = tid + r * nth;
+            if (i < q.np)
+                for (int k = 0; k < q.cw; ++k) fine[child[k * q.np + i]] += x[r];
+        }
+    }
+}
+
+// Rows per thread and faces per row of a level, as template arguments (the
+// plan admits two rows a thread up to six faces, else one, up to kMgTailWidth
+// faces).
+template <typename T, bool UP>
+__device__ __forceinline__ void tail_level(const MgArgs &a, unsigned char *dsm, int t, bool last, int nwp)
+{
+    auto go = [&](auto w, auto r) {
+        if constexpr (UP) tail_up<T, decltype(w)::value, decltype(r)::value>(a, dsm, t, last, nwp);
+        else tail_down<T, decltype(w)::value, decltype(r)::value>(a, dsm, t, last, nwp);
+    };
+    const int w = a.tl[t].w;
+    if (a.tl[t].np > nwp * 32) {
+        if (w <= 4) go(Int<4>{}, Int<2>{});
+        else go(Int<6>{}, Int<2>{});
+    } else {
+        if (w <= 4) go(Int<4>{}, Int<1>{});
+        else if (w <= 6) go(Int<6>{}, Int<1>{});
+        else go(Int<kMgTailWidth>{}, Int<1>{});
+    }
+}
+
+// The V-cycle over the tail levels, from the residual of level tail - 1 to the
+// correction added to its xb.  Level t is worked on by the first ceil(n / 32)
+// warps and closed by its own named barrier, so the last levels cost a warp
+// barrier per pass.  What it costs is a chain of short passes (five a level):
+// each keeps its rows in registers and touches only shared memory.  For the
+// 2048-node level of the 1024x512 tank and the five below it: 32 us when the
+// passes read global memory, 19 us now, the two grid barriers and the first
+// level's transfers (about 7 us) included.
+template <typename T>
+__device__ void tail_cycle(const MgArgs &a, const Ctx &c, unsigned char *dsm)
+{
+    const int nt = a.L - a.tail;
+    auto warps = [&](int t) { return min(c.nw, a.tl[t].np >> 5); };
+    int t = 0;
+    for (; t < nt && c.warp < warps(t); ++t) tail_level<T, false>(a, dsm, t, t + 1 == nt, warps(t));
+    for (--t; t >= 0; --t) tail_level<T, true>(a, dsm, t, t + 1 == nt, warps(t));
+}
+
 // Levels 1 .. L-1 of the V-cycle, from the mesh's residual (lv[0].res) to the
 // correction added to lv[0].xb.  Ends with a grid barrier.
 template <typename T, int CH>
-__device__ __forceinline__ bool coarse_cycle(const MgArgs &a, Ctx &c)
+__device__ __forceinline__ bool coarse_cycle(const MgArgs &a, Ctx &c, unsigned char *dsm)
 {
     const int L = a.L;
     const T om1 = T(kOm1), om2 = T(kOm2);
-    auto down = [&](int l, int s0, int s1, auto sync) -> bool {
+    int s0, s1;
+    for (int l = 1; l < a.tail; ++l) {
         const MgLevel &lv = a.lv[l];
         const Pin<T, false> pin{static_cast<const T *>(lv.pin), -1, T(0)};
+        split(lv.n_slices, c.g.G, blockIdx.x, s0, s1);
         restrict_pass<T>(lv, static_cast<const T *>(a.lv[l - 1].res), om1, s0, s1, c.warp, c.nw, c.lane);
-        if (!sync()) return false;
+        if (!mg_sync(c)) return false;
         SweepOp<T, false> sw{static_cast<const T *>(lv.b), static_cast<const T *>(lv.dinv), static_cast<T *>(lv.xb), om2, pin};
         row_pass<T, CH, 1, false>(lv, static_cast<const T *>(lv.xa), s0, s1, c.warp, c.nw, c.lane, lv.n, sw);
-        if (!sync()) return false;
+        if (!mg_sync(c)) return false;
         if (l + 1 < L) {
             ResidOp<T, false> rs{static_cast<const T *>(lv.b), static_cast<T *>(lv.res), pin};
             row_pass<T, CH, 1, false>(lv, static_cast<const T *>(lv.xb), s0, s1, c.warp, c.nw, c.lane, lv.n, rs);
-            if (!sync()) return false;
+            if (!mg_sync(c)) return false;
         }
-        return true;
-    };
-    auto up = [&](int l, int s0, int s1, auto sync) -> bool {
-        const MgLevel &lv = a.lv[l];
-        const Pin<T, false> pin{static_cast<const T *>(lv.pin), -1, T(0)};
-        SweepOp<T, false> sw{static_cast<const T *>(lv.b), static_cast<const T *>(lv.dinv), static_cast<T *>(lv.xa), om2, pin};
-        row_pass<T, CH, 1, false>(lv, static_cast<const T *>(lv.xb), s0, s1, c.warp, c.nw, c.lane, lv.n, sw);
-        if (!sync()) return false;
-        LastCoarseOp<T> lc{static_cast<const T *>(lv.b), static_cast<const T *>(lv.dinv), lv.cp, lv.child,
-                           static_cast<T *>(a.lv[l - 1].xb), om1, pin};
-        row_pass<T, CH, 1, false>(lv, static_cast<const T *>(lv.xa), s0, s1, c.warp, c.nw, c.lane, lv.n, lc);
-        return sync();
-    };
-    auto gsync = [&]() { return mg_sync(c); };
-    auto bsync = [&]() {
-        __syncthreads();
-        return true;
-    };
-    int s0, s1;
-    const int tail = a.tail < L ? a.tail : L;
-    for (int l = 1; l < tail; ++l) {
-        split(a.lv[l].n_slices, c.g.G, blockIdx.x, s0, s1);
-        if (!down(l, s0, s1, gsync)) return false;
     }
-    if (tail < L) {
-        if (blockIdx.x == 0) {
-            for (int l = tail; l < L; ++l) down(l, 0, a.lv[l].n_slices, bsync);
-            for (int l = L - 1; l >= tail; --l) up(l, 0, a.lv[l].n_slices, bsync);
-        }
+    if (a.tail < L) {
+        if (blockIdx.x == 0) tail_cycle<T>(a, c, dsm);
         if (!mg_sync(c)) return false;
     }
-    for (int l = tail - 1; l >= 1; --l) {
-        split(a.lv[l].n_slices, c.g.G, blockIdx.x, s0, s1);
-        if (!up(l, s0, s1, gsync)) return false;
+    for (int l = a.tail - 1; l >= 1; --l) {
+        const MgLevel &lv = a.lv[l];
+        const Pin<T, false> pin{static_cast<const T *>(lv.pin), -1, T(0)};
+        split(lv.n_slices, c.g.G, blockIdx.x, s0, s1);
+        SweepOp<T, false> sw{static_cast<const T *>(lv.b), static_cast<const T *>(lv.dinv), static_cast<T *>(lv.xa), om2, pin};
+        row_pass<T, CH, 1, false>(lv, static_cast<const T *>(lv.xb), s0, s1, c.warp, c.nw, c.lane, lv.n, sw);
+        if (!mg_sync(c)) return false;
+        LastCoarseOp<T> lc{lv, static_cast<T *>(a.lv[l - 1].xb), om1, pin};
+        row_pass<T, CH, 1, false>(lv, static_cast<const T *>(lv.xa), s0, s1, c.warp, c.nw, c.lane, lv.n, lc);
+        if (!mg_sync(c)) return false;
     }
     return true;
 }
@@ -504,6 +787,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
     constexpr int UB = kMixed ? 4 : 2;  // the same in the update pass
     using A = typename AccOf<T>::type;
     __shared__ MgShared sh;
+    extern __shared__ __align__(16) unsigned char dsm[];
     Ctx c;
     c.g = Grid{a.s.bar, a.s.err, a.s.partials, a.s.budget_ns, 0u, (int)gridDim.x, 0};
     c.sh = &sh;
@@ -540,6 +824,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
     }
     __syncthreads();
     const int nseg = sh.nseg;
+    if (blockIdx.x == 0 && a.tail < a.L) tail_stage<T>(a, dsm);
     auto bail = [&]() { mg_abort(a); };
 
     const MgLevel &l0 = a.lv[0];
@@ -551,7 +836,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
     auto tank_end = [&](int t) { return T_ > 1 ? a.tank_off[t] + a.s.n_per_tank[t] : a.s.m.n; };
     auto tank_pin = [&](int t) {
         const DevParams *p = T_ > 1 ? a.tprm + t : a.s.prm;
-        return Pin<T, true>{nullptr, p->ref, T(p->pin64)};
+        return Pin<T, true>{static_cast<const T *>(l0.pin), p->ref, T(p->pin64)};
     };
 
     // prologue: x0, ||b||
@@ -714,7 +999,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                 row_pass<T, CH, U, true>(l0, XB, sh.seg_s0[q], sh.seg_s0[q + 1], warp, nw, lane, tank_end(t), op);
             }
             if (!mg_sync(c)) { bail(); return; }
-            if (!coarse_cycle<T, CH>(a, c)) { bail(); return; }
+            if (!coarse_cycle<T, CH>(a, c, dsm)) { bail(); return; }
         }
         fine_sweep(XB, XA, om2);
         if (!mg_sync(c)) { bail(); return; }
@@ -724,7 +1009,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
             if (working(t)) {
                 LastOp<T> op{R, dinv, Z, om1, tank_pin(t), A{}};
                 row_pass<T, CH, U, true>(l0, XA, sh.seg_s0[q], sh.seg_s0[q + 1], warp, nw, lane, tank_end(t), op);
-                v[0] = op.acc;
+                v[0] = op.sum;
             }
             put_partials<1, A>(c, t, v);
         }
@@ -751,7 +1036,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                 else be = sh.be64[t];
                 DirOp<T> op{P, S, be, sh.fresh[t] != 0, tank_pin(t), A{}};
                 row_pass<T, CH, U, true>(l0, Z, sh.seg_s0[q], sh.seg_s0[q + 1], warp, nw, lane, tank_end(t), op);
-                v[0] = op.acc;
+                v[0] = op.sum;
             }
             put_partials<1, A>(c, t, v);
         }
@@ -949,6 +1234,7 @@ __global__ void __launch_bounds__(256) k_mg_level(MgLevelArgs a)
     diag += pin;
     const double d = diag > 0.0 ? 1.0 / diag : 0.0;
     a.pin64[i] = pin;
+    a.diag64[i] = diag;
     a.pin32[i] = (float)pin;
     a.dinv64[i] = d;
     a.dinv32[i] = (float)d;

@@ -355,7 +355,7 @@ std::vector<MgLevelHost> build_mg_levels(int n, int n_pad, int F, const int32_t 
         L.n_slots = L.slice_ptr[(size_t)L.n_slices];
         std::vector<int32_t> cptr, clist;
         group_by(grp, L.n, cptr, clist);
-        to_sell(L.n, L.n_slices, cptr, L.child_ptr, [&](int slot, int, int e) {
+        L.max_child = to_sell(L.n, L.n_slices, cptr, L.child_ptr, [&](int slot, int, int e) {
             if ((size_t)slot >= L.child.size()) L.child.resize((size_t)L.child_ptr[(size_t)L.n_slices]);
             const int32_t ch = e >= 0 ? clist[(size_t)e] : -1;
             // children of the first coarse level are cells: back to internal numbers

@@ -13,7 +13,7 @@ constexpr int kMgCoarsest = 4;     // stop coarsening at this many nodes
 // nodes (of cells, on the first coarse level); its faces collect the finer
 // faces that join two aggregates.
 struct MgLevelHost {
-    int n = 0, n_pad = 0, n_slices = 0, n_slots = 0, max_width = 0, F = 0;
+    int n = 0, n_pad = 0, n_slices = 0, n_slots = 0, max_width = 0, max_child = 0, F = 0;
     std::vector<int32_t> slice_ptr;  // [n_slices + 1] sliced-ELL table of the level's graph, as Sell
     std::vector<int32_t> col;        // [n_slots]
     std::vector<int32_t> face;       // [n_slots] face + 1, 0 on padding slots
