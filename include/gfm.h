@@ -279,7 +279,7 @@ gfm_status gfm_solve_host(gfm_handle h, const double *alpha_host, const double *
  *   V  [n]     cell volumes (required).
  *   xf [3][F]  face centres, or NULL for the midpoints of the two cell centres
  *              (exact on uniform hex meshes).
- * Works on batched handles (densities per tank).  One kernel launch, FP64.
+ * Works on batched handles (densities per tank).  FP64.
  * Errors: GFM_ERR_ARG (NULL p or V, both outputs NULL, U without phi),
  * GFM_ERR_STATE (grad before gfm_assemble), GFM_ERR_CUDA.
  */

@@ -42,7 +42,12 @@ struct gfm_ctx {
     double *val64 = nullptr;
     float *val32 = nullptr;
     // face arrays (caller order)
-    double *lambda = nullptr, *gamma = nullptr, *jump = nullptr, *sigma = nullptr, *phi = nullptr;
+    double *lambda = nullptr, *gamma = nullptr, *jump = nullptr, *phi = nullptr;
+    double *cface = nullptr;  // c_f = (S.S)/(S.d)
+    double2 *gs = nullptr;    // (gamma, sigma): the pair the cell sums gather
+    double4 *grad_rec = nullptr;  // [2 F] records of the gradient's face pass
+    double2 *sd = nullptr;        // [F] (S.d, 1 / (S.d))
+    int32_t *cf_ptr = nullptr, *cell_face = nullptr;  // faces of each cell, caller order (CellFaces)
     double *dl_dlam = nullptr;
     int8_t *kind = nullptr;
     // cell arrays
@@ -147,7 +152,7 @@ cudaError_t dalloc(T **p, size_t count)
 void free_all(gfm_ctx *h)
 {
     void *ptrs[] = {h->owner, h->neighbour, h->Sf, h->C, h->perm, h->iperm, h->slice_ptr, h->col, h->face,
-                    h->val64, h->val32, h->lambda, h->gamma, h->jump, h->sigma, h->phi, h->dl_dlam, h->kind,
+                    h->val64, h->val32, h->lambda, h->gamma, h->jump, h->cface, h->gs, h->grad_rec, h->sd, h->cf_ptr, h->cell_face, h->phi, h->dl_dlam, h->kind,
                     h->alpha, h->b, h->diag, h->dinv, h->x64, h->r64, h->p64, h->q64, h->rhs, h->tmp_user,
                     h->tmp_user2, h->UP0, h->UP1, h->Q0, h->Q1, h->P32, h->R32, h->S32, h->E, h->dinv32, h->stage_alpha,
                     h->stage_phi, h->stage_p, h->prm, h->bar,
@@ -622,7 +627,7 @@ gfm_status alloc_upload(gfm_ctx *h, cudaStream_t s)
     A(owner, F); A(neighbour, F); A(Sf, 3 * (size_t)F); A(C, 3 * (size_t)n);
     A(perm, n); A(iperm, np); A(slice_ptr, (size_t)h->ht.n_slices + 1); A(col, ns); A(face, ns);
     A(val64, ns); A(val32, ns);
-    A(lambda, F); A(gamma, F); A(jump, F); A(sigma, F); A(phi, F); A(dl_dlam, F); A(kind, F);
+    A(lambda, F); A(gamma, F); A(jump, F); A(cface, F); A(gs, F); A(grad_rec, 2 * (size_t)F); A(sd, F); A(phi, F); A(dl_dlam, F); A(kind, F);
     A(alpha, n); A(b, np); A(diag, np); A(dinv, np); A(x64, np); A(r64, np); A(p64, np); A(q64, np);
     A(rhs, np); A(tmp_user, n); A(tmp_user2, n); A(UP0, np); A(UP1, np); A(Q0, np); A(Q1, np); A(P32, np); A(R32, np); A(S32, np); A(E, np);
     A(dinv32, np);
@@ -663,7 +668,8 @@ gfm_status alloc_upload(gfm_ctx *h, cudaStream_t s)
     return GFM_OK;
 }
 
-// Compact operator table (after the mesh is on the device).  Usable when
+// c_f and S.d of every face, the cells' faces in caller order, and the compact
+// operator table (after the mesh is on the device).  The table is usable when
 // every slot's neighbour lies within a signed 16-bit offset of its own cell
 // and the faces fall into few classes of bit-identical c_f = S.S/S.d (per
 // tank in a batch): off the interface a face's FP32 coefficient is then one
@@ -672,6 +678,26 @@ gfm_status alloc_upload(gfm_ctx *h, cudaStream_t s)
 gfm_status setup_compact(gfm_ctx *h, cudaStream_t s)
 {
     h->ct_ok = false;
+    const int F = h->F;
+    GFM_CUDA(h, gfm::launch_face_c(h->n, F, h->owner, h->neighbour, h->Sf, h->C, h->cface, h->sd, s));
+    {
+        const int ns = (h->n + 31) / 32;
+        std::vector<int32_t> ptr((size_t)ns + 1, 0);
+        if (dalloc(&h->cf_ptr, (size_t)ns + 1) != cudaSuccess) return fail(h, GFM_ERR_NOMEM, "cell-face table");
+        GFM_CUDA(h, gfm::launch_cell_face_width(sell_of(h), h->perm, h->cf_ptr + 1, s));
+        GFM_CUDA(h, cudaMemcpyAsync(ptr.data() + 1, h->cf_ptr + 1, sizeof(int32_t) * ns, cudaMemcpyDeviceToHost, s));
+        GFM_CUDA(h, cudaStreamSynchronize(s));
+        long long total = 0;
+        for (int q = 1; q <= ns; ++q) {
+            total += 32LL * ptr[(size_t)q];
+            if (total > INT32_MAX) return fail(h, GFM_ERR_ARG, "mesh too large for 32-bit slot offsets");
+            ptr[(size_t)q] = (int32_t)total;
+        }
+        if (dalloc(&h->cell_face, (size_t)total) != cudaSuccess) return fail(h, GFM_ERR_NOMEM, "cell-face table");
+        GFM_CUDA(h, cudaMemcpyAsync(h->cf_ptr, ptr.data(), sizeof(int32_t) * (ns + 1), cudaMemcpyHostToDevice, s));
+        GFM_CUDA(h, gfm::launch_cell_faces(sell_of(h), h->perm, h->cf_ptr, h->cell_face, s));
+        GFM_CUDA(h, cudaStreamSynchronize(s));
+    }
     const gfm::HostTables &ht = h->ht;
     for (int sl = 0; sl < ht.n_slices; ++sl) {
         const int base = ht.slice_ptr[(size_t)sl], w = (ht.slice_ptr[(size_t)sl + 1] - base) / gfm::kSlice;
@@ -683,14 +709,9 @@ gfm_status setup_compact(gfm_ctx *h, cudaStream_t s)
                 if (off < -32768 || off > 32767) return GFM_OK;
             }
     }
-    const int F = h->F;
-    double *dc = nullptr;
-    if (dalloc(&dc, (size_t)F) != cudaSuccess) return fail(h, GFM_ERR_NOMEM, "compact table set-up");
     std::vector<double> c((size_t)F);
-    cudaError_t e = gfm::launch_face_c(h->n, F, h->owner, h->neighbour, h->Sf, h->C, dc, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c.data(), dc, sizeof(double) * F, cudaMemcpyDeviceToHost, s);
+    cudaError_t e = cudaMemcpyAsync(c.data(), h->cface, sizeof(double) * F, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(dc);
     if (e != cudaSuccess) return cuda_fail(h, e, "compact table set-up");
     const int max_cls = (gfm::kMaxDict - 1) / 2;
     std::vector<int32_t> fcls((size_t)F), ctank;
@@ -741,7 +762,7 @@ MgFuture start_mg(const gfm_ctx *h, const std::vector<int32_t> &owner, const std
     static_assert(gfm::kMgLevels == gfm::kMgMaxLevels, "level limits differ");
     auto build = [h, &owner, &nb, &Sf, &C]() {
         return gfm::build_mg_levels(h->n, h->ht.n_pad, h->F, owner.data(), nb.data(), Sf.data(), C.data(),
-                                    h->ht.perm.data());
+                                    h->ht.perm.data(), h->ht.face.data(), h->ht.n_slots);
     };
     try {
         return std::async(std::launch::async, build);
@@ -841,6 +862,16 @@ gfm_status plan_batch(gfm_ctx *h)
     if (e != cudaSuccess) return cuda_fail(h, e, "uploading the CTA table");
     h->cta_grid = grid;
     return GFM_OK;
+}
+
+// RN(1 / b) for div_known, 0 where its conditions do not hold.
+double known_inverse(double b)
+{
+    int e = 0;
+    const double m = std::frexp(b, &e);
+    if (!(b > 0.0) || !std::isfinite(b) || e < -200 || e > 200) return 0.0;
+    if (m == 1.0 - 1.1102230246251565e-16) return 0.0;  // a significand of all ones
+    return 1.0 / b;
 }
 
 gfm::CoarseArgs coarse_args(gfm_ctx *h)
@@ -1136,13 +1167,12 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
     h->phys = *phys;
     h->ref_internal = (h->batched || phys->ref_cell >= 0) ? (h->batched ? 0 : h->ht.perm[(size_t)phys->ref_cell]) : -1;
     GFM_CUDA(h, cudaMemcpyAsync(h->alpha, alpha, sizeof(double) * h->n, cudaMemcpyDeviceToDevice, s));
-    GFM_CUDA(h, cudaMemcpyAsync(h->phi, phi, sizeof(double) * h->F, cudaMemcpyDeviceToDevice, s));
     GFM_CUDA(h, cudaMemsetAsync(h->prm, 0, sizeof(gfm::DevParams), s));
     if (h->batched) {
         for (int t = 0; t < h->T; ++t) {
             const gfm_phys &ph = phys[t];
-            gfm::TankPhys tp{ph.rho_w, ph.rho_a, ph.g[0], ph.g[1], ph.g[2], ph.ref_value,
-                             h->ht.perm[(size_t)h->bt.coff[(size_t)t] + ph.ref_cell], 0};
+            gfm::TankPhys tp{ph.rho_w, ph.rho_a, ph.g[0], ph.g[1], ph.g[2], ph.ref_value, known_inverse(ph.rho_w),
+                             known_inverse(ph.rho_a), h->ht.perm[(size_t)h->bt.coff[(size_t)t] + ph.ref_cell], 0};
             h->tphys_h[t] = tp;
             gfm::DevParams dp{};
             dp.ref = tp.ref;
@@ -1156,19 +1186,22 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
     fa.F = h->F;
     fa.owner = h->owner;
     fa.neighbour = h->neighbour;
-    fa.Sf = h->Sf;
+    fa.c = h->cface;
     fa.C = h->C;
     fa.alpha = h->alpha;
-    fa.phi = h->phi;
+    fa.phi = phi;
+    fa.phi_copy = h->phi;
     fa.rho_w = phys->rho_w;
     fa.rho_a = phys->rho_a;
     fa.g0 = phys->g[0];
     fa.g1 = phys->g[1];
     fa.g2 = phys->g[2];
+    fa.inv_w = known_inverse(phys->rho_w);
+    fa.inv_a = known_inverse(phys->rho_a);
     fa.lambda = h->lambda;
     fa.gamma = h->gamma;
     fa.jump = h->jump;
-    fa.sigma = h->sigma;
+    fa.gs = h->gs;
     fa.kind = h->kind;
     fa.ftank = h->batched ? h->ftank : nullptr;
     fa.tphys = h->batched ? h->tphys : nullptr;
@@ -1178,8 +1211,13 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
     // the compact table's codes hold only while gamma_f off the interface is
     // c_f / rho of the phase, i.e. without a face Rhie-Chow coefficient
     const bool use_ct = h->ct_ok && !h->rau_set;
+    // A pinned system is preconditioned by multigrid, whose coarse levels
+    // follow from gamma; the one-phase regions are then only reported
+    // (gfm_get_coarse finds them).  Unpinned systems and gfm_set_coarse(0)
+    // take the Jacobi forms, the only ones that read the compact table.
+    const bool use_mg = h->ref_internal >= 0 && h->coarse_max > 0;
     int launched = 2;
-    if (use_ct) {
+    if (use_ct && !use_mg) {
         gfm::DictArgs da{};
         da.n_cls = h->n_cls;
         da.ccls = h->ccls;
@@ -1193,8 +1231,7 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
     }
     gfm::CellArgs ca{};
     ca.m = sell_of(h);
-    ca.gamma = h->gamma;
-    ca.sigma = h->sigma;
+    ca.gs = h->gs;
     ca.ref = h->ref_internal;
     ca.ref_value = phys->ref_value;
     ca.b = h->b;
@@ -1206,20 +1243,16 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
     ca.stank = h->batched ? h->stank : nullptr;
     ca.tphys = h->batched ? h->tphys : nullptr;
     ca.tprm = h->batched ? h->tprm : nullptr;
-    ca.ent = use_ct ? h->ent : nullptr;
+    ca.ent = use_ct && !use_mg ? h->ent : nullptr;
     ca.fcls = h->fcls;
     ca.kind = h->kind;
     ca.pad_code = 2 * h->n_cls;
     GFM_CUDA(h, gfm::launch_cells(ca, s));
     h->ent_valid = use_ct;
-    // A pinned system is preconditioned by multigrid, whose coarse levels
-    // follow from gamma; the one-phase regions are then only reported
-    // (gfm_get_coarse finds them).  Unpinned systems and gfm_set_coarse(0)
-    // take the Jacobi forms.
     h->mg_valid = false;
     h->asm_max = h->coarse_max;
     h->asm_min_size = h->coarse_min_size;
-    if (h->ref_internal >= 0 && h->coarse_max > 0) {
+    if (use_mg) {
         for (size_t l = 0; l < h->mg.size(); ++l) {
             const MgDev &d = h->mg[l];
             gfm::MgLevelArgs ma{};
@@ -1232,7 +1265,7 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
             ma.mem_ptr = d.mem_ptr;
             ma.mem = d.mem;
             ma.scale = d.scale;
-            ma.fine_gamma = l == 0 ? h->gamma : h->mg[l - 1].gamma;
+            ma.fine_gamma = l == 0 ? h->val64 : h->mg[l - 1].gamma;
             ma.fine_pin = l == 0 ? nullptr : h->mg[l - 1].pin64;
             ma.prm = h->prm;
             ma.stank = h->batched ? h->stank : nullptr;
@@ -1403,10 +1436,10 @@ gfm_status gfm_gradient(gfm_handle h, const double *p, const double *V, const do
     clear_stale_error();
     cudaStream_t s = (cudaStream_t)stream;
     gfm::GradArgs a{};
-    a.m = sell_of(h);
     a.n = h->n;
     a.F = h->F;
-    a.iperm = h->iperm;
+    a.cf = gfm::CellFaces{h->cf_ptr, h->cell_face};
+    a.sd = h->sd;
     a.owner = h->owner;
     a.neighbour = h->neighbour;
     a.Sf = h->Sf;
@@ -1415,17 +1448,21 @@ gfm_status gfm_gradient(gfm_handle h, const double *p, const double *V, const do
     a.xf = xf;
     a.lambda = h->lambda;
     a.jump = h->jump;
+    a.kind = h->kind;
     a.p = p;
     a.phi = phi;
     a.rho_w = h->phys.rho_w;
     a.rho_a = h->phys.rho_a;
-    a.stank = h->batched ? h->stank : nullptr;
+    a.inv_w = known_inverse(a.rho_w);
+    a.inv_a = known_inverse(a.rho_a);
+    a.ftank = h->batched ? h->ftank : nullptr;
     a.tphys = h->batched ? h->tphys : nullptr;
+    a.rec = h->grad_rec;
     a.grad = grad;
     a.U = U;
     GFM_CUDA(h, gfm::launch_gradient(a, s));
-    h->prof.launches = 1;
-    h->prof.launches_total += 1;
+    h->prof.launches = 2;
+    h->prof.launches_total += 2;
     return GFM_OK;
 }
 
@@ -1461,10 +1498,10 @@ gfm_status gfm_nonorth_correct(gfm_handle h, const double *p, const double *V, c
         if (e != cudaSuccess) return fail(h, GFM_ERR_NOMEM, "allocating the correction workspace");
     }
     gfm::GradArgs ga{};
-    ga.m = sell_of(h);
     ga.n = h->n;
     ga.F = h->F;
-    ga.iperm = h->iperm;
+    ga.cf = gfm::CellFaces{h->cf_ptr, h->cell_face};
+    ga.sd = h->sd;
     ga.owner = h->owner;
     ga.neighbour = h->neighbour;
     ga.Sf = h->Sf;
@@ -1473,10 +1510,14 @@ gfm_status gfm_nonorth_correct(gfm_handle h, const double *p, const double *V, c
     ga.xf = xf;
     ga.lambda = h->lambda;
     ga.jump = h->jump;
+    ga.kind = h->kind;
     ga.p = p;
     ga.rho_w = h->phys.rho_w;
     ga.rho_a = h->phys.rho_a;
-    ga.stank = h->batched ? h->stank : nullptr;
+    ga.inv_w = known_inverse(ga.rho_w);
+    ga.inv_a = known_inverse(ga.rho_a);
+    ga.rec = h->grad_rec;
+    ga.ftank = h->batched ? h->ftank : nullptr;
     ga.tphys = h->batched ? h->tphys : nullptr;
     ga.grad = h->grad_scr;
     GFM_CUDA(h, gfm::launch_gradient(ga, s));
@@ -1487,22 +1528,22 @@ gfm_status gfm_nonorth_correct(gfm_handle h, const double *p, const double *V, c
     na.neighbour = h->neighbour;
     na.Sf = h->Sf;
     na.C = h->C;
-    na.xf = xf;
+    na.c = h->cface;
     na.rau = h->rau_set ? h->rau : nullptr;
     na.G = h->grad_scr;
+    na.rec = h->grad_rec;
     na.phi = h->phi;
     na.gamma = h->gamma;
     na.jump = h->jump;
     na.corr = h->nonorth_corr;
     na.phi_eff = h->phi_eff;
-    na.sigma = h->sigma;
+    na.gs = h->gs;
     GFM_CUDA(h, gfm::launch_nonorth(na, s));
-    // the cell sums again: b from the corrected sigma (diag and the tables
-    // are rewritten with the same values; the compact table is unchanged)
+    // the cell sums again: b alone, from the corrected sigma
     gfm::CellArgs ca{};
     ca.m = sell_of(h);
-    ca.gamma = h->gamma;
-    ca.sigma = h->sigma;
+    ca.gs = h->gs;
+    ca.source_only = true;
     ca.ref = h->ref_internal;
     ca.ref_value = h->phys.ref_value;
     ca.b = h->b;
@@ -1515,7 +1556,7 @@ gfm_status gfm_nonorth_correct(gfm_handle h, const double *p, const double *V, c
     ca.tphys = h->batched ? h->tphys : nullptr;
     ca.tprm = h->batched ? h->tprm : nullptr;
     GFM_CUDA(h, gfm::launch_cells(ca, s));
-    int launched = 3;
+    int launched = 4;
     if (h->ref_internal < 0) {
         GFM_CUDA(h, gfm::launch_bsums(h->b, h->n, h->prm, s));
         ++launched;
@@ -1552,12 +1593,11 @@ gfm_status gfm_piso_step(gfm_handle h, const gfm_solve_opts *opts, int32_t n_sol
             if (st != GFM_OK) return st;
         } else {
             const double *phik = phi_star + (size_t)k * h->F;
-            GFM_CUDA(h, cudaMemcpyAsync(h->phi, phik, sizeof(double) * h->F, cudaMemcpyDeviceToDevice, s));
-            GFM_CUDA(h, gfm::launch_sigma(h->F, h->phi, h->gamma, h->jump, h->sigma, s));
+            GFM_CUDA(h, gfm::launch_sigma(h->F, phik, h->gamma, h->jump, h->gs, h->phi, s));
             gfm::CellArgs ca{};
             ca.m = sell_of(h);
-            ca.gamma = h->gamma;
-            ca.sigma = h->sigma;
+            ca.gs = h->gs;
+            ca.source_only = true;
             ca.ref = h->ref_internal;
             ca.ref_value = h->phys.ref_value;
             ca.b = h->b;
@@ -1605,11 +1645,10 @@ gfm_status gfm_iso_advect(gfm_handle h, const double *alpha, const double *phi, 
     if (!(dt >= 0.0) || !std::isfinite(dt) || nvt < 3) return fail(h, GFM_ERR_ARG, "dt >= 0 and nvt >= 3");
     clear_stale_error();
     gfm::IsoArgs a{};
-    a.m = sell_of(h);
     a.n = h->n;
     a.F = h->F;
     a.nvt = nvt;
-    a.iperm = h->iperm;
+    a.cf = gfm::CellFaces{h->cf_ptr, h->cell_face};
     a.owner = h->owner;
     a.neighbour = h->neighbour;
     a.alpha = alpha;

@@ -11,12 +11,25 @@ namespace gfm {
 
 enum : int8_t { kDry = 0, kWet = 1, kIfOwnerWet = 2, kIfOwnerDry = 3 };
 
+// a / b correctly rounded from inv = RN(1 / b): one Newton step on the
+// quotient with an exact remainder (Markstein, IBM J. Res. Dev. 34, 1990), for
+// |a| far from under- and overflow and a normal b whose significand is not
+// all ones; the caller passes inv = 0 when b is not.  Three instructions of
+// the FP64 pipe instead of a divide's ten or so.
+__device__ __forceinline__ double div_known(double a, double b, double inv)
+{
+    const int e = (__double2hiint(a) >> 20) & 0x7ff;
+    if (inv == 0.0 || e < 0x100 || e > 0x6ff) return a / b;
+    const double q = a * inv;
+    return fma(fma(-q, b, a), inv, q);
+}
+
 // One thread per internal face (caller order).
 //   wet = alpha >= 0.5 (Sec. 3.1: the alpha = 0.5 contour is the interface;
 //   alpha exactly 0.5 is taken as wet).
 //   interface face: wet owner != wet neighbour.  W = wet cell, D = dry cell.
 //   lambda = (alpha_W - 0.5) / (alpha_W - alpha_D)                 Eq. 13
-//   c      = (S.S) / (S.d),  d = C_nb - C_own
+//   c      = (S.S) / (S.d),  d = C_nb - C_own  (geometry: k_face_c, once per handle)
 //   gamma  = c / (lambda rho_w + (1 - lambda) rho_a)  = c beta+ beta- / beta_w   Eqs. 16-18, 20
 //            (times the face Rhie-Chow coefficient rau_f when one is set)
 //   x_G    = C_W + lambda (C_D - C_W)                              Eq. 12
@@ -25,26 +38,62 @@ enum : int8_t { kDry = 0, kWet = 1, kIfOwnerWet = 2, kIfOwnerDry = 3 };
 //   sigma  = phi + gamma J   (the face's total source flux)
 // Off the interface lambda is 1 (both wet) or 0 (both dry), which yields the
 // phase density exactly.
-__global__ void k_faces(FaceArgs a)
+// What bounds it: the FP64 pipe (a warp's FP64 instruction takes 16 cycles of
+// it, whether one lane or 32 are active) and the random gather of the
+// neighbour's alpha.  So c comes from a table instead of S (24 bytes) and two
+// gathered centres, the division by a phase density is div_known's, and a
+// block first settles its faces off the interface and then packs the few on it
+// into full warps: in a random cell order nearly every warp holds one.
+// With the cell sums gathering (gamma, sigma) as one pair and the first coarse
+// level reading its members' slots, assembly and read-back of 256x128x128 cells
+// in a random order went from 1990 to 1019 us.
+__global__ void __launch_bounds__(256) k_faces(FaceArgs a)
 {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= a.F) return;
-    const int o = a.owner[f], nb = a.neighbour[f];
-    const size_t n = (size_t)a.n, F = (size_t)a.F;
-    const double ao = a.alpha[o], an = a.alpha[nb];
-    const bool wo = ao >= 0.5, wn = an >= 0.5;
-    int8_t kind;
-    double lam;
-    int W = o, D = nb;
-    if (wo == wn) {
-        kind = wo ? kWet : kDry;
-        lam = wo ? 1.0 : 0.0;
-    } else {
-        kind = wo ? kIfOwnerWet : kIfOwnerDry;
-        if (!wo) { W = nb; D = o; }
-        const double aW = a.alpha[W], aD = a.alpha[D];
-        lam = (aW - 0.5) / (aW - aD);
+    __shared__ int list[256];
+    __shared__ int wcount[8];
+    const int f0 = blockIdx.x * 256, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const size_t n = (size_t)a.n;
+    auto put = [&](int f, int8_t kind, double lam, double gam, double J) {
+        const double ph = a.phi[f];
+        if (a.rau) gam = gam * a.rau[f];  // face Rhie-Chow coefficient 1/a_P
+        a.lambda[f] = lam;
+        a.gamma[f] = gam;
+        a.jump[f] = J;
+        a.gs[f] = make_double2(gam, ph + gam * J);
+        a.phi_copy[f] = ph;
+        a.kind[f] = kind;
+    };
+    bool iface = false;
+    if (f0 + (int)threadIdx.x < a.F) {
+        const int f = f0 + threadIdx.x;
+        const bool wo = a.alpha[a.owner[f]] >= 0.5, wn = a.alpha[a.neighbour[f]] >= 0.5;
+        iface = wo != wn;
+        if (!iface) {
+            double rho = wo ? a.rho_w : a.rho_a, inv = wo ? a.inv_w : a.inv_a;
+            if (a.ftank) {
+                const TankPhys *tp = a.tphys + a.ftank[f];
+                rho = wo ? tp->rho_w : tp->rho_a;
+                inv = wo ? tp->inv_w : tp->inv_a;
+            }
+            put(f, wo ? kWet : kDry, wo ? 1.0 : 0.0, div_known(a.c[f], rho, inv), 0.0);
+        }
     }
+    const unsigned m = __ballot_sync(0xffffffffu, iface);
+    if (lane == 0) wcount[warp] = __popc(m);
+    __syncthreads();
+    int before = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        before += w < warp ? wcount[w] : 0;
+        total += wcount[w];
+    }
+    if (total == 0) return;
+    if (iface) list[before + __popc(m & ((1u << lane) - 1u))] = f0 + threadIdx.x;
+    __syncthreads();
+    if ((int)threadIdx.x >= total) return;
+    const int f = list[threadIdx.x];
+    const int o = a.owner[f], nb = a.neighbour[f];
+    const double ao = a.alpha[o], an = a.alpha[nb];
     double rho_w = a.rho_w, rho_a = a.rho_a, g0 = a.g0, g1 = a.g1, g2 = a.g2;
     if (a.ftank) {
         const TankPhys tp = a.tphys[a.ftank[f]];
@@ -54,38 +103,31 @@ __global__ void k_faces(FaceArgs a)
         g1 = tp.g1;
         g2 = tp.g2;
     }
-    const double Sx = a.Sf[f], Sy = a.Sf[F + f], Sz = a.Sf[2 * F + f];
-    const double dx = a.C[nb] - a.C[o];
-    const double dy = a.C[n + nb] - a.C[n + o];
-    const double dz = a.C[2 * n + nb] - a.C[2 * n + o];
-    const double c = (Sx * Sx + Sy * Sy + Sz * Sz) / (Sx * dx + Sy * dy + Sz * dz);
-    const double rf = lam * rho_w + (1.0 - lam) * rho_a;
-    double gam = c / rf;
-    if (a.rau) gam = gam * a.rau[f];  // face Rhie-Chow coefficient 1/a_P
-    double J = 0.0;
-    if (kind >= kIfOwnerWet) {
-        const double xg0 = a.C[W] + lam * (a.C[D] - a.C[W]);
-        const double xg1 = a.C[n + W] + lam * (a.C[n + D] - a.C[n + W]);
-        const double xg2 = a.C[2 * n + W] + lam * (a.C[2 * n + D] - a.C[2 * n + W]);
-        const double H = (rho_w - rho_a) * ((g0 * xg0 + g1 * xg1) + g2 * xg2);
-        J = (kind == kIfOwnerWet) ? H : -H;
-    }
-    a.lambda[f] = lam;
-    a.gamma[f] = gam;
-    a.jump[f] = J;
-    a.sigma[f] = a.phi[f] + gam * J;
-    a.kind[f] = kind;
+    const bool wo = ao >= 0.5;
+    const int W = wo ? o : nb, D = wo ? nb : o;
+    const double aW = wo ? ao : an, aD = wo ? an : ao;
+    const double lam = (aW - 0.5) / (aW - aD);
+    const double gam = a.c[f] / (lam * rho_w + (1.0 - lam) * rho_a);
+    const double xg0 = a.C[W] + lam * (a.C[D] - a.C[W]);
+    const double xg1 = a.C[n + W] + lam * (a.C[n + D] - a.C[n + W]);
+    const double xg2 = a.C[2 * n + W] + lam * (a.C[2 * n + D] - a.C[2 * n + W]);
+    const double H = (rho_w - rho_a) * ((g0 * xg0 + g1 * xg1) + g2 * xg2);
+    put(f, wo ? kIfOwnerWet : kIfOwnerDry, lam, gam, wo ? H : -H);
 }
 
 // One thread per internal cell (lane l of slice s = cell 32 s + l).  Walks
 // the cell's faces in ascending caller face order:
 //   diag_i = sum gamma_f,  b_i = -sum s_if sigma_f  (s = +1 owner, -1 neighbour)
 // fills the sliced-ELL coefficients (FP64 and FP32 copies), and applies the
-// pin: b_r += diag_r * ref_value, diag_r += diag_r.
-__global__ void k_cells(CellArgs a)
+// pin: b_r += diag_r * ref_value, diag_r += diag_r.  SOURCE: b alone, for a
+// new sigma on the same coefficients.
+// Bound by the gathers of (gamma, sigma), one 16-byte load per slot: the loads
+// of four slots are in flight together, the sums keep the face order.
+template <bool SOURCE>
+__global__ void __launch_bounds__(256) k_cells(CellArgs a)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t == 0 && !a.stank) a.prm->ref = a.ref;
+    if (!SOURCE && t == 0 && !a.stank) a.prm->ref = a.ref;
     if (t >= a.m.n_pad) return;
     const int s = t >> 5, l = t & 31;
     int ref = a.ref;
@@ -101,31 +143,51 @@ __global__ void k_cells(CellArgs a)
     const int base = a.m.slice_ptr[s];
     const int w = (a.m.slice_ptr[s + 1] - base) >> 5;
     double diag = 0.0, b = 0.0;
-    for (int k = 0; k < w; ++k) {
-        const int slot = base + k * kSlice + l;
-        const int code = a.m.face[slot];
-        if (code == 0) {
-            a.m.val64[slot] = 0.0;
-            a.m.val32[slot] = 0.0f;
-            if (a.ent) a.ent[slot] = (uint32_t)a.pad_code << 16;  // itself, coefficient 0
-            continue;
+    for (int k0 = 0; k0 < w; k0 += 4) {
+        int code[4];
+        double2 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) code[q] = k0 + q < w ? a.m.face[base + (k0 + q) * kSlice + l] : 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int f = (code[q] > 0 ? code[q] : -code[q]) - 1;
+            v[q] = make_double2(0.0, 0.0);
+            if (code[q] != 0) {
+                if (SOURCE) v[q].y = a.gs[f].y;
+                else v[q] = a.gs[f];
+            }
         }
-        const int f = (code > 0 ? code : -code) - 1;
-        const double g = a.gamma[f];
-        const double sg = a.sigma[f];
-        diag = diag + g;
-        b = (code > 0) ? b - sg : b + sg;
-        a.m.val64[slot] = g;
-        a.m.val32[slot] = (float)g;
-        if (a.ent) {
-            // off the interface the coefficient is the class's one for the
-            // face's phase; interface faces read val32 (escape)
-            const int8_t kd = a.kind[f];
-            const uint32_t vc = kd == kWet ? (uint32_t)(2 * a.fcls[f]) : kd == kDry ? (uint32_t)(2 * a.fcls[f] + 1)
-                                                                                  : kEscape;
-            const int off = a.m.col[slot] - t;
-            a.ent[slot] = (vc << 16) | ((uint32_t)off & 0xFFFFu);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (k0 + q >= w) break;
+            const int slot = base + (k0 + q) * kSlice + l;
+            if (code[q] != 0) {
+                b = (code[q] > 0) ? b - v[q].y : b + v[q].y;
+                if (!SOURCE) diag = diag + v[q].x;
+            }
+            if (SOURCE) continue;
+            a.m.val64[slot] = v[q].x;
+            a.m.val32[slot] = (float)v[q].x;
+            if (a.ent) {
+                // off the interface the coefficient is the class's one for the
+                // face's phase; interface faces read val32 (escape); a padding
+                // slot is the cell itself with coefficient 0
+                uint32_t vc = (uint32_t)a.pad_code;
+                int off = 0;
+                if (code[q] != 0) {
+                    const int f = (code[q] > 0 ? code[q] : -code[q]) - 1;
+                    const int8_t kd = a.kind[f];
+                    vc = kd == kWet ? (uint32_t)(2 * a.fcls[f]) : kd == kDry ? (uint32_t)(2 * a.fcls[f] + 1) : kEscape;
+                    off = a.m.col[slot] - t;
+                }
+                a.ent[slot] = (vc << 16) | ((uint32_t)off & 0xFFFFu);
+            }
         }
+    }
+    if (SOURCE) {
+        if (t == ref) b = b + prm->pin64 * ref_value;
+        a.b[t] = valid ? b : 0.0;
+        return;
     }
     if (t == ref) {
         b = b + diag * ref_value;
@@ -140,19 +202,23 @@ __global__ void k_cells(CellArgs a)
 }
 
 // sigma = phi + gamma J for a new predicted flux on an assembled system (the
-// interface, the coefficients and the jump unchanged), rounded as in k_faces.
+// interface, the coefficients and the jump unchanged), rounded as in k_faces;
+// phi is kept for the corrected flux.
 __global__ void k_sigma(int F, const double *__restrict__ phi, const double *__restrict__ gamma,
-                        const double *__restrict__ jump, double *__restrict__ sigma)
+                        const double *__restrict__ jump, double2 *__restrict__ gs, double *__restrict__ phi_copy)
 {
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f >= F) return;
-    sigma[f] = phi[f] + gamma[f] * jump[f];
+    const double ph = phi[f], g = gamma[f];
+    gs[f] = make_double2(g, ph + g * jump[f]);
+    phi_copy[f] = ph;
 }
 
-// c_f = (S.S)/(S.d) per face, the geometric factor of gamma_f, rounded as in
-// k_faces (the compact table groups faces of bit-identical c_f into classes).
+// c_f = (S.S)/(S.d) per face, the geometric factor of gamma_f (the compact
+// table groups faces of bit-identical c_f into classes).
 __global__ void k_face_c(int n, int F, const int32_t *__restrict__ owner, const int32_t *__restrict__ neighbour,
-                         const double *__restrict__ Sf, const double *__restrict__ C, double *__restrict__ out)
+                         const double *__restrict__ Sf, const double *__restrict__ C, double *__restrict__ out,
+                         double2 *__restrict__ sd)
 {
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f >= F) return;
@@ -162,7 +228,40 @@ __global__ void k_face_c(int n, int F, const int32_t *__restrict__ owner, const 
     const double dx = C[nb] - C[o];
     const double dy = C[nn + nb] - C[nn + o];
     const double dz = C[2 * nn + nb] - C[2 * nn + o];
-    out[f] = (Sx * Sx + Sy * Sy + Sz * Sz) / (Sx * dx + Sy * dy + Sz * dz);
+    const double b = Sx * dx + Sy * dy + Sz * dz;
+    out[f] = (Sx * Sx + Sy * Sy + Sz * Sz) / b;
+    // an inverse for div_known: not for extreme exponents or a significand of all ones
+    const long long bits = __double_as_longlong(b);
+    const int e = (int)(bits >> 52) & 0x7ff;
+    const bool ok = e >= 0x300 && e <= 0x500 && (bits & 0xfffffffffffffLL) != 0xfffffffffffffLL;
+    sd[f] = make_double2(b, ok ? 1.0 / b : 0.0);
+}
+
+// Widths of the caller-order slices (32 cells), and their faces.
+__global__ void k_cell_face_width(Sell m, const int32_t *__restrict__ perm, int32_t *__restrict__ width)
+{
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    int deg = 0;
+    if (c < m.n) {
+        const int i = perm[c], base = m.slice_ptr[i >> 5], w = (m.slice_ptr[(i >> 5) + 1] - base) >> 5;
+        for (int k = 0; k < w; ++k) deg += m.face[base + k * kSlice + (i & 31)] != 0;
+    }
+    for (int off = 16; off; off >>= 1) deg = max(deg, __shfl_xor_sync(0xffffffffu, deg, off));
+    if ((c & 31) == 0 && c < m.n) width[c >> 5] = deg;
+}
+
+__global__ void k_cell_faces(Sell m, const int32_t *__restrict__ perm, const int32_t *__restrict__ ptr,
+                             int32_t *__restrict__ out)
+{
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const int o = ptr[c >> 5], wo = (ptr[(c >> 5) + 1] - o) >> 5;
+    int i = 0, base = 0, w = 0;
+    if (c < m.n) {
+        i = perm[c];
+        base = m.slice_ptr[i >> 5];
+        w = (m.slice_ptr[(i >> 5) + 1] - base) >> 5;
+    }
+    for (int k = 0; k < wo; ++k) out[o + k * kSlice + (c & 31)] = k < w ? m.face[base + k * kSlice + (i & 31)] : 0;
 }
 
 // Dictionary of the compact table: the off-interface coefficients
@@ -311,7 +410,8 @@ cudaError_t launch_faces(const FaceArgs &a, cudaStream_t s)
 
 cudaError_t launch_cells(const CellArgs &a, cudaStream_t s)
 {
-    k_cells<<<blocks_for(a.m.n_pad, 256), 256, 0, s>>>(a);
+    if (a.source_only) k_cells<true><<<blocks_for(a.m.n_pad, 256), 256, 0, s>>>(a);
+    else k_cells<false><<<blocks_for(a.m.n_pad, 256), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -322,18 +422,31 @@ cudaError_t launch_bsums(const double *b, int32_t n, DevParams *prm, cudaStream_
 }
 
 cudaError_t launch_face_c(int32_t n, int32_t F, const int32_t *owner, const int32_t *neighbour, const double *Sf,
-                          const double *C, double *c, cudaStream_t s)
+                          const double *C, double *c, double2 *sd, cudaStream_t s)
 {
     if (F <= 0) return cudaSuccess;
-    k_face_c<<<blocks_for(F, 256), 256, 0, s>>>(n, F, owner, neighbour, Sf, C, c);
+    k_face_c<<<blocks_for(F, 256), 256, 0, s>>>(n, F, owner, neighbour, Sf, C, c, sd);
     return cudaGetLastError();
 }
 
-cudaError_t launch_sigma(int32_t F, const double *phi, const double *gamma, const double *jump, double *sigma,
-                         cudaStream_t s)
+cudaError_t launch_cell_face_width(const Sell &m, const int32_t *perm, int32_t *width, cudaStream_t s)
+{
+    k_cell_face_width<<<blocks_for(m.n, 256), 256, 0, s>>>(m, perm, width);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cell_faces(const Sell &m, const int32_t *perm, const int32_t *ptr, int32_t *out, cudaStream_t s)
+{
+    // whole slices: every thread of a warp has one
+    k_cell_faces<<<(m.n + 31) / 32, 32, 0, s>>>(m, perm, ptr, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sigma(int32_t F, const double *phi, const double *gamma, const double *jump, double2 *gs,
+                         double *phi_copy, cudaStream_t s)
 {
     if (F <= 0) return cudaSuccess;
-    k_sigma<<<blocks_for(F, 256), 256, 0, s>>>(F, phi, gamma, jump, sigma);
+    k_sigma<<<blocks_for(F, 256), 256, 0, s>>>(F, phi, gamma, jump, gs, phi_copy);
     return cudaGetLastError();
 }
 

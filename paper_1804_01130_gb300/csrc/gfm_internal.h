@@ -19,6 +19,7 @@ constexpr int kCoarseEParts = 128;    // blocks summing E = Z^T A Z
 // Physics of one tank of a batch (device copy of gfm_phys, ref internal).
 struct TankPhys {
     double rho_w, rho_a, g0, g1, g2, ref_value;
+    double inv_w, inv_a;  // 1 / density as div_known takes it
     int32_t ref;  // internal index of the pinned cell, -1 = none
     int32_t pad;
 };
@@ -139,10 +140,11 @@ struct SolveArgs {
 struct FaceArgs {
     int32_t n, F;
     const int32_t *owner, *neighbour;
-    const double *Sf, *C;
+    const double *c, *C;     // c_f = (S.S)/(S.d); cell centres
     const double *alpha, *phi;
-    double rho_w, rho_a, g0, g1, g2;
-    double *lambda, *gamma, *jump, *sigma;
+    double rho_w, rho_a, g0, g1, g2, inv_w, inv_a;
+    double *lambda, *gamma, *jump, *phi_copy;
+    double2 *gs;             // (gamma, sigma)
     int8_t *kind;
     const int32_t *ftank;    // batched: tank of each face (else nullptr)
     const TankPhys *tphys;   // batched: physics per tank
@@ -152,7 +154,8 @@ cudaError_t launch_faces(const FaceArgs &a, cudaStream_t s);
 
 struct CellArgs {
     Sell m;
-    const double *gamma, *sigma;
+    const double2 *gs;  // (gamma, sigma) per face
+    bool source_only;   // b alone
     int32_t ref;  // internal index of the pinned cell, -1 none
     double ref_value;
     double *b, *diag, *dinv;
@@ -172,12 +175,21 @@ struct CellArgs {
 cudaError_t launch_cells(const CellArgs &a, cudaStream_t s);
 
 // sigma = phi + gamma J for a new predicted flux (coefficients unchanged)
-cudaError_t launch_sigma(int32_t F, const double *phi, const double *gamma, const double *jump, double *sigma,
-                         cudaStream_t s);
+cudaError_t launch_sigma(int32_t F, const double *phi, const double *gamma, const double *jump, double2 *gs,
+                         double *phi_copy, cudaStream_t s);
 
-// c_f = (S.S)/(S.d) of every face, rounded exactly as the face assembly does
+// c_f = (S.S)/(S.d) of every face, and (S.d, its inverse as div_known takes it)
 cudaError_t launch_face_c(int32_t n, int32_t F, const int32_t *owner, const int32_t *neighbour, const double *Sf,
-                          const double *C, double *c, cudaStream_t s);
+                          const double *C, double *c, double2 *sd, cudaStream_t s);
+
+// Faces of each cell in the caller's cell order, ascending: +(f+1) if the cell
+// owns face f, -(f+1) if not, 0 past the last.  Sliced-ELL over slices of 32
+// caller cells: slot k of cell c at ptr[c / 32] + k * 32 + c % 32.
+struct CellFaces {
+    const int32_t *ptr, *face;
+};
+cudaError_t launch_cell_face_width(const Sell &m, const int32_t *perm, int32_t *width, cudaStream_t s);
+cudaError_t launch_cell_faces(const Sell &m, const int32_t *perm, const int32_t *ptr, int32_t *out, cudaStream_t s);
 
 // Dictionary of the compact table: dict[2k] = (float)(c_k / rho_w),
 // dict[2k+1] = (float)(c_k / rho_a) for geometric class k (densities of the
@@ -239,17 +251,19 @@ cudaError_t launch_adjoint_cells(const AdjointArgs &a, cudaStream_t s);
 
 // ---- gradient and velocity reconstruction (gfm_gradient.cu) ----------------
 struct GradArgs {
-    Sell m;
     int32_t n, F;
-    const int32_t *iperm;              // internal -> caller (-1 padding)
+    CellFaces cf;
     const int32_t *owner, *neighbour;  // caller order
+    const double2 *sd;                 // [F] (S.d, 1 / (S.d) as div_known takes it)
     const double *Sf, *C, *V, *xf;     // xf nullable: face centres half-way between cell centres
     const double *lambda, *jump;       // assembled interface fraction and oriented jump
+    const int8_t *kind;                // 0: both cells dry, 1: both wet, else an interface face
     const double *p;                   // caller order p_d
     const double *phi;                 // face flux for U (nullable when U is)
-    double rho_w, rho_a;
-    const int32_t *stank;              // batched: tank of each slice (else nullptr)
+    double rho_w, rho_a, inv_w, inv_a;
+    const int32_t *ftank;              // batched: tank of each face (else nullptr)
     const TankPhys *tphys;             // batched: densities per tank
+    double4 *rec;                      // [2 F] scratch: the faces' records
     double *grad, *U;                  // [3][n] caller order, either nullable
 };
 cudaError_t launch_gradient(const GradArgs &a, cudaStream_t s);
@@ -260,19 +274,21 @@ cudaError_t launch_gradient(const GradArgs &a, cudaStream_t s);
 struct NonorthArgs {
     int32_t n, F;
     const int32_t *owner, *neighbour;
-    const double *Sf, *C, *xf;  // xf nullable
+    const double *Sf, *C, *c;   // c = (S.S)/(S.d)
     const double *rau;          // nullable
     const double *G;
+    const double4 *rec;         // launch_gradient's records of G alone
     const double *phi, *gamma, *jump;
-    double *corr, *phi_eff, *sigma;
+    double *corr, *phi_eff;
+    double2 *gs;  // (gamma, sigma)
 };
 cudaError_t launch_nonorth(const NonorthArgs &a, cudaStream_t s);
 
 // ---- isoAdvector advection step (gfm_iso.cu) ------------------------------
 struct IsoArgs {
-    Sell m;
     int32_t n, F, nvt;
-    const int32_t *iperm, *owner, *neighbour;
+    CellFaces cf;
+    const int32_t *owner, *neighbour;
     const double *alpha, *phi;
     double dt;
     const int32_t *fv_ptr;   // [F+1]

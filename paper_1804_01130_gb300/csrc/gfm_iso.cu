@@ -20,7 +20,7 @@
 // whose upwind cell has no isoface carries that cell's alpha throughout.
 //
 // A thread per face and a lane per triangle (FP64 geometry); then one thread
-// per cell sums its faces' volumes in ascending face order through the sliced-ELL table:
+// per cell sums its faces' volumes in ascending face order:
 //     alpha_P(t + dt) = alpha_P(t) - 1/V_P sum_f s_Pf dV_f.
 #include "gfm_internal.h"
 
@@ -185,19 +185,20 @@ __global__ void __launch_bounds__(256) k_iso_flux(IsoArgs a)
 
 __global__ void __launch_bounds__(256) k_iso_cells(IsoArgs a)
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= a.m.n_pad) return;
-    const int c = a.iperm[t];
-    if (c < 0) return;
-    const int s = t / kSlice, l = t % kSlice;
-    const int base = a.m.slice_ptr[s];
-    const int w = (a.m.slice_ptr[s + 1] - base) / kSlice;
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= a.n) return;
+    const int base = a.cf.ptr[c >> 5], w = (a.cf.ptr[(c >> 5) + 1] - base) >> 5, lane = c & 31;
     double acc = 0.0;
-    for (int k = 0; k < w; ++k) {
-        const int code = a.m.face[base + k * kSlice + l];
-        if (code == 0) continue;
-        const int f = (code > 0 ? code : -code) - 1;
-        acc = (code > 0) ? acc + a.dV[f] : acc - a.dV[f];
+    for (int k0 = 0; k0 < w; k0 += 3) {
+        int code[3];
+        double v[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) code[q] = k0 + q < w ? a.cf.face[base + (k0 + q) * kSlice + lane] : 0;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) v[q] = code[q] != 0 ? a.dV[(code[q] > 0 ? code[q] : -code[q]) - 1] : 0.0;
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (code[q] != 0) acc = code[q] > 0 ? acc + v[q] : acc - v[q];
     }
     a.alpha_new[c] = a.alpha[c] - acc / a.V[c];
 }
@@ -209,7 +210,7 @@ cudaError_t launch_iso(const IsoArgs &a, cudaStream_t s)
     if (a.F > 0) k_iso_flux<<<(a.F + 255) / 256, 256, 0, s>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !a.alpha_new) return e;
-    k_iso_cells<<<(a.m.n_pad + 255) / 256, 256, 0, s>>>(a);
+    k_iso_cells<<<(a.n + 255) / 256, 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -239,7 +239,8 @@ int to_sell(int n, int n_slices, const std::vector<int32_t> &cnt_ptr, std::vecto
 }  // namespace
 
 std::vector<MgLevelHost> build_mg_levels(int n, int n_pad, int F, const int32_t *owner, const int32_t *nb,
-                                         const double *Sf, const double *C, const int32_t *perm)
+                                         const double *Sf, const double *C, const int32_t *perm,
+                                         const int32_t *slot_face, int n_slots)
 {
     std::vector<MgLevelHost> levels;
     // the mesh, its cells numbered in internal order without the padding cells
@@ -340,8 +341,22 @@ std::vector<MgLevelHost> build_mg_levels(int n, int n_pad, int F, const int32_t 
             const double r = s > 0.0 ? strength(cur, f) / s : 0.5;
             L.scale[(size_t)f] = std::min(2.0, std::max(0.05, r));
         }
-        if (levels.empty())  // members in the caller's face numbers
-            for (auto &m : L.mem) m = at[(size_t)m];
+        if (levels.empty()) {  // members in the caller's face numbers, or as slots
+            std::vector<int32_t> slot;
+            if (slot_face) {
+                slot.resize((size_t)F);
+                parallel_ranges(n_slots, [&](int lo, int hi) {
+                    for (int q = lo; q < hi; ++q)
+                        if (slot_face[q] > 0) slot[(size_t)slot_face[q] - 1] = q;
+                });
+            }
+            parallel_ranges((int)L.mem.size(), [&](int lo, int hi) {
+                for (int q = lo; q < hi; ++q) {
+                    const int32_t f = at[(size_t)L.mem[(size_t)q]];
+                    L.mem[(size_t)q] = slot_face ? slot[(size_t)f] : f;
+                }
+            });
+        }
         Adj adj;
         build_adj(cur, adj);
         L.max_width = to_sell(L.n, L.n_slices, adj.ptr, L.slice_ptr, [&](int slot, int i, int e) {

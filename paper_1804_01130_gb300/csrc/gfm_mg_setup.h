@@ -21,12 +21,16 @@ struct MgLevelHost {
     std::vector<int32_t> child;      // finer node, -1 on padding slots
     std::vector<double> scale;       // [F] geometric factor of the face's coefficient
     std::vector<int32_t> mem_ptr;    // [F + 1] finer faces of each face, ascending
-    std::vector<int32_t> mem;        // (caller faces on the first coarse level)
+    std::vector<int32_t> mem;        // (caller faces or slots on the first coarse level)
 };
 
 // Coarse levels of the mesh (caller owner/neighbour, area vectors Sf [3][F]
 // and centres C [3][n], perm = caller -> internal cell; n_pad internal cells).
+// With the mesh table's slot_face [n_slots] (HostTables::face) the first
+// level's members are its faces' slots in their owners' rows, which lie near
+// each other, instead of caller faces.
 std::vector<MgLevelHost> build_mg_levels(int n, int n_pad, int F, const int32_t *owner, const int32_t *nb,
-                                         const double *Sf, const double *C, const int32_t *perm);
+                                         const double *Sf, const double *C, const int32_t *perm,
+                                         const int32_t *slot_face = nullptr, int n_slots = 0);
 
 }  // namespace gfm
