@@ -346,8 +346,8 @@ gfm_status gfm_nonorth_correct(gfm_handle h, const double *p, const double *V, c
  * diagonal).  The call only enqueues work on `stream` and never
  * synchronises.
  *
- * Scratch: the CG vectors, the per-CTA partial sums and the barrier counter
- * live in one fixed array in the library's device code, 8.05 MiB for
+ * Scratch: the exchanged CG vectors, the per-CTA partial sums and the barrier counter
+ * live in one fixed array in the library's device code, 4.07 MiB for
  * n <= GFM_NOALLOC_MAX_CELLS; every GPU that loads the library's device code
  * holds it until the process exits.  n beyond that limit returns
  * GFM_ERR_ARG before anything is enqueued.  The first call on a device looks
