@@ -337,8 +337,7 @@ float prof_elapsed(gfm_ctx *h, int a, int b)
 void clear_stale_error() { (void)cudaGetLastError(); }
 
 // Launch shape of the multigrid solve.  The default tuning (512 x 1) takes
-// the most threads the kernel allows in one CTA per SM (1024 in FP32, 512 in
-// FP64): its passes are bound by gather latency.  Other tunings are taken as
+// what mg_kernel picks (512 or 1024 threads in one CTA per SM).  Other tunings are taken as
 // they are.  A small mesh gets a CTA per 8 slices, since every CTA more makes
 // the grid barriers dearer.
 struct MgPlan {
@@ -352,7 +351,7 @@ gfm_status plan_mg(gfm_ctx *h, gfm::Mode mode, MgPlan *mp)
 {
     const bool mixed = mode == gfm::Mode::MIXED;
     int most = 0;
-    mp->kernel = gfm::mg_kernel(mixed, h->ht.max_width, &most);
+    mp->kernel = gfm::mg_kernel(mixed, h->ht.max_width, h->ht.n_slices / h->sm_count, &most);
     const bool standard = h->tuning.threads == 512 && h->tuning.ctas_per_sm == 1;
     const int t = standard ? most : std::min(h->tuning.threads, most);
     int per = h->tuning.ctas_per_sm, occ = 0;

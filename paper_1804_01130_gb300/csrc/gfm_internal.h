@@ -355,7 +355,7 @@ struct MgArgs {
     void *z, *p, *sv, *e;     // z = M^{-1} r, direction, A p, FP32 correction
     MgLevel lv[kMgLevels];
 };
-const void *mg_kernel(bool mixed, int max_width, int *max_threads);
+const void *mg_kernel(bool mixed, int max_width, int slices_per_sm, int *max_threads);
 
 struct MgLevelArgs {
     int32_t n_slices;

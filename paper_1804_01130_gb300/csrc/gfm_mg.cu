@@ -36,7 +36,8 @@
 // across tank borders; a CTA writes one partial sum per (CTA, tank) segment,
 // to slot CTA + tank, and every CTA adds each tank's segments in the same
 // order, so all CTAs take identical decisions and results are
-// bit-reproducible.
+// bit-reproducible.  A tank that has converged, or waits for the others to ask
+// for a replacement, gives its share of the CTAs to those still iterating.
 #include "gfm_grid.cuh"
 
 namespace gfm {
@@ -61,9 +62,9 @@ struct MgShared {
     int act[kMaxTanks], flag[kMaxTanks], wait[kMaxTanks], fresh[kMaxTanks];
     int iters[kMaxTanks], updates[kMaxTanks], stall[kMaxTanks], last_rep[kMaxTanks], restarts[kMaxTanks];
     int c0[kMaxTanks], c1[kMaxTanks];  // first and last CTA holding slices of the tank
-    int seg_s0[kMaxTanks + 1], seg_tank[kMaxTanks];
+    int seg_s0[kMaxTanks], seg_s1[kMaxTanks], seg_tank[kMaxTanks];  // this CTA's segments
     int wide[kMaxTanks];
-    int nseg, n_wide, any_active, any_flag, fail;
+    int nseg, n_wide, any_active, any_flag, replan, fail;
 };
 
 // ---- sums ------------------------------------------------------------------
@@ -103,11 +104,13 @@ struct Ctx {
 };
 
 // Plain grid barrier (an error raised elsewhere is seen at the next wait).
+// Thread 0's acquire and the CTA barrier order the other CTAs' writes before
+// every thread's reads; a V-cycle passes some twenty of these.
 __device__ __forceinline__ bool mg_sync(Ctx &c)
 {
     __syncthreads();
     c.g.epoch += 1u;
-    if (threadIdx.x == 0) c.sh->fail = grid_arrive_wait(c.g) ? 0 : 1;
+    if (threadIdx.x == 0) c.sh->fail = grid_arrive_wait<false>(c.g) ? 0 : 1;
     __syncthreads();
     return c.sh->fail == 0;
 }
@@ -700,6 +703,13 @@ __device__ void tail_cycle(const MgArgs &a, const Ctx &c, unsigned char *dsm)
     for (--t; t >= 0; --t) tail_level<T, true>(a, dsm, t, t + 1 == nt, warps(t));
 }
 
+// A row pass on a coarse level (two slices in flight per warp measured the same).
+template <typename T, int CH, typename Op>
+__device__ __forceinline__ void coarse_pass(const MgLevel &lv, const T *X, int s0, int s1, const Ctx &c, Op &op)
+{
+    row_pass<T, CH, 1, false>(lv, X, s0, s1, c.warp, c.nw, c.lane, lv.n, op);
+}
+
 // Levels 1 .. L-1 of the V-cycle, from the mesh's residual (lv[0].res) to the
 // correction added to lv[0].xb.  Ends with a grid barrier.
 template <typename T, int CH>
@@ -715,11 +725,11 @@ __device__ __forceinline__ bool coarse_cycle(const MgArgs &a, Ctx &c, unsigned c
         restrict_pass<T>(lv, static_cast<const T *>(a.lv[l - 1].res), om1, s0, s1, c.warp, c.nw, c.lane);
         if (!mg_sync(c)) return false;
         SweepOp<T, false> sw{static_cast<const T *>(lv.b), static_cast<const T *>(lv.dinv), static_cast<T *>(lv.xb), om2, pin};
-        row_pass<T, CH, 1, false>(lv, static_cast<const T *>(lv.xa), s0, s1, c.warp, c.nw, c.lane, lv.n, sw);
+        coarse_pass<T, CH>(lv, static_cast<const T *>(lv.xa), s0, s1, c, sw);
         if (!mg_sync(c)) return false;
         if (l + 1 < L) {
             ResidOp<T, false> rs{static_cast<const T *>(lv.b), static_cast<T *>(lv.res), pin};
-            row_pass<T, CH, 1, false>(lv, static_cast<const T *>(lv.xb), s0, s1, c.warp, c.nw, c.lane, lv.n, rs);
+            coarse_pass<T, CH>(lv, static_cast<const T *>(lv.xb), s0, s1, c, rs);
             if (!mg_sync(c)) return false;
         }
     }
@@ -732,10 +742,10 @@ __device__ __forceinline__ bool coarse_cycle(const MgArgs &a, Ctx &c, unsigned c
         const Pin<T, false> pin{static_cast<const T *>(lv.pin), -1, T(0)};
         split(lv.n_slices, c.g.G, blockIdx.x, s0, s1);
         SweepOp<T, false> sw{static_cast<const T *>(lv.b), static_cast<const T *>(lv.dinv), static_cast<T *>(lv.xa), om2, pin};
-        row_pass<T, CH, 1, false>(lv, static_cast<const T *>(lv.xb), s0, s1, c.warp, c.nw, c.lane, lv.n, sw);
+        coarse_pass<T, CH>(lv, static_cast<const T *>(lv.xb), s0, s1, c, sw);
         if (!mg_sync(c)) return false;
         LastCoarseOp<T> lc{lv, static_cast<T *>(a.lv[l - 1].xb), om1, pin};
-        row_pass<T, CH, 1, false>(lv, static_cast<const T *>(lv.xa), s0, s1, c.warp, c.nw, c.lane, lv.n, lc);
+        coarse_pass<T, CH>(lv, static_cast<const T *>(lv.xa), s0, s1, c, lc);
         if (!mg_sync(c)) return false;
     }
     return true;
@@ -779,12 +789,11 @@ __device__ void mg_abort(const MgArgs &a)
 
 }  // namespace
 
-template <typename T, int CH, int NT>
+template <typename T, int CH, int NT, int U>
 __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
 {
     constexpr bool kMixed = sizeof(T) == 4;
-    constexpr int U = kMixed ? 2 : 1;  // slices in flight per warp in the row passes
-    constexpr int UB = kMixed ? 4 : 2;  // the same in the update pass
+    constexpr int UB = kMixed ? 4 : 2;  // slices in flight per warp in the update pass (U: in the row passes)
     using A = typename AccOf<T>::type;
     __shared__ MgShared sh;
     extern __shared__ __align__(16) unsigned char dsm[];
@@ -798,32 +807,63 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
     c.P = (int)gridDim.x + a.T;
     const int T_ = a.T, lane = c.lane, warp = c.warp, nw = c.nw;
     const T om1 = T(kOm1), om2 = T(kOm2);
-    int s_lo, s_hi;
-    split(a.s.m.n_slices, c.g.G, blockIdx.x, s_lo, s_hi);
-    // this CTA's segments and every tank's CTAs
-    for (int t = threadIdx.x; t < T_; t += blockDim.x) {
-        const long long G = c.g.G, ns = a.s.m.n_slices;
-        const int f = T_ > 1 ? a.tank_off[t] >> 5 : 0, e = T_ > 1 ? a.tank_off[t + 1] >> 5 : (int)ns;
-        sh.c0[t] = (int)(((f + 1) * G - 1) / ns);
-        sh.c1[t] = (int)((e * G - 1) / ns);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int m = 0, nwd = 0;
-        for (int t = 0; t < T_; ++t) {
-            const int f = T_ > 1 ? a.tank_off[t] >> 5 : 0, e = T_ > 1 ? a.tank_off[t + 1] >> 5 : a.s.m.n_slices;
-            if (f < s_hi && e > s_lo) {
-                sh.seg_s0[m] = max(f, s_lo);
-                sh.seg_tank[m++] = t;
+    auto working = [&](int t) { return sh.act[t] == kMgGo && sh.wait[t] == 0; };
+    // Share the slices of the tanks for which want(t) holds among the CTAs:
+    // equal contiguous stretches across tank borders.  A pure function of the
+    // tanks' state, so every CTA builds the same table.
+    auto plan = [&](auto want) {
+        __syncthreads();
+        if (threadIdx.x < 32) {  // lane l takes tanks l, l + 32, ...
+            auto first = [&](int t) { return T_ > 1 ? a.tank_off[t] >> 5 : 0; };
+            auto count = [&](int t) { return (T_ > 1 ? a.tank_off[t + 1] >> 5 : a.s.m.n_slices) - first(t); };
+            int ns = 0;
+            for (int t = lane; t < T_; t += 32) ns += want(t) ? count(t) : 0;
+#pragma unroll
+            for (int o = 16; o; o >>= 1) ns += __shfl_xor_sync(0xffffffffu, ns, o);
+            const long long G = min(c.g.G, ns), b = blockIdx.x, N = max(ns, 1);
+            const int lo = b < G ? (int)(N * b / G) : ns, hi = b < G ? (int)(N * (b + 1) / G) : ns;
+            int off0 = 0, m = 0, nwd = 0;
+            for (int t0 = 0; t0 < T_; t0 += 32) {
+                const int t = t0 + lane;
+                const int n = t < T_ && want(t) ? count(t) : 0;
+                int inc = n;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, inc, o);
+                    if (lane >= o) inc += y;
+                }
+                const int off = off0 + inc - n;
+                int c0 = 0, c1 = -1;
+                if (n > 0) {
+                    c0 = (int)(((off + 1) * G - 1) / N);
+                    c1 = (int)(((off + n) * G - 1) / N);
+                }
+                if (t < T_) {
+                    sh.c0[t] = c0;
+                    sh.c1[t] = c1;
+                }
+                const unsigned below = (1u << lane) - 1u;
+                const bool wide = c1 - c0 + 1 > kSegLane, here = n > 0 && off < hi && off + n > lo;
+                const unsigned wm = __ballot_sync(0xffffffffu, wide), hm = __ballot_sync(0xffffffffu, here);
+                if (wide) sh.wide[nwd + __popc(wm & below)] = t;
+                if (here) {
+                    const int q = m + __popc(hm & below);
+                    sh.seg_s0[q] = first(t) + max(off, lo) - off;
+                    sh.seg_s1[q] = first(t) + min(off + n, hi) - off;
+                    sh.seg_tank[q] = t;
+                }
+                m += __popc(hm);
+                nwd += __popc(wm);
+                off0 += __shfl_sync(0xffffffffu, inc, 31);
             }
-            if (sh.c1[t] - sh.c0[t] + 1 > kSegLane) sh.wide[nwd++] = t;
+            if (lane == 0) {
+                sh.nseg = m;
+                sh.n_wide = nwd;
+            }
         }
-        sh.seg_s0[m] = s_hi;
-        sh.nseg = m;
-        sh.n_wide = nwd;
-    }
-    __syncthreads();
-    const int nseg = sh.nseg;
+        __syncthreads();
+    };
+    plan([](int) { return true; });
     if (blockIdx.x == 0 && a.tail < a.L) tail_stage<T>(a, dsm);
     auto bail = [&]() { mg_abort(a); };
 
@@ -840,10 +880,10 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
     };
 
     // prologue: x0, ||b||
-    for (int q = 0; q < nseg; ++q) {
+    for (int q = 0; q < sh.nseg; ++q) {
         const int t = sh.seg_tank[q], end = tank_end(t);
         double vb[1] = {0.0};
-        for (int s = sh.seg_s0[q] + warp; s < sh.seg_s0[q + 1]; s += nw) {
+        for (int s = sh.seg_s0[q] + warp; s < sh.seg_s1[q]; s += nw) {
             const int i = s * kSlice + lane;
             if (i < end) {
                 a.s.x64[i] = a.s.use_x0 ? a.s.p_user[a.s.iperm[i]] : 0.0;
@@ -880,25 +920,26 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
     // r = b - A x (FP64) for the flagged tanks, x += e first (mixed); also
     // the V-cycle's first sweep from zero.  Then the tanks' decisions.
     auto replace = [&](bool first) -> bool {
+        if (T_ > 1 && !first) plan([&](int t) { return sh.flag[t] != kFlagNone; });
         if (kMixed && !first) {
-            for (int q = 0; q < nseg; ++q) {
+            for (int q = 0; q < sh.nseg; ++q) {
                 const int t = sh.seg_tank[q], end = tank_end(t);
                 if (sh.flag[t] == kFlagNone) continue;
                 const double isc = sh.isc[t];
-                for (int sb = sh.seg_s0[q] + warp; sb < sh.seg_s0[q + 1]; sb += 4 * nw) {
+                for (int sb = sh.seg_s0[q] + warp; sb < sh.seg_s1[q]; sb += 4 * nw) {
                     T e[4];
                     double x[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const int i = (sb + u * nw) * kSlice + lane;
-                        const bool ok = sb + u * nw < sh.seg_s0[q + 1] && i < end;
+                        const bool ok = sb + u * nw < sh.seg_s1[q] && i < end;
                         e[u] = ok ? E[i] : T(0);
                         x[u] = ok ? a.s.x64[i] : 0.0;
                     }
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const int i = (sb + u * nw) * kSlice + lane;
-                        if (sb + u * nw < sh.seg_s0[q + 1] && i < end) {
+                        if (sb + u * nw < sh.seg_s1[q] && i < end) {
                             a.s.x64[i] = fma((double)e[u], isc, x[u]);
                             E[i] = T(0);
                         }
@@ -907,7 +948,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
             }
             if (!mg_sync(c)) return false;
         }
-        for (int q = 0; q < nseg; ++q) {
+        for (int q = 0; q < sh.nseg; ++q) {
             const int t = sh.seg_tank[q], end = tank_end(t);
             A v[1] = {A{}};
             if (sh.flag[t] != kFlagNone) {
@@ -916,7 +957,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                 const int ref = pp->ref;
                 const double pin = pp->pin64;
                 const bool with_x = !first || a.s.use_x0;
-                for (int s = sh.seg_s0[q] + warp; s < sh.seg_s0[q + 1]; s += nw) {
+                for (int s = sh.seg_s0[q] + warp; s < sh.seg_s1[q]; s += nw) {
                     const int i = s * kSlice + lane;
                     if (i < end) {
                         const double bi = a.s.b[i];
@@ -974,17 +1015,17 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
             if (threadIdx.x == 0) sh.any_active = active;
         }
         __syncthreads();
+        if (T_ > 1) plan(working);
         return true;
     };
     if (!replace(true)) { bail(); return; }
 
-    auto working = [&](int t) { return sh.act[t] == kMgGo && sh.wait[t] == 0; };
     auto fine_sweep = [&](const T *X, T *out, T w) {
-        for (int q = 0; q < nseg; ++q) {
+        for (int q = 0; q < sh.nseg; ++q) {
             const int t = sh.seg_tank[q];
             if (!working(t)) continue;
             SweepOp<T, true> op{R, dinv, out, w, tank_pin(t)};
-            row_pass<T, CH, U, true>(l0, X, sh.seg_s0[q], sh.seg_s0[q + 1], warp, nw, lane, tank_end(t), op);
+            row_pass<T, CH, U, true>(l0, X, sh.seg_s0[q], sh.seg_s1[q], warp, nw, lane, tank_end(t), op);
         }
     };
     while (sh.any_active) {
@@ -992,23 +1033,23 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
         fine_sweep(XA, XB, om2);
         if (!mg_sync(c)) { bail(); return; }
         if (a.L > 1) {
-            for (int q = 0; q < nseg; ++q) {
+            for (int q = 0; q < sh.nseg; ++q) {
                 const int t = sh.seg_tank[q];
                 if (!working(t)) continue;
                 ResidOp<T, true> op{R, RES, tank_pin(t)};
-                row_pass<T, CH, U, true>(l0, XB, sh.seg_s0[q], sh.seg_s0[q + 1], warp, nw, lane, tank_end(t), op);
+                row_pass<T, CH, U, true>(l0, XB, sh.seg_s0[q], sh.seg_s1[q], warp, nw, lane, tank_end(t), op);
             }
             if (!mg_sync(c)) { bail(); return; }
             if (!coarse_cycle<T, CH>(a, c, dsm)) { bail(); return; }
         }
         fine_sweep(XB, XA, om2);
         if (!mg_sync(c)) { bail(); return; }
-        for (int q = 0; q < nseg; ++q) {
+        for (int q = 0; q < sh.nseg; ++q) {
             const int t = sh.seg_tank[q];
             A v[1] = {A{}};
             if (working(t)) {
                 LastOp<T> op{R, dinv, Z, om1, tank_pin(t), A{}};
-                row_pass<T, CH, U, true>(l0, XA, sh.seg_s0[q], sh.seg_s0[q + 1], warp, nw, lane, tank_end(t), op);
+                row_pass<T, CH, U, true>(l0, XA, sh.seg_s0[q], sh.seg_s1[q], warp, nw, lane, tank_end(t), op);
                 v[0] = op.sum;
             }
             put_partials<1, A>(c, t, v);
@@ -1027,7 +1068,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
         }
         __syncthreads();
         // p = z + beta p, s = A p, p.s
-        for (int q = 0; q < nseg; ++q) {
+        for (int q = 0; q < sh.nseg; ++q) {
             const int t = sh.seg_tank[q];
             A v[1] = {A{}};
             if (working(t) && sh.flag[t] == kFlagNone) {
@@ -1035,7 +1076,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                 if constexpr (kMixed) be = sh.be32[t];
                 else be = sh.be64[t];
                 DirOp<T> op{P, S, be, sh.fresh[t] != 0, tank_pin(t), A{}};
-                row_pass<T, CH, U, true>(l0, Z, sh.seg_s0[q], sh.seg_s0[q + 1], warp, nw, lane, tank_end(t), op);
+                row_pass<T, CH, U, true>(l0, Z, sh.seg_s0[q], sh.seg_s1[q], warp, nw, lane, tank_end(t), op);
                 v[0] = op.sum;
             }
             put_partials<1, A>(c, t, v);
@@ -1052,8 +1093,8 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
         }
         __syncthreads();
         // e += alpha p (FP64: x), r -= alpha s, the next V-cycle's first sweep, r.r
-        for (int q = 0; q < nseg; ++q) {
-            const int t = sh.seg_tank[q], end = tank_end(t), e1 = sh.seg_s0[q + 1];
+        for (int q = 0; q < sh.nseg; ++q) {
+            const int t = sh.seg_tank[q], end = tank_end(t), e1 = sh.seg_s1[q];
             A v[1] = {A{}};
             if (working(t) && sh.flag[t] == kFlagNone) {
                 T al;
@@ -1096,7 +1137,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
         // convergence idles until the round, which comes when no tank is left
         // iterating or some tank must not wait.
         if (threadIdx.x < 32) {
-            bool now = false, asked = false, going = false;
+            bool now = false, asked = false, going = false, waits = false;
             for (int t = threadIdx.x; t < T_; t += 32) {
                 if (sh.act[t] != kMgGo) continue;
                 if (sh.wait[t]) {
@@ -1116,11 +1157,11 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                 } else if (!(rho > 0.81 * sh.rho_stop[t])) {
                     sh.flag[t] = kFlagUpdate;
                     sh.wait[t] = 1;
-                    asked = true;
+                    asked = waits = true;
                 } else if (kMixed && (rho <= 1e-6 * sh.rho_max[t] || it - sh.last_rep[t] >= 40)) {
                     sh.flag[t] = kFlagUpdate;
                     sh.wait[t] = 1;
-                    asked = true;
+                    asked = waits = true;
                 } else {
                     going = true;
                 }
@@ -1128,22 +1169,31 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
             now = __any_sync(0xffffffffu, now);
             asked = __any_sync(0xffffffffu, asked);
             going = __any_sync(0xffffffffu, going);
-            if (threadIdx.x == 0) sh.any_flag = now || (asked && !going);
+            waits = __any_sync(0xffffffffu, waits);
+            if (threadIdx.x == 0) {
+                sh.any_flag = now || (asked && !going);
+                sh.replan = waits;
+            }
         }
         __syncthreads();
-        if (sh.any_flag && !replace(false)) { bail(); return; }
+        if (sh.any_flag) {
+            if (!replace(false)) { bail(); return; }
+        } else if (T_ > 1 && sh.replan) {
+            plan(working);
+        }
     }
 
     // the record: true FP64 residual (r in r64), solution in caller order,
     // normalised L1 residual sum|r| / (sum|A x - x_avg rowsum| + sum|b - x_avg rowsum|)
+    if (T_ > 1) plan([](int) { return true; });
     if (!mg_sync(c)) { bail(); return; }
-    for (int q = 0; q < nseg; ++q) {
+    for (int q = 0; q < sh.nseg; ++q) {
         const int t = sh.seg_tank[q], end = tank_end(t);
         const DevParams *pp = T_ > 1 ? a.tprm + t : a.s.prm;
         const int ref = pp->ref;
         const double pin = pp->pin64;
         double v[2] = {0.0, 0.0};
-        for (int s = sh.seg_s0[q] + warp; s < sh.seg_s0[q + 1]; s += nw) {
+        for (int s = sh.seg_s0[q] + warp; s < sh.seg_s1[q]; s += nw) {
             const int i = s * kSlice + lane;
             if (i < end) {
                 const double xi = a.s.x64[i];
@@ -1162,13 +1212,13 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
         sh.rho[t] = sh.tot[0][t];
     }
     __syncthreads();
-    for (int q = 0; q < nseg; ++q) {
+    for (int q = 0; q < sh.nseg; ++q) {
         const int t = sh.seg_tank[q], end = tank_end(t);
         const DevParams *pp = T_ > 1 ? a.tprm + t : a.s.prm;
         const int ref = pp->ref;
         const double pin = pp->pin64, xavg = sh.xavg[t];
         double v[2] = {0.0, 0.0};
-        for (int s = sh.seg_s0[q] + warp; s < sh.seg_s0[q + 1]; s += nw) {
+        for (int s = sh.seg_s0[q] + warp; s < sh.seg_s1[q]; s += nw) {
             const int i = s * kSlice + lane;
             if (i < end) {
                 const double r = a.s.r64[i], bi = a.s.b[i], rs = i == ref ? pin : 0.0;
@@ -1246,13 +1296,20 @@ cudaError_t launch_mg_level(const MgLevelArgs &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// Instantiations by faces per row chunk and by precision; *threads in: the
-// wanted threads per CTA, out: at most what the instantiation allows.
-const void *mg_kernel(bool mixed, int max_width, int *max_threads)
+// Instantiations by precision, faces per row chunk and threads per CTA
+// (*max_threads).  FP32: 1024 threads a CTA hide the gathers' latency where an
+// SM has many rows; with few, what counts is the latency of some twenty grid
+// barriers and of the tail's passes, which 512 threads pass faster.  601x203
+// cells (25 slices an SM): 2.57 ms with 1024, 2.15 with 512; 1024x512 (108): 123
+// and 127 us a V-cycle; 256x128x128 (862): 11.8 and 13.8 ms.
+const void *mg_kernel(bool mixed, int max_width, int slices_per_sm, int *max_threads)
 {
-    *max_threads = mixed ? 1024 : 512;
-    if (mixed) return max_width <= 4 ? (const void *)k_solve_mg<float, 4, 1024> : (const void *)k_solve_mg<float, 6, 1024>;
-    return max_width <= 4 ? (const void *)k_solve_mg<double, 4, 512> : (const void *)k_solve_mg<double, 6, 512>;
+    const bool w4 = max_width <= 4;
+    const bool wide = mixed && slices_per_sm > 64;
+    *max_threads = wide ? 1024 : 512;
+    if (wide) return w4 ? (const void *)k_solve_mg<float, 4, 1024, 1> : (const void *)k_solve_mg<float, 6, 1024, 1>;
+    if (mixed) return w4 ? (const void *)k_solve_mg<float, 4, 512, 1> : (const void *)k_solve_mg<float, 6, 512, 1>;
+    return w4 ? (const void *)k_solve_mg<double, 4, 512, 1> : (const void *)k_solve_mg<double, 6, 512, 1>;
 }
 
 }  // namespace gfm
