@@ -343,6 +343,7 @@ void clear_stale_error() { (void)cudaGetLastError(); }
 struct MgPlan {
     const void *kernel = nullptr;
     int grid = 0, threads = 0, tail = 0;
+    int cache_slots = 0, cache_slices = 0, cache_val = 0;
     size_t dyn = 0;
     gfm::MgTail tl[gfm::kMgTailMax] = {};
 };
@@ -404,10 +405,29 @@ gfm_status plan_mg(gfm_ctx *h, gfm::Mode mode, MgPlan *mp)
         off = (off + 15) & ~15;
     }
     mp->dyn = (size_t)off;
-    GFM_CUDA(h, cudaFuncSetAttribute(mp->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, off));
+    mp->grid = std::max(1, std::min(h->sm_count * per, (h->ht.n_slices + 7) / 8));
+    // The mesh's table in shared memory, where the largest share fits beside
+    // nothing else (CTA 0 then holds the tail and no share).
+    const int skip = mp->tail < L ? 1 : 0, parts = mp->grid - skip;
+    if (!h->batched && parts >= 1) {
+        const long long ns = h->ht.n_slices;
+        int slots = 0, slices = 0;
+        for (long long b = 0; b < parts; ++b) {
+            const int s0 = (int)(ns * b / parts), s1 = (int)(ns * (b + 1) / parts);
+            slots = std::max(slots, h->ht.slice_ptr[(size_t)s1] - h->ht.slice_ptr[(size_t)s0]);
+            slices = std::max(slices, s1 - s0);
+        }
+        const long long val = (4LL * (slices + 1 + (long long)slots) + 15) & ~15LL;
+        if (slots > 0 && val + (long long)ts * slots <= budget) {
+            mp->cache_slots = slots;
+            mp->cache_slices = slices;
+            mp->cache_val = (int)val;
+            mp->dyn = std::max(mp->dyn, (size_t)(val + (long long)ts * slots));
+        }
+    }
+    GFM_CUDA(h, cudaFuncSetAttribute(mp->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mp->dyn));
     GFM_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, mp->kernel, t, mp->dyn));
     if (occ < per) return fail(h, GFM_ERR_ARG, "launch shape cannot be co-resident with its shared memory");
-    mp->grid = std::max(1, std::min(h->sm_count * per, (h->ht.n_slices + 7) / 8));
     mp->threads = t;
     return GFM_OK;
 }
@@ -493,6 +513,9 @@ gfm_status enqueue_solve(gfm_ctx *h, const gfm_solve_opts *o, const double *rhs,
         m.s = a;
         m.L = (int)h->mg.size() + 1;
         m.tail = mp.tail;
+        m.cache_slots = mp.cache_slots;
+        m.cache_slices = mp.cache_slices;
+        m.cache_val = mp.cache_val;
         std::copy(std::begin(mp.tl), std::end(mp.tl), std::begin(m.tl));
         m.T = h->batched ? h->T : 1;
         m.tank_off = h->tioff;

@@ -350,6 +350,8 @@ struct MgArgs {
     int32_t tail;    // levels from this one on run in CTA 0 alone, in shared memory
     MgTail tl[kMgTailMax];  // [L - tail]
     int32_t T;       // tanks (1: a single mesh)
+    int32_t cache_slots, cache_slices, cache_val;  // > 0: the mesh's table in shared memory (slots and slices
+                                                   // of the largest share, byte offset of the coefficients)
     const int32_t *tank_off;  // batched: [T+1] internal cell offsets
     const DevParams *tprm;    // batched: pin of each tank
     void *z, *p, *sv, *e;     // z = M^{-1} r, direction, A p, FP32 correction

@@ -213,13 +213,23 @@ __device__ __forceinline__ T row_sweep(T acc, T x, T b, T w, T d, T p)
     else return fma(w * d, b - fma(p, x, acc), x);
 }
 
+// This CTA's share of the mesh's table in shared memory (col == nullptr: not
+// held): slice pointers and slots from slice s0, slot base on.
+template <typename T>
+struct RowCache {
+    const int32_t *sp, *col;
+    const T *val;
+    int s0, base;
+};
+
 // Rows of slices s0 + w0, + nw, ... below s1 (U of them in flight per warp,
 // chunks of CH faces), then op.post(i, x_i, acc_i, pre) with pre = op.pre(i)
 // loaded before the gathers.
 template <typename T, int CH, int U, bool FINE, typename Op>
-__device__ __forceinline__ void row_pass(const MgLevel &lv, const T *X, int s0, int s1, int w0, int nw, int lane, int n,
-                                         Op &op)
+__device__ __forceinline__ void row_pass(const MgLevel &lv, const RowCache<T> &rc, const T *X, int s0, int s1, int w0,
+                                         int nw, int lane, int n, Op &op)
 {
+    const bool held = FINE && rc.col != nullptr;
     const T *__restrict__ val = static_cast<const T *>(lv.val);
     const int32_t *__restrict__ col = lv.col;
     for (int sb = s0 + w0; sb < s1; sb += U * nw) {
@@ -235,8 +245,13 @@ __device__ __forceinline__ void row_pass(const MgLevel &lv, const T *X, int s0, 
             xi[u] = T(0);
             acc[u] = T(0);
             if (s < s1 && i < n) {
-                base[u] = __ldg(lv.sp + s);
-                w[u] = (__ldg(lv.sp + s + 1) - base[u]) >> 5;
+                if (held) {
+                    base[u] = rc.sp[s - rc.s0];
+                    w[u] = (rc.sp[s - rc.s0 + 1] - base[u]) >> 5;
+                } else {
+                    base[u] = __ldg(lv.sp + s);
+                    w[u] = (__ldg(lv.sp + s + 1) - base[u]) >> 5;
+                }
                 xi[u] = X[i];
                 pr[u] = op.pre(i);
             }
@@ -251,7 +266,10 @@ __device__ __forceinline__ void row_pass(const MgLevel &lv, const T *X, int s0, 
                 for (int q = 0; q < CH; ++q) {
                     const bool ok = k0 + q < w[u];
                     const int slot = base[u] + (k0 + q) * kSlice + lane;
-                    if constexpr (FINE) {  // read once per pass
+                    if (FINE && held) {
+                        j[u][q] = ok ? rc.col[slot - rc.base] : 0;
+                        gm[u][q] = ok ? rc.val[slot - rc.base] : T(0);
+                    } else if constexpr (FINE) {  // read once per pass
                         j[u][q] = ok ? __ldcs(col + slot) : 0;
                         gm[u][q] = ok ? __ldcs(val + slot) : T(0);
                     } else {
@@ -707,7 +725,7 @@ __device__ void tail_cycle(const MgArgs &a, const Ctx &c, unsigned char *dsm)
 template <typename T, int CH, typename Op>
 __device__ __forceinline__ void coarse_pass(const MgLevel &lv, const T *X, int s0, int s1, const Ctx &c, Op &op)
 {
-    row_pass<T, CH, 1, false>(lv, X, s0, s1, c.warp, c.nw, c.lane, lv.n, op);
+    row_pass<T, CH, 1, false>(lv, RowCache<T>{}, X, s0, s1, c.warp, c.nw, c.lane, lv.n, op);
 }
 
 // Levels 1 .. L-1 of the V-cycle, from the mesh's residual (lv[0].res) to the
@@ -820,8 +838,11 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
             for (int t = lane; t < T_; t += 32) ns += want(t) ? count(t) : 0;
 #pragma unroll
             for (int o = 16; o; o >>= 1) ns += __shfl_xor_sync(0xffffffffu, ns, o);
-            const long long G = min(c.g.G, ns), b = blockIdx.x, N = max(ns, 1);
-            const int lo = b < G ? (int)(N * b / G) : ns, hi = b < G ? (int)(N * (b + 1) / G) : ns;
+            // with the mesh's table held in shared memory, CTA 0 has the tail's there
+            const int skip = a.cache_slots > 0 && a.tail < a.L ? 1 : 0;
+            const long long G = min(c.g.G - skip, ns), b = (long long)blockIdx.x - skip, N = max(ns, 1);
+            const bool on = b >= 0 && b < G;
+            const int lo = on ? (int)(N * b / G) : ns, hi = on ? (int)(N * (b + 1) / G) : ns;
             int off0 = 0, m = 0, nwd = 0;
             for (int t0 = 0; t0 < T_; t0 += 32) {
                 const int t = t0 + lane;
@@ -835,8 +856,8 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                 const int off = off0 + inc - n;
                 int c0 = 0, c1 = -1;
                 if (n > 0) {
-                    c0 = (int)(((off + 1) * G - 1) / N);
-                    c1 = (int)(((off + n) * G - 1) / N);
+                    c0 = (int)(((off + 1) * G - 1) / N) + skip;
+                    c1 = (int)(((off + n) * G - 1) / N) + skip;
                 }
                 if (t < T_) {
                     sh.c0[t] = c0;
@@ -865,6 +886,24 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
     };
     plan([](int) { return true; });
     if (blockIdx.x == 0 && a.tail < a.L) tail_stage<T>(a, dsm);
+    // Hold this CTA's share of the mesh's table in shared memory where every
+    // CTA's fits (a single mesh, whose shares stay the same): the passes then
+    // wait for one L2 round trip per row, the gathers', instead of three.
+    // 1024x512 cells in FP32, us a pass: 9.4 -> 6.6.
+    RowCache<T> rc{};
+    if (a.cache_slots > 0 && sh.nseg > 0) {
+        const int s0 = sh.seg_s0[0], ns = sh.seg_s1[0] - s0, base = a.s.m.slice_ptr[s0];
+        int32_t *sp = reinterpret_cast<int32_t *>(dsm), *col = sp + a.cache_slices + 1;
+        T *val = reinterpret_cast<T *>(dsm + a.cache_val);
+        for (int k = threadIdx.x; k <= ns; k += blockDim.x) sp[k] = a.s.m.slice_ptr[s0 + k];
+        const int total = a.s.m.slice_ptr[s0 + ns] - base;
+        for (int k = threadIdx.x; k < total; k += blockDim.x) {
+            col[k] = a.s.m.col[base + k];
+            val[k] = static_cast<const T *>(a.lv[0].val)[base + k];
+        }
+        rc = RowCache<T>{sp, col, val, s0, base};
+        __syncthreads();
+    }
     auto bail = [&]() { mg_abort(a); };
 
     const MgLevel &l0 = a.lv[0];
@@ -1025,7 +1064,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
             const int t = sh.seg_tank[q];
             if (!working(t)) continue;
             SweepOp<T, true> op{R, dinv, out, w, tank_pin(t)};
-            row_pass<T, CH, U, true>(l0, X, sh.seg_s0[q], sh.seg_s1[q], warp, nw, lane, tank_end(t), op);
+            row_pass<T, CH, U, true>(l0, rc, X, sh.seg_s0[q], sh.seg_s1[q], warp, nw, lane, tank_end(t), op);
         }
     };
     while (sh.any_active) {
@@ -1037,7 +1076,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                 const int t = sh.seg_tank[q];
                 if (!working(t)) continue;
                 ResidOp<T, true> op{R, RES, tank_pin(t)};
-                row_pass<T, CH, U, true>(l0, XB, sh.seg_s0[q], sh.seg_s1[q], warp, nw, lane, tank_end(t), op);
+                row_pass<T, CH, U, true>(l0, rc, XB, sh.seg_s0[q], sh.seg_s1[q], warp, nw, lane, tank_end(t), op);
             }
             if (!mg_sync(c)) { bail(); return; }
             if (!coarse_cycle<T, CH>(a, c, dsm)) { bail(); return; }
@@ -1049,7 +1088,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
             A v[1] = {A{}};
             if (working(t)) {
                 LastOp<T> op{R, dinv, Z, om1, tank_pin(t), A{}};
-                row_pass<T, CH, U, true>(l0, XA, sh.seg_s0[q], sh.seg_s1[q], warp, nw, lane, tank_end(t), op);
+                row_pass<T, CH, U, true>(l0, rc, XA, sh.seg_s0[q], sh.seg_s1[q], warp, nw, lane, tank_end(t), op);
                 v[0] = op.sum;
             }
             put_partials<1, A>(c, t, v);
@@ -1076,7 +1115,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                 if constexpr (kMixed) be = sh.be32[t];
                 else be = sh.be64[t];
                 DirOp<T> op{P, S, be, sh.fresh[t] != 0, tank_pin(t), A{}};
-                row_pass<T, CH, U, true>(l0, Z, sh.seg_s0[q], sh.seg_s1[q], warp, nw, lane, tank_end(t), op);
+                row_pass<T, CH, U, true>(l0, rc, Z, sh.seg_s0[q], sh.seg_s1[q], warp, nw, lane, tank_end(t), op);
                 v[0] = op.sum;
             }
             put_partials<1, A>(c, t, v);
