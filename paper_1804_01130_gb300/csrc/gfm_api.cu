@@ -508,6 +508,11 @@ gfm_status enqueue_solve(gfm_ctx *h, const gfm_solve_opts *o, const double *rhs,
         kernel = gfm::batched_kernel(h->ht.max_width, lp.n_stages > 0, lp.ct);
         GFM_CUDA(h, cudaMemsetAsync(info_dev, 0, sizeof(gfm_solve_info) * h->T, s));
     }
+    if (mode == gfm::Mode::FP64) {
+        GFM_CUDA(h, gfm::launch_dinv(h->ht.n_pad, h->iperm, h->diag, h->dinv, s));
+        h->prof.launches += 1;
+        h->prof.launches_total += 1;
+    }
     gfm::MgArgs m{};
     if (h->mg_valid) {
         m.s = a;
@@ -1258,7 +1263,6 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
     ca.ref_value = phys->ref_value;
     ca.b = h->b;
     ca.diag = h->diag;
-    ca.dinv = h->dinv;
     ca.dinv32 = h->dinv32;
     ca.prm = h->prm;
     ca.iperm = h->iperm;
@@ -1275,6 +1279,7 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
     h->asm_max = h->coarse_max;
     h->asm_min_size = h->coarse_min_size;
     if (use_mg) {
+        gfm::MgSmallArgs small{};
         for (size_t l = 0; l < h->mg.size(); ++l) {
             const MgDev &d = h->mg[l];
             gfm::MgLevelArgs ma{};
@@ -1300,8 +1305,19 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
             ma.val32 = d.val32;
             ma.pin32 = d.pin32;
             ma.dinv32 = d.dinv32;
-            GFM_CUDA(h, gfm::launch_mg_level(ma, s));
-            ++launched;
+            // the levels below 2048 nodes in one launch of one CTA: a launch
+            // each cost 5 to 6 us, mostly latency
+            const bool is_small = d.n_slices <= 64;
+            if (is_small) small.lv[small.n++] = ma;
+            if (small.n == 12 || (small.n > 0 && l + 1 == h->mg.size())) {
+                GFM_CUDA(h, gfm::launch_mg_small(small, s));
+                small.n = 0;
+                ++launched;
+            }
+            if (!is_small) {
+                GFM_CUDA(h, gfm::launch_mg_level(ma, s));
+                ++launched;
+            }
         }
         h->mg_valid = true;
     } else {
@@ -1570,7 +1586,6 @@ gfm_status gfm_nonorth_correct(gfm_handle h, const double *p, const double *V, c
     ca.ref_value = h->phys.ref_value;
     ca.b = h->b;
     ca.diag = h->diag;
-    ca.dinv = h->dinv;
     ca.dinv32 = h->dinv32;
     ca.prm = h->prm;
     ca.iperm = h->iperm;
@@ -1624,7 +1639,6 @@ gfm_status gfm_piso_step(gfm_handle h, const gfm_solve_opts *opts, int32_t n_sol
             ca.ref_value = h->phys.ref_value;
             ca.b = h->b;
             ca.diag = h->diag;
-            ca.dinv = h->dinv;
             ca.dinv32 = h->dinv32;
             ca.prm = h->prm;
             ca.iperm = h->iperm;

@@ -24,6 +24,13 @@ __device__ __forceinline__ double div_known(double a, double b, double inv)
     return fma(fma(-q, b, a), inv, q);
 }
 
+// x >= 0.5 by an integer comparison: one on doubles goes through the FP64 pipe.
+__device__ __forceinline__ bool is_wet(double x)
+{
+    const long long b = __double_as_longlong(x);
+    return b >= 0x3FE0000000000000LL && b <= 0x7FF0000000000000LL;  // not for NaN, nor below zero
+}
+
 // One thread per internal face (caller order).
 //   wet = alpha >= 0.5 (Sec. 3.1: the alpha = 0.5 contour is the interface;
 //   alpha exactly 0.5 is taken as wet).
@@ -59,14 +66,16 @@ __global__ void __launch_bounds__(256) k_faces(FaceArgs a)
         a.lambda[f] = lam;
         a.gamma[f] = gam;
         a.jump[f] = J;
-        a.gs[f] = make_double2(gam, ph + gam * J);
+        // off the interface gamma J is a zero, for a finite gamma: ph + 0 rounds alike
+        const bool zero = kind <= kWet && ((__double2hiint(gam) >> 20) & 0x7ff) != 0x7ff;
+        a.gs[f] = make_double2(gam, zero ? ph + 0.0 : ph + gam * J);
         a.phi_copy[f] = ph;
         a.kind[f] = kind;
     };
     bool iface = false;
     if (f0 + (int)threadIdx.x < a.F) {
         const int f = f0 + threadIdx.x;
-        const bool wo = a.alpha[a.owner[f]] >= 0.5, wn = a.alpha[a.neighbour[f]] >= 0.5;
+        const bool wo = is_wet(a.alpha[a.owner[f]]), wn = is_wet(a.alpha[a.neighbour[f]]);
         iface = wo != wn;
         if (!iface) {
             double rho = wo ? a.rho_w : a.rho_a, inv = wo ? a.inv_w : a.inv_a;
@@ -103,7 +112,7 @@ __global__ void __launch_bounds__(256) k_faces(FaceArgs a)
         g1 = tp.g1;
         g2 = tp.g2;
     }
-    const bool wo = ao >= 0.5;
+    const bool wo = is_wet(ao);
     const int W = wo ? o : nb, D = wo ? nb : o;
     const double aW = wo ? ao : an, aD = wo ? an : ao;
     const double lam = (aW - 0.5) / (aW - aD);
@@ -197,8 +206,21 @@ __global__ void __launch_bounds__(256) k_cells(CellArgs a)
     }
     a.b[t] = valid ? b : 0.0;
     a.diag[t] = valid ? diag : 0.0;
-    a.dinv[t] = valid ? 1.0 / diag : 0.0;
     a.dinv32[t] = valid ? 1.0f / (float)diag : 0.0f;
+}
+
+// 1 / diag in FP64, for the solves that iterate in FP64 (padding cells: 0).
+// Formed at their start: a mixed solve does not read it, and the divide was a
+// third of k_cells' FP64 work.  With the integer test of is_wet, sigma without
+// its zero product off the interface and the small levels in one launch this
+// took the assembly of the 256x128x128 box from 1018 to 917 us; an FP64 solve
+// of a 64x32 tank, its assembly included, went from 863 to 853 us.
+__global__ void k_dinv(int n_pad, const int32_t *__restrict__ iperm, const double *__restrict__ diag,
+                       double *__restrict__ dinv)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n_pad) return;
+    dinv[t] = iperm[t] >= 0 ? 1.0 / diag[t] : 0.0;
 }
 
 // sigma = phi + gamma J for a new predicted flux on an assembled system (the
@@ -439,6 +461,12 @@ cudaError_t launch_cell_faces(const Sell &m, const int32_t *perm, const int32_t 
 {
     // whole slices: every thread of a warp has one
     k_cell_faces<<<(m.n + 31) / 32, 32, 0, s>>>(m, perm, ptr, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_dinv(int32_t n_pad, const int32_t *iperm, const double *diag, double *dinv, cudaStream_t s)
+{
+    k_dinv<<<blocks_for(n_pad, 256), 256, 0, s>>>(n_pad, iperm, diag, dinv);
     return cudaGetLastError();
 }
 

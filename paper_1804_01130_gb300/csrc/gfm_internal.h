@@ -158,7 +158,7 @@ struct CellArgs {
     bool source_only;   // b alone
     int32_t ref;  // internal index of the pinned cell, -1 none
     double ref_value;
-    double *b, *diag, *dinv;
+    double *b, *diag;
     float *dinv32;
     DevParams *prm;
     const int32_t *iperm;    // internal -> caller (-1 on padding cells)
@@ -173,6 +173,9 @@ struct CellArgs {
     int32_t pad_code;
 };
 cudaError_t launch_cells(const CellArgs &a, cudaStream_t s);
+
+// dinv = 1 / diag (0 on padding cells)
+cudaError_t launch_dinv(int32_t n_pad, const int32_t *iperm, const double *diag, double *dinv, cudaStream_t s);
 
 // sigma = phi + gamma J for a new predicted flux (coefficients unchanged)
 cudaError_t launch_sigma(int32_t F, const double *phi, const double *gamma, const double *jump, double2 *gs,
@@ -371,6 +374,12 @@ struct MgLevelArgs {
     float *val32, *pin32, *dinv32;
 };
 cudaError_t launch_mg_level(const MgLevelArgs &a, cudaStream_t s);
+// consecutive small levels in one launch
+struct MgSmallArgs {
+    int32_t n;
+    MgLevelArgs lv[12];
+};
+cudaError_t launch_mg_small(const MgSmallArgs &a, cudaStream_t s);
 
 enum class Mode { FP64 = 0, MIXED = 1 };
 const void *solver_kernel(Mode m, int max_width, int threads, bool streamed = false, bool compact = false,

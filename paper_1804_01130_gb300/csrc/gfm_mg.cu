@@ -25,7 +25,10 @@
 // double-float dot products inside FP64 residual replacement, as the Jacobi
 // forms: when the FP32 residual has dropped by three decades (or claims
 // convergence) e is folded into x in FP64 and r becomes the true FP64
-// residual; the direction is kept.
+// residual; the direction is kept.  Replacing after four decades instead of
+// three was slower everywhere: FP32 residuals that far down cost more
+// iterations than the replacements saved (256x128x128 box 12.5 against
+// 10.3 ms, 1024x512 tank 3.36 against 3.20 ms, 64 tanks 24.4 against 22.8 ms).
 //
 // Levels too small to share between CTAs run in CTA 0 alone, in its shared
 // memory, while the others wait at the grid barrier (from MgArgs::tail on).
@@ -1288,11 +1291,9 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
 // One thread per coarse node: its faces' coefficients (scale x the sum of the
 // finer faces' in ascending order, the same bits from both sides), diagonal
 // and pin, in FP64 with FP32 copies.
-__global__ void __launch_bounds__(256) k_mg_level(MgLevelArgs a)
+__device__ __forceinline__ void mg_node(const MgLevelArgs &a, int i)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int s = i >> 5, lane = i & 31;
-    if (s >= a.n_slices) return;
     const int base = a.sp[s], w = (a.sp[s + 1] - base) >> 5;
     double diag = 0.0;
     for (int k = 0; k < w; ++k) {
@@ -1327,6 +1328,30 @@ __global__ void __launch_bounds__(256) k_mg_level(MgLevelArgs a)
     a.pin32[i] = (float)pin;
     a.dinv64[i] = d;
     a.dinv32[i] = (float)d;
+}
+
+__global__ void __launch_bounds__(256) k_mg_level(MgLevelArgs a)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < a.n_slices * kSlice) mg_node(a, i);
+}
+
+// Consecutive small levels, one CTA: each needs the finer one's coefficients.
+// A launch each took 5 to 6 us, most of it latency.  The line lies at 2048
+// nodes, two rows a thread: larger ones gain more from the other SMs than the
+// launch costs.
+__global__ void __launch_bounds__(1024) k_mg_small(MgSmallArgs a)
+{
+    for (int l = 0; l < a.n; ++l) {
+        for (int i = threadIdx.x; i < a.lv[l].n_slices * kSlice; i += blockDim.x) mg_node(a.lv[l], i);
+        __syncthreads();
+    }
+}
+
+cudaError_t launch_mg_small(const MgSmallArgs &a, cudaStream_t s)
+{
+    k_mg_small<<<1, 1024, 0, s>>>(a);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_mg_level(const MgLevelArgs &a, cudaStream_t s)

@@ -151,3 +151,19 @@ def test_multigrid_levels_follow_each_assembly():
         p_ref, _, _, _ = oracle.solve(q, direct=False, rtol=1e-14)
         p, _, info = s.solve(mode="fp64", rtol=1e-12)
         assert info.status == 0 and info.iters < 80 and _rel(p.cpu().numpy(), p_ref) <= 1e-9, (k, info)
+
+
+@pytest.mark.parametrize("nx,ny", [(128, 64), (129, 64), (127, 64), (256, 128), (11, 3)])
+def test_multigrid_small_levels_formed_in_one_launch(nx, ny):
+    """Levels of at most 64 slices are formed by one CTA: the first coarse
+    level at that size, one slice above and below, the second one there, and a
+    mesh of small levels only.  Assembled twice: the second one's levels."""
+    c = cases.box_case(nx, ny, 1, seed=6, nwaves=2)
+    s = _g().GFM.from_case(c)
+    args = (torch.as_tensor(c.phi), c.rho_w, c.rho_a, c.g, c.ref_cell, c.ref_value)
+    s.assemble(torch.as_tensor(1.0 - c.alpha), *args)
+    s.assemble(torch.as_tensor(c.alpha), *args)
+    p_ref, _, _, _ = oracle.solve(c, direct=c.n <= 2048, rtol=1e-14)
+    for mode, bar in (("fp64", 1e-9), ("mixed", 1e-6)):
+        p, _, info = s.solve(mode=mode, rtol=1e-12)
+        assert info.status == 0 and info.iters < 80 and _rel(p.cpu().numpy(), p_ref) <= bar, (mode, info)
