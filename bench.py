@@ -35,12 +35,14 @@ end-to-end rate through the public API on host buffers.
 The default run (tank2d, one GPU) also measures box3d and batch64 and adds
 them to the same JSON line under "workloads": the tank's FP32 working set
 stays in L2, so its roofline fraction is an effective-bandwidth figure, while
-the box and the batch stream ~370-450 MB per iteration through HBM.
+the box and the batch stream ~1.2-1.5 GB per V-cycle through HBM and L2.
 
 Iterations are not alike on the two sides: a GPU iteration is one FP32 PCG
-step preconditioned by Jacobi plus the coarse space of one-phase regions; an
-oracle iteration is one FP64 Jacobi-PCG step.  cpu_baseline therefore reports
-both the oracle's fixed-count rate and its time to the workload's tolerance.
+step preconditioned by a multigrid V-cycle (some five operator passes over the
+mesh, and 20 to 60 iterations a solve); an oracle iteration is one FP64
+Jacobi-PCG step (one pass, 1 700 to 4 800 iterations).  cpu_baseline therefore
+reports both the oracle's fixed-count rate and its time to the workload's
+tolerance, and ms_per_step and speedup are the figures to compare.
 
 Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl gfm|reference]
                        [--workload tank2d|box3d|batch64] [--no-sub]
@@ -244,6 +246,15 @@ def _bytes_model(n, F, iters, refinements):
     return n * iters * (52 + 12 * F / n) + n * refinements * (24 + 16 * F / n)
 
 
+def _vcycle_bytes_model(n, F, iters, refinements):
+    """Algorithmic bytes of the multigrid solve's mesh level: five passes over
+    the FP32 rows (12 B per face and pass; x, r and 1/D read, x written: 16 B
+    per cell and pass), the CG updates of z, p, s, e, r (36 B per cell), and
+    (24 + 16 F/n) per cell and FP64 residual replacement.  The coarse levels
+    (a third more in 2D, a seventh in 3D) are left out."""
+    return n * iters * (116 + 60 * F / n) + n * refinements * (24 + 16 * F / n)
+
+
 # ---------------------------------------------------------------------------
 # workloads
 # ---------------------------------------------------------------------------
@@ -273,14 +284,14 @@ class SingleMesh:
         # launch shape picked by the library's autotuner on this system
         self.h.assemble(self.alpha, self.phi, **self.phys)
         thr, per_sm, _ = self.h.autotune(mode="mixed", rtol=self.rtol, inner_rtol=INNER_RTOL, trials=2)
-        # the iteration form the autotuner kept: two passes and two all-reduces per
-        # FP32 iteration (k_solve_mixed) or one fused pass and one (k_solve_fused)
-        form = self.h.iteration_form()
-        self.kernel = "k_solve_fused" if form == 2 else "k_solve_mixed"
+        # pinned and with a coarse space (the default): one iteration is a
+        # conjugate-gradient step with a multigrid V-cycle, the mesh level read five
+        # times; cell-iterations/s are not those of a Jacobi iteration, times are
+        self.kernel = "k_solve_mg"
         self.config = {"cells": c.n, "faces": c.F, "rtol": self.rtol, "inner_rtol": INNER_RTOL, "mode": "mixed",
                        "renumber": RENUMBER_NAME[RENUMBER[key]],
-                       "launch": {"threads": thr, "ctas_per_sm": per_sm, "autotuned": True,
-                                  "form": "fused" if form == 2 else "two-pass"}}
+                       "iteration": "CG step with one V(2,2) multigrid cycle",
+                       "launch": {"threads": thr, "ctas_per_sm": per_sm, "autotuned": True}}
 
     def close(self):
         self.h.close()
@@ -301,7 +312,7 @@ class SingleMesh:
     def result(self):
         info = self.g.GFM.info_from_device(self.h._info_dev)
         ok = info.status == 0
-        return ok, self.n * info.iters, _bytes_model(self.n, self.F, info.iters, info.refinements), \
+        return ok, self.n * info.iters, _vcycle_bytes_model(self.n, self.F, info.iters, info.refinements), \
             {"iters_per_solve": info.iters, "refinements": info.refinements, "rel_res_l2": info.rel_res_l2}
 
     def extras(self, flush, stream, check_oracle: bool):
@@ -493,7 +504,7 @@ class Batch64:
         recs = self.h.infos_from_device(self.h._info_dev)
         ok = all(r.status == 0 for r in recs)
         ci = sum(t.n * r.iters for t, r in zip(self.tanks, recs))
-        by = sum(_bytes_model(t.n, t.F, r.iters, r.refinements) for t, r in zip(self.tanks, recs))
+        by = sum(_vcycle_bytes_model(t.n, t.F, r.iters, r.refinements) for t, r in zip(self.tanks, recs))
         its = [r.iters for r in recs]
         return ok, ci, by, {"iters_per_tank_min": min(its), "iters_per_tank_max": max(its),
                             "worst_rel_res_l2": max(r.rel_res_l2 for r in recs)}
@@ -729,7 +740,7 @@ def _cpu_baseline(key, seconds: float, tol_budget_s: float = 45.0):
     tt, its, ok = _oracle_time_to_tol(systems, rtol, dt / iters, tol_budget_s)
     return {"value": ci / dt, "unit": UNIT, "cores": int(oracle.max_threads()), "kind": "oracle",
             "sample": f"{iters} Jacobi-PCG iterations of the FP64 CSR oracle on {what} ({dt:.1f} s)",
-            "iteration": "one FP64 Jacobi-PCG step (no coarse space): not the GPU's two-level FP32 step",
+            "iteration": "one FP64 Jacobi-PCG step (no coarse levels): not the GPU's V-cycle step",
             "time_to_tol": {"rtol": rtol, "seconds": tt, "iters": its, "converged": ok,
                             "on": what, "from": "x = 0, Jacobi-PCG, stop on the true residual"}}
 
@@ -821,14 +832,15 @@ def measure(key, steps, warmup, rank, world, dev, stream, flush, *, check_oracle
     kms = statistics.mean(kernel_ms)
     achieved = by / (kms * 1e-3) / 1e9
     peak, peak_kind = _peaks()
-    kname = getattr(w, "kernel", "k_solve_batched" if key == "batch64" else "k_solve_mixed")
+    kname = getattr(w, "kernel", "k_solve_mg")
     trec, sha = _traffic_record(key, kname)
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": (trec["dram_bytes_per_launch"] if trec else None),
             "kernel": kname, "kernel_ms": kms,
             "peak_kind": peak_kind, "frac_of_spec_8000_gbs": achieved / 8000.0,
             "algorithmic_bytes_per_launch": by, "solver_source_sha": sha,
-            "bytes_model": "(52 + 12 F/n) B per cell-iteration + (24 + 16 F/n) B per cell per FP64 replacement"}
+            "bytes_model": "(116 + 60 F/n) B per cell-iteration (mesh level of a V-cycle) + (24 + 16 F/n) B per "
+                           "cell per FP64 replacement"}
     if trec is None:
         roof["traffic_note"] = "no DRAM capture of this kernel on the current solver source"
     if key == "tank2d":

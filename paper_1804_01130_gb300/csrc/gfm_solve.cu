@@ -1,8 +1,9 @@
 // Persistent, cooperative solver kernels for the GFM pressure equation.
 //
 // The paper names no linear solver (it reports residual levels only,
-// Sec. 4.1.1); both kernels run Jacobi-preconditioned conjugate gradients on
-// the symmetric positive definite pinned system of Sec. 3.1.
+// Sec. 4.1.1); these kernels run Jacobi-preconditioned conjugate gradients.
+// They serve the systems without multigrid levels, unpinned ones and those of
+// gfm_set_coarse(0); the others are gfm_mg.cu's.
 //
 //  k_solve_fp64  : textbook PCG, all FP64, three passes per iteration
 //                  (SpMV + p.q | x, r update + preconditioner + r.z | new
