@@ -1305,9 +1305,8 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
             ma.val32 = d.val32;
             ma.pin32 = d.pin32;
             ma.dinv32 = d.dinv32;
-            // the levels below 2048 nodes in one launch of one CTA: a launch
-            // each cost 5 to 6 us, mostly latency
-            const bool is_small = d.n_slices <= 64;
+            // the levels of up to 256 nodes in one launch of one CTA (k_mg_small)
+            const bool is_small = d.n_slices <= 8;
             if (is_small) small.lv[small.n++] = ma;
             if (small.n == 12 || (small.n > 0 && l + 1 == h->mg.size())) {
                 GFM_CUDA(h, gfm::launch_mg_small(small, s));

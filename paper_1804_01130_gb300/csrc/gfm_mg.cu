@@ -1373,10 +1373,11 @@ __global__ void __launch_bounds__(256) k_mg_level(MgLevelArgs a)
 }
 
 // Consecutive small levels, one CTA: each needs the finer one's coefficients.
-// A launch each took 5 to 6 us, most of it latency.  The line lies at 2048
-// nodes, two rows a thread: larger ones gain more from the other SMs than the
-// launch costs.
-__global__ void __launch_bounds__(1024) k_mg_small(MgSmallArgs a)
+// A launch each took 5 to 6 us, most of it latency.  The line lies at 256
+// nodes, a row a thread: above it one SM's FP64 pipe costs more than the
+// launch saves (at 2048 nodes the assembly of the 256x128x128 box took 876 us,
+// at 256 it takes 869; the 1024x512 tank, assembled and solved, 3129 and 3112).
+__global__ void __launch_bounds__(256) k_mg_small(MgSmallArgs a)
 {
     for (int l = 0; l < a.n; ++l) {
         for (int i = threadIdx.x; i < a.lv[l].n_slices * kSlice; i += blockDim.x) mg_node(a.lv[l], i);
@@ -1386,7 +1387,7 @@ __global__ void __launch_bounds__(1024) k_mg_small(MgSmallArgs a)
 
 cudaError_t launch_mg_small(const MgSmallArgs &a, cudaStream_t s)
 {
-    k_mg_small<<<1, 1024, 0, s>>>(a);
+    k_mg_small<<<1, 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 
