@@ -546,7 +546,7 @@ gfm_status enqueue_solve(gfm_ctx *h, const gfm_solve_opts *o, const double *rhs,
         m.z = second(v1);
         m.p = mixed ? (void *)h->P32 : (void *)h->p64;
         m.sv = mixed ? (void *)h->S32 : (void *)h->q64;
-        m.e = h->E;
+        m.e = mixed ? (void *)h->E : (void *)h->UP0;
         for (size_t l = 0; l < h->mg.size(); ++l) {
             const MgDev &d = h->mg[l];
             gfm::MgLevel &lv = m.lv[l + 1];

@@ -357,7 +357,7 @@ struct MgArgs {
                                                    // of the largest share, byte offset of the coefficients)
     const int32_t *tank_off;  // batched: [T+1] internal cell offsets
     const DevParams *tprm;    // batched: pin of each tank
-    void *z, *p, *sv, *e;     // z = M^{-1} r, direction, A p, FP32 correction
+    void *z, *p, *sv, *e;     // z = M^{-1} r, direction, A p, correction since the last replacement
     MgLevel lv[kMgLevels];
 };
 const void *mg_kernel(bool mixed, int max_width, int slices_per_sm, int *max_threads);

@@ -21,7 +21,10 @@
 // s = A z + beta s.
 //
 // Precision.  GFM_FP64 (T = double): everything FP64; the result is accepted
-// on the true residual b - A x.  GFM_MIXED (T = float): FP32 iterations with
+// on the true residual b - A x, from which the directions start anew.  The
+// steps are summed in e and folded into x there, so that x carries one
+// rounding and not one per step: where the rounding of x is all that is left of
+// the residual this is 5-10% less, as low as the Jacobi form gets.  GFM_MIXED (T = float): FP32 iterations with
 // double-float dot products inside FP64 residual replacement, as the Jacobi
 // forms: when the FP32 residual has dropped by three decades (or claims
 // convergence) e is folded into x in FP64 and r becomes the true FP64
@@ -51,6 +54,10 @@ constexpr int kMgNR = 2;       // most values one all-reduce sums
 constexpr float kOm1 = 0.56418f;  // Chebyshev degree 2 on [0.35, 2]: 1 / (1.175 +- 0.825 cos(pi/4))
 constexpr float kOm2 = 1.69016f;
 constexpr int kSegLane = 8;    // tanks with more segments are summed by a warp
+// Most iterations between residual replacements, after which the stall test
+// ends a solve that gets nowhere.  FP64: far above what a solve takes (20 to
+// 240), since every replacement restarts its directions.
+constexpr int kMgCheck32 = 40, kMgCheck64 = 400;
 
 enum MgAct : int { kMgGo = 0, kMgConverged = 1, kMgNotConverged = 2, kMgBreakdown = 3 };
 enum MgFlag : int { kFlagNone = 0, kFlagUpdate = 1, kFlagRestart = 2, kFlagCap = 3 };
@@ -67,7 +74,7 @@ struct MgShared {
     int c0[kMaxTanks], c1[kMaxTanks];  // first and last CTA holding slices of the tank
     int seg_s0[kMaxTanks], seg_s1[kMaxTanks], seg_tank[kMaxTanks];  // this CTA's segments
     int wide[kMaxTanks];
-    int nseg, n_wide, any_active, any_flag, replan, fail;
+    int nseg, n_wide, any_active, any_flag, replan, fail, polish;
 };
 
 // ---- sums ------------------------------------------------------------------
@@ -912,7 +919,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
     const MgLevel &l0 = a.lv[0];
     T *R = static_cast<T *>(l0.b), *XA = static_cast<T *>(l0.xa), *XB = static_cast<T *>(l0.xb);
     T *RES = static_cast<T *>(l0.res), *Z = static_cast<T *>(a.z), *P = static_cast<T *>(a.p), *S = static_cast<T *>(a.sv);
-    T *E = static_cast<T *>(a.e);  // FP32 correction (mixed); unused in FP64
+    T *E = static_cast<T *>(a.e);  // correction since the last replacement
     const T *dinv = static_cast<const T *>(l0.dinv);
     // pinned cell and end of the real cells of a tank
     auto tank_end = [&](int t) { return T_ > 1 ? a.tank_off[t] + a.s.n_per_tank[t] : a.s.m.n; };
@@ -929,7 +936,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
             const int i = s * kSlice + lane;
             if (i < end) {
                 a.s.x64[i] = a.s.use_x0 ? a.s.p_user[a.s.iperm[i]] : 0.0;
-                if constexpr (kMixed) E[i] = T(0);
+                E[i] = T(0);
                 const double bi = a.s.b[i];
                 vb[0] = fma(bi, bi, vb[0]);
             }
@@ -959,11 +966,15 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
     __syncthreads();
     const int cap_updates = a.s.max_refine + 1 + (kMixed ? (int)(2.0 * log10(1.0 / a.s.rtol)) : 0);
 
-    // r = b - A x (FP64) for the flagged tanks, x += e first (mixed); also
+    // r = b - A x (FP64) for the flagged tanks, x += e first; also
     // the V-cycle's first sweep from zero.  Then the tanks' decisions.
-    auto replace = [&](bool first) -> bool {
+    // polish > 0 (FP64): x += D^{-1} r on every second cell instead.  A claim
+    // refuted by less than 1.4 leaves r to the rounding of x, which these sweeps
+    // undo where it is largest: six of them take 15-20% off, and what the
+    // Jacobi form can reach, which ends in such single-cell steps, is reached.
+    auto replace_pass = [&](bool first, int polish) -> bool {
         if (T_ > 1 && !first) plan([&](int t) { return sh.flag[t] != kFlagNone; });
-        if (kMixed && !first) {
+        if (!first) {
             for (int q = 0; q < sh.nseg; ++q) {
                 const int t = sh.seg_tank[q], end = tank_end(t);
                 if (sh.flag[t] == kFlagNone) continue;
@@ -975,7 +986,8 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                     for (int u = 0; u < 4; ++u) {
                         const int i = (sb + u * nw) * kSlice + lane;
                         const bool ok = sb + u * nw < sh.seg_s1[q] && i < end;
-                        e[u] = ok ? E[i] : T(0);
+                        if (polish > 0) e[u] = ok && ((i ^ polish) & 1) ? dinv[i] * R[i] : T(0);
+                        else e[u] = ok ? E[i] : T(0);
                         x[u] = ok ? a.s.x64[i] : 0.0;
                     }
 #pragma unroll
@@ -1016,22 +1028,32 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
         }
         if (!mg_allreduce<1, A>(c)) return false;
         if (threadIdx.x < 32) {
-            bool active = false;
+            bool active = false, again = false;
             for (int t = threadIdx.x; t < T_; t += 32) {
                 const int f = sh.flag[t];
                 if (sh.act[t] == kMgGo && f != kFlagNone) {
-                    sh.flag[t] = kFlagNone;
-                    sh.wait[t] = 0;
-                    sh.last_rep[t] = sh.iters[t];
-                    ++sh.updates[t];
                     const double rr = sh.tot[0][t];
                     const double rel2 = rr / (sh.bnorm[t] * sh.sc[t] * (sh.bnorm[t] * sh.sc[t]));
                     // FP32 residual entries carry 6e-8 each: stay below the target by as much
                     const double tol2 = a.s.rtol * a.s.rtol * (kMixed ? 1.0 - 1e-6 : 1.0);
+                    if (!kMixed && f == kFlagUpdate && polish < 6 && rel2 > tol2 && rel2 <= 2.0 * tol2) {
+                        again = active = true;
+                        continue;
+                    }
+                    sh.flag[t] = kFlagNone;
+                    sh.wait[t] = 0;
+                    sh.last_rep[t] = sh.iters[t];
+                    ++sh.updates[t];
                     sh.fresh[t] |= (f == kFlagRestart) ? 1 : 0;
                     // the recurrence had drifted from the true residual: its
-                    // direction is no longer conjugate to anything
-                    if (!(rr <= 4.0 * sh.rho[t])) sh.fresh[t] = 1;
+                    // direction is no longer conjugate to anything.  In FP64
+                    // that holds at every replacement: one comes when the
+                    // recurrence claims convergence, where the true residual
+                    // may be as long as the recurrence's but is mostly the
+                    // rounding of x and points elsewhere.  Steps with an old
+                    // direction and a new residual made it grow there (from
+                    // 6e-13 to 3e-10 and on to the iteration cap).
+                    if (!kMixed || !(rr <= 4.0 * sh.rho[t])) sh.fresh[t] = 1;
                     sh.rho_max[t] = rr;
                     if (rel2 <= tol2) sh.act[t] = kMgConverged;
                     else if (f == kFlagCap) sh.act[t] = kMgNotConverged;
@@ -1044,7 +1066,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                         } else {
                             ++sh.stall[t];
                         }
-                        if (sh.act[t] == kMgGo && (sh.stall[t] > (kMixed ? 8 : 2) || sh.updates[t] > cap_updates))
+                        if (sh.act[t] == kMgGo && (sh.stall[t] > (kMixed ? 8 : 3) || sh.updates[t] > cap_updates))
                             sh.act[t] = kMgNotConverged;
                     } else {
                         sh.best[t] = rel2;
@@ -1054,10 +1076,21 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                 active |= sh.act[t] == kMgGo;
             }
             active = __any_sync(0xffffffffu, active);
-            if (threadIdx.x == 0) sh.any_active = active;
+            again = __any_sync(0xffffffffu, again);
+            if (threadIdx.x == 0) {
+                sh.any_active = active;
+                sh.polish = again;
+            }
         }
         __syncthreads();
         if (T_ > 1) plan(working);
+        return true;
+    };
+    auto replace = [&](bool first) -> bool {
+        if (!replace_pass(first, 0)) return false;
+        if constexpr (!kMixed)
+            for (int k = 1; sh.polish; ++k)
+                if (!replace_pass(false, k)) return false;
         return true;
     };
     if (!replace(true)) { bail(); return; }
@@ -1134,7 +1167,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
             sh.fresh[t] = 0;
         }
         __syncthreads();
-        // e += alpha p (FP64: x), r -= alpha s, the next V-cycle's first sweep, r.r
+        // e += alpha p, r -= alpha s, the next V-cycle's first sweep, r.r
         for (int q = 0; q < sh.nseg; ++q) {
             const int t = sh.seg_tank[q], end = tank_end(t), e1 = sh.seg_s1[q];
             A v[1] = {A{}};
@@ -1142,9 +1175,6 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                 T al;
                 if constexpr (kMixed) al = sh.al32[t];
                 else al = sh.al64[t];
-                T *X;
-                if constexpr (kMixed) X = E;
-                else X = a.s.x64;
                 for (int sb = sh.seg_s0[q] + warp; sb < e1; sb += UB * nw) {
                     T p[UB], s[UB], r[UB], x[UB], d[UB];
 #pragma unroll
@@ -1154,14 +1184,14 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                         p[u] = ok ? P[i] : T(0);
                         s[u] = ok ? S[i] : T(0);
                         r[u] = ok ? R[i] : T(0);
-                        x[u] = ok ? X[i] : T(0);
+                        x[u] = ok ? E[i] : T(0);
                         d[u] = ok ? dinv[i] : T(0);
                     }
 #pragma unroll
                     for (int u = 0; u < UB; ++u) {
                         const int i = (sb + u * nw) * kSlice + lane;
                         if (sb + u * nw < e1 && i < end) {
-                            X[i] = fma(al, p[u], x[u]);
+                            E[i] = fma(al, p[u], x[u]);
                             const T rn = fma(-al, s[u], r[u]);
                             R[i] = rn;
                             XA[i] = om1 * d[u] * rn;
@@ -1175,9 +1205,13 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
         if (!mg_allreduce<1, A>(c)) { bail(); return; }
         // A tank asks for a residual replacement when its residual claims
         // convergence, can no longer be trusted in FP32 (three decades below
-        // the last true one) or cannot go on.  In a batch a tank that claims
-        // convergence idles until the round, which comes when no tank is left
-        // iterating or some tank must not wait.
+        // the last true one), has gone kMgCheck32 or kMgCheck64 iterations without one, or
+        // cannot go on.  In a batch a tank that claims convergence idles until
+        // the round, which comes when no tank is left iterating or some tank
+        // must not wait.  In FP64 each claim that the true residual refuted
+        // halves the next one's target: near the rounding floor the true
+        // residual is the recurrence's and x's rounding added up, so a claim
+        // just below the tolerance would be refuted again and again.
         if (threadIdx.x < 32) {
             bool now = false, asked = false, going = false, waits = false;
             for (int t = threadIdx.x; t < T_; t += 32) {
@@ -1196,11 +1230,11 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                 if (it >= a.s.max_iters) {
                     sh.flag[t] = kFlagCap;
                     now = true;
-                } else if (!(rho > 0.81 * sh.rho_stop[t])) {
+                } else if (!(rho > (kMixed ? 0.81 : ldexp(0.81, -2 * min(sh.updates[t] - 1, 8))) * sh.rho_stop[t])) {
                     sh.flag[t] = kFlagUpdate;
                     sh.wait[t] = 1;
                     asked = waits = true;
-                } else if (kMixed && (rho <= 1e-6 * sh.rho_max[t] || it - sh.last_rep[t] >= 40)) {
+                } else if ((kMixed && rho <= 1e-6 * sh.rho_max[t]) || it - sh.last_rep[t] >= (kMixed ? kMgCheck32 : kMgCheck64)) {
                     sh.flag[t] = kFlagUpdate;
                     sh.wait[t] = 1;
                     asked = waits = true;
