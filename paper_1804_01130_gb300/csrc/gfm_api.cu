@@ -217,6 +217,21 @@ struct LaunchPlan {
     size_t dyn = 0;
 };
 
+// Let kernel k be launched with `dyn` bytes of dynamic shared memory.  The limit
+// belongs to the function, shared by every handle and host thread, so it is
+// always set to the same value, the most the device gives the kernel: set to
+// one handle's own need it could fall below another's between that one's plan
+// and its launch (cudaLaunchCooperativeKernel then failed).
+gfm_status allow_shared_memory(gfm_ctx *h, const void *k, size_t dyn)
+{
+    cudaFuncAttributes fa;
+    GFM_CUDA(h, cudaFuncGetAttributes(&fa, k));
+    const int most = h->smem_optin - (int)fa.sharedSizeBytes;
+    if ((long long)dyn > most) return fail(h, GFM_ERR_ARG, "launch shape needs more shared memory than the device has");
+    GFM_CUDA(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    return GFM_OK;
+}
+
 gfm_status plan_launch(gfm_ctx *h, gfm::Mode mode, LaunchPlan *lp)
 {
     const int t = h->tuning.threads;
@@ -297,7 +312,8 @@ gfm_status plan_launch(gfm_ctx *h, gfm::Mode mode, LaunchPlan *lp)
     if (n_stages)
         k = h->batched ? gfm::batched_kernel(h->ht.max_width, true, ct)
                        : gfm::solver_kernel(mode, h->ht.max_width, t, true, ct, fused);
-    GFM_CUDA(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    const gfm_status st = allow_shared_memory(h, k, dyn);
+    if (st != GFM_OK) return st;
     int occ = 0;
     GFM_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, t, dyn));
     if (occ < per) return fail(h, GFM_ERR_ARG, "launch shape cannot be co-resident with its shared-memory staging");
@@ -425,7 +441,8 @@ gfm_status plan_mg(gfm_ctx *h, gfm::Mode mode, MgPlan *mp)
             mp->dyn = std::max(mp->dyn, (size_t)(val + (long long)ts * slots));
         }
     }
-    GFM_CUDA(h, cudaFuncSetAttribute(mp->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mp->dyn));
+    const gfm_status st = allow_shared_memory(h, mp->kernel, mp->dyn);
+    if (st != GFM_OK) return st;
     GFM_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, mp->kernel, t, mp->dyn));
     if (occ < per) return fail(h, GFM_ERR_ARG, "launch shape cannot be co-resident with its shared memory");
     mp->threads = t;
