@@ -463,8 +463,10 @@ gfm_status gfm_iso_advect(gfm_handle h, const double *alpha, const double *phi, 
  * of HBM bandwidth, and interface slots add a dependent load: it was slower
  * on the 3D box and the 64-tank batch, hence off by default.
  * gfm_get_table (host pointers, any may be NULL): whether the compact form
- * is usable for this mesh, its number of classes, and whether the last
- * assembly wrote it.
+ * is usable for this mesh, its number of classes, and whether it can hold the
+ * last assembled system (usable, no face coefficient set).  An assembly whose
+ * solves take the Jacobi forms then wrote it; a multigrid solve reads neither
+ * table, so an assembly for it leaves the compact one out.
  */
 gfm_status gfm_set_table(gfm_handle h, int32_t compact, int32_t force_stream);
 gfm_status gfm_get_table(gfm_handle h, int32_t *compact_usable, int32_t *n_classes, int32_t *compact_valid);

@@ -95,7 +95,9 @@ struct gfm_ctx {
     // compact operator table for the streamed mixed pass (see Sell::ent):
     // usable when every neighbour offset fits 16 bits and the faces fall
     // into at most (kMaxDict - 1) / 2 classes of bit-identical c_f
-    bool ct_ok = false, ent_valid = false;
+    bool ct_ok = false;
+    bool ent_valid = false;  // the last assembly wrote the table
+    bool ct_holds = false;   // the table can hold the last assembled system
     bool ct_pref = false;       // gfm_set_table: use the compact table when usable (off by default)
     bool force_stream = false;  // gfm_set_table: stream the tables even when they fit
     int n_cls = 0;
@@ -1291,7 +1293,8 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
     ca.kind = h->kind;
     ca.pad_code = 2 * h->n_cls;
     GFM_CUDA(h, gfm::launch_cells(ca, s));
-    h->ent_valid = use_ct;
+    h->ent_valid = use_ct && !use_mg;
+    h->ct_holds = use_ct;
     h->mg_valid = false;
     h->asm_max = h->coarse_max;
     h->asm_min_size = h->coarse_min_size;
@@ -1737,7 +1740,7 @@ gfm_status gfm_get_table(gfm_handle h, int32_t *compact_usable, int32_t *n_class
     if (!h) return GFM_ERR_ARG;
     if (compact_usable) *compact_usable = h->ct_ok ? 1 : 0;
     if (n_classes) *n_classes = h->n_cls;
-    if (compact_valid) *compact_valid = h->ent_valid ? 1 : 0;
+    if (compact_valid) *compact_valid = h->ct_holds ? 1 : 0;
     return GFM_OK;
 }
 

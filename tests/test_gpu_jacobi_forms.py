@@ -61,6 +61,27 @@ def test_compact_table_gives_the_full_ones_bits(name, renumber, stream):
     assert _rel(out[0][0].cpu().numpy(), p_ref) <= 1e-6
 
 
+def test_table_of_a_system_that_changes_its_solver():
+    """Multigrid assemblies leave the compact table out: one in between must
+    not leave an older system's table to a Jacobi solve."""
+    c, d = cases.box_case(40, 24, 1, seed=3, ka=0.12), cases.box_case(40, 24, 1, seed=9, ka=0.05, nwaves=2)
+    s, out = _g().GFM.from_case(c), []
+    s.set_table(compact=True, force_stream=True)
+    for q, vectors in ((c, 0), (d, 8), (d, 0)):
+        s.set_coarse(vectors)
+        s.assemble(torch.as_tensor(q.alpha), torch.as_tensor(q.phi), q.rho_w, q.rho_a, q.g, q.ref_cell, q.ref_value)
+        assert s.table_info()["compact_valid"]  # it can hold the system, whichever solver runs
+        out.append(s.solve(mode="mixed", rtol=1e-10)[0].cpu().numpy())
+    for p, q in zip(out, (c, d, d)):
+        assert _rel(p, oracle.solve(q, direct=True)[0]) <= 1e-6
+    rau = torch.as_tensor(np.random.default_rng(4).uniform(0.5, 2.0, d.F))
+    for vectors in (8, 0):
+        s.set_coarse(vectors)
+        s.set_rau(rau)
+        s.assemble(torch.as_tensor(d.alpha), torch.as_tensor(d.phi), d.rho_w, d.rho_a, d.g, d.ref_cell, d.ref_value)
+        assert not s.table_info()["compact_valid"]
+
+
 @pytest.mark.parametrize("compact", [False, True])
 @pytest.mark.parametrize("stream", [False, True])
 def test_batch_of_tanks(stream, compact):
