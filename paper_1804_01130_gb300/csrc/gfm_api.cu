@@ -45,7 +45,7 @@ struct gfm_ctx {
     double *lambda = nullptr, *gamma = nullptr, *jump = nullptr, *phi = nullptr;
     double *cface = nullptr;  // c_f = (S.S)/(S.d)
     double2 *gs = nullptr;    // (gamma, sigma): the pair the cell sums gather
-    double4 *grad_rec = nullptr;  // [2 F] records of the gradient's face pass
+    double4 *grad_rec = nullptr;  // [2 F] records of the gradient's face pass, from its first use on
     double2 *sd = nullptr;        // [F] (S.d, 1 / (S.d))
     int32_t *cf_ptr = nullptr, *cell_face = nullptr;  // faces of each cell, caller order (CellFaces)
     double *dl_dlam = nullptr;
@@ -218,6 +218,24 @@ struct LaunchPlan {
     bool fused = false;                               // MIXED: the one-pass, one-all-reduce form
     size_t dyn = 0;
 };
+
+// The gradient's face records (64 bytes a face), allocated at the first gradient
+// or correction: a handle that only solves or advects has no use for them.
+// That call may be under stream capture, where cudaMalloc is allowed to a
+// thread in relaxed mode.
+gfm_status need_grad_rec(gfm_ctx *h)
+{
+    if (h->grad_rec) return GFM_OK;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    GFM_CUDA(h, cudaThreadExchangeStreamCaptureMode(&mode));
+    const cudaError_t e = dalloc(&h->grad_rec, 2 * (size_t)h->F);
+    GFM_CUDA(h, cudaThreadExchangeStreamCaptureMode(&mode));
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        return fail(h, GFM_ERR_NOMEM, "allocating the gradient's face records");
+    }
+    return GFM_OK;
+}
 
 // Let kernel k be launched with `dyn` bytes of dynamic shared memory.  The limit
 // belongs to the function, shared by every handle and host thread, so it is
@@ -673,7 +691,7 @@ gfm_status alloc_upload(gfm_ctx *h, cudaStream_t s)
     A(owner, F); A(neighbour, F); A(Sf, 3 * (size_t)F); A(C, 3 * (size_t)n);
     A(perm, n); A(iperm, np); A(slice_ptr, (size_t)h->ht.n_slices + 1); A(col, ns); A(face, ns);
     A(val64, ns); A(val32, ns);
-    A(lambda, F); A(gamma, F); A(jump, F); A(cface, F); A(gs, F); A(grad_rec, 2 * (size_t)F); A(sd, F); A(phi, F); A(dl_dlam, F); A(kind, F);
+    A(lambda, F); A(gamma, F); A(jump, F); A(cface, F); A(gs, F); A(sd, F); A(phi, F); A(dl_dlam, F); A(kind, F);
     A(alpha, n); A(b, np); A(diag, np); A(dinv, np); A(x64, np); A(r64, np); A(p64, np); A(q64, np);
     A(rhs, np); A(tmp_user, n); A(tmp_user2, n); A(UP0, np); A(UP1, np); A(Q0, np); A(Q1, np); A(P32, np); A(R32, np); A(S32, np); A(E, np);
     A(dinv32, np);
@@ -1492,6 +1510,8 @@ gfm_status gfm_gradient(gfm_handle h, const double *p, const double *V, const do
     if (grad && !h->assembled) return fail(h, GFM_ERR_STATE, "gradient before assemble");
     clear_stale_error();
     cudaStream_t s = (cudaStream_t)stream;
+    const gfm_status st = need_grad_rec(h);
+    if (st != GFM_OK) return st;
     gfm::GradArgs a{};
     a.n = h->n;
     a.F = h->F;
@@ -1554,6 +1574,8 @@ gfm_status gfm_nonorth_correct(gfm_handle h, const double *p, const double *V, c
         if (e == cudaSuccess) e = dalloc(&h->phi_eff, (size_t)h->F);
         if (e != cudaSuccess) return fail(h, GFM_ERR_NOMEM, "allocating the correction workspace");
     }
+    const gfm_status st = need_grad_rec(h);
+    if (st != GFM_OK) return st;
     gfm::GradArgs ga{};
     ga.n = h->n;
     ga.F = h->F;
