@@ -1026,7 +1026,7 @@ gfm_status gfm_create(const gfm_mesh *mesh, int32_t renumber, gfm_stream stream,
     h->n = n;
     h->F = F;
     gfm_status st = init_device(h);
-    do {
+    do try {
         if (st != GFM_OK) break;
         std::vector<int32_t> ho((size_t)F), hn((size_t)F);
         std::vector<double> hC((size_t)3 * n), hS((size_t)3 * F);
@@ -1066,6 +1066,8 @@ gfm_status gfm_create(const gfm_mesh *mesh, int32_t renumber, gfm_stream stream,
         st = setup_compact(h, s);
         if (st != GFM_OK) break;
         st = setup_mg(h, mg, s);
+    } catch (const std::exception &) {  // the host copies of the mesh, the tables
+        st = fail(h, GFM_ERR_NOMEM, "host memory");
     } while (0);
     if (st != GFM_OK) {
         fprintf(stderr, "gfm_create: %s\n", h->last_error.c_str());
@@ -1092,7 +1094,7 @@ gfm_status gfm_create_batched(const gfm_mesh *meshes, int32_t n_tanks, int32_t r
     clear_stale_error();
     cudaStream_t s = (cudaStream_t)stream;
     gfm_status st = init_device(h);
-    do {
+    do try {
         if (st != GFM_OK) break;
         std::vector<std::vector<int32_t>> ho((size_t)n_tanks), hn((size_t)n_tanks);
         std::vector<std::vector<double>> hC((size_t)n_tanks), hS((size_t)n_tanks);
@@ -1187,6 +1189,8 @@ gfm_status gfm_create_batched(const gfm_mesh *meshes, int32_t n_tanks, int32_t r
         st = setup_mg(h, mg, s);
         if (st != GFM_OK) break;
         st = plan_batch(h);
+    } catch (const std::exception &) {  // the host copies of the mesh, the tables
+        st = fail(h, GFM_ERR_NOMEM, "host memory");
     } while (0);
     if (st != GFM_OK) {
         fprintf(stderr, "gfm_create_batched: %s\n", h->last_error.c_str());

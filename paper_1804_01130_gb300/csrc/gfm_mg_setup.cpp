@@ -3,7 +3,9 @@
 // coefficients are formed on the device by every assembly).
 //
 // Each level merges nodes by passes of pairwise matching (two passes, groups
-// of four, on 2D-like meshes; three, groups of eight, on 3D-like ones).  A
+// of four, on 2D-like meshes; three, groups of eight, on 3D-like ones), the
+// repeated pairwise aggregation of Notay (Electron. Trans. Numer. Anal. 37,
+// 123-146, 2010) with a strength taken from the geometry.  A
 // node is matched with its unmatched neighbour across the strongest face,
 // the strength being the two-point coefficient |S|^2 / (S.d) of the merged
 // face and the current centroids, so stretched cells are first merged along
@@ -21,8 +23,8 @@
 // merged cells.
 #include <algorithm>
 #include <cmath>
+#include <exception>
 #include <numeric>
-#include <system_error>
 #include <thread>
 
 #include "gfm_mg_setup.h"
@@ -59,7 +61,7 @@ void parallel_ranges(int n, Fn fn)
     int t = 0;
     try {
         for (; t < nt; ++t) th.emplace_back(fn, (int)((long long)n * t / nt), (int)((long long)n * (t + 1) / nt));
-    } catch (const std::system_error &) {  // no thread to be had: the rest here
+    } catch (const std::exception &) {  // no thread (or memory for one) to be had: the rest here
         fn((int)((long long)n * t / nt), n);
     }
     for (auto &q : th) q.join();
