@@ -34,7 +34,7 @@ UNITS = {
     "gfm_gradient.cu": [],
     "gfm_iso.cu": [],
 }
-HEADERS = ["gfm_internal.h", "gfm_grid.cuh", "gfm_setup.h", "gfm_mg_setup.h"]
+HEADERS = ["gfm_internal.h", "gfm_grid.cuh", "gfm_div.cuh", "gfm_setup.h", "gfm_mg_setup.h"]
 
 
 def nvcc() -> str:

@@ -5,24 +5,12 @@
 // rounds exactly as written, left to right, so the face quantities and the
 // ordered per-cell sums are bit-reproducible against any IEEE-754 FP64
 // evaluation of the same formulas in the same order.
+#include "gfm_div.cuh"
 #include "gfm_internal.h"
 
 namespace gfm {
 
 enum : int8_t { kDry = 0, kWet = 1, kIfOwnerWet = 2, kIfOwnerDry = 3 };
-
-// a / b correctly rounded from inv = RN(1 / b): one Newton step on the
-// quotient with an exact remainder (Markstein, IBM J. Res. Dev. 34, 1990), for
-// |a| far from under- and overflow and a normal b whose significand is not
-// all ones; the caller passes inv = 0 when b is not.  Three instructions of
-// the FP64 pipe instead of a divide's ten or so.
-__device__ __forceinline__ double div_known(double a, double b, double inv)
-{
-    const int e = (__double2hiint(a) >> 20) & 0x7ff;
-    if (inv == 0.0 || e < 0x100 || e > 0x6ff) return a / b;
-    const double q = a * inv;
-    return fma(fma(-q, b, a), inv, q);
-}
 
 // x >= 0.5 by an integer comparison: one on doubles goes through the FP64 pipe.
 __device__ __forceinline__ bool is_wet(double x)

@@ -37,20 +37,12 @@
 // order each costs a whole DRAM granule.  201x101x99 cells in a random order,
 // gradient and velocity: 2090 -> 757 us (1410 with the cells in internal
 // order and both centres gathered by the face pass).
+#include "gfm_div.cuh"
 #include "gfm_internal.h"
 
 namespace gfm {
 
 namespace {
-
-// a / b correctly rounded from inv = RN(1 / b), 0 where that does not hold (see gfm_assemble.cu)
-__device__ __forceinline__ double div_known(double a, double b, double inv)
-{
-    const int e = (__double2hiint(a) >> 20) & 0x7ff;
-    if (inv == 0.0 || e < 0x100 || e > 0x6ff) return a / b;
-    const double q = a * inv;
-    return fma(fma(-q, b, a), inv, q);
-}
 
 // A whole record in one 32-byte access (sm_100 and later), a full sector.
 __device__ __forceinline__ void store_record(double4 *p, double x, double y, double z, double w)
