@@ -60,12 +60,7 @@ struct gfm_ctx {
     float *R32 = nullptr, *S32 = nullptr, *E = nullptr, *dinv32 = nullptr;
     // two-level preconditioner (coarse space of connected one-phase regions)
     int32_t *cc_parent = nullptr, *cc_size = nullptr, *cc_cand = nullptr, *cc_counters = nullptr;
-    int32_t *cc_bcount = nullptr, *cc_boff = nullptr;
-    double *cc_epart = nullptr;
-    int8_t *comp = nullptr;
-    gfm::CrossFace *cross = nullptr;
     gfm::Coarse *coarse = nullptr;
-    int max_cross = 0;
     int coarse_max = gfm::kMaxCoarse, coarse_min_size = 64;
     int asm_max = 0, asm_min_size = 64;  // the same as the last assembly took them
     // multigrid hierarchy; used by pinned systems unless gfm_set_coarse(0)
@@ -81,7 +76,7 @@ struct gfm_ctx {
     int4 *cta = nullptr;
     int2 *tank_cta = nullptr;
     int32_t *tcoff = nullptr, *tioff = nullptr;  // [T+1] caller / internal cell offsets of the tanks
-    gfm::TankCoarse *tco = nullptr;              // [T] coarse space of each tank
+    gfm::TankCoarse *tco = nullptr;              // [T] one-phase regions of each tank
     std::vector<double> bweight;  // per-tank work weights of the CTA table (empty: by slices)
     gfm_solve_info *binfos = nullptr, *binfos_h = nullptr;
     // host-buffer entry point staging
@@ -159,8 +154,7 @@ void free_all(gfm_ctx *h)
                     h->tmp_user2, h->UP0, h->UP1, h->Q0, h->Q1, h->P32, h->R32, h->S32, h->E, h->dinv32, h->stage_alpha,
                     h->stage_phi, h->stage_p, h->prm, h->bar,
                     h->err, h->partials, h->dinfo, h->cc_parent, h->cc_size, h->cc_cand, h->cc_counters,
-                    h->cc_bcount, h->cc_boff, h->cc_epart,
-                    h->comp, h->cross, h->coarse, h->ftank, h->stank, h->tncell, h->tphys, h->tprm, h->cta,
+                    h->coarse, h->ftank, h->stank, h->tncell, h->tphys, h->tprm, h->cta,
                     h->tank_cta, h->binfos, h->tcoff, h->tioff, h->tco, h->rau, h->nonorth_corr, h->phi_eff,
                     h->grad_scr, h->ent, h->fcls, h->ctank, h->ccls, h->dict};
     for (void *p : ptrs)
@@ -519,9 +513,6 @@ gfm_status enqueue_solve(gfm_ctx *h, const gfm_solve_opts *o, const double *rhs,
     a.max_refine = o->max_refine;
     a.use_x0 = use_x0;
     a.budget_ns = (unsigned long long)(o->timeout_ms * 1e6);
-    a.coarse = h->coarse;
-    a.comp = h->comp;
-    a.cross = h->cross;
     a.cache_cap = lp.cache_cap;
     a.meta_slots = lp.meta_slots;
     a.n_stages = lp.n_stages;
@@ -541,7 +532,6 @@ gfm_status enqueue_solve(gfm_ctx *h, const gfm_solve_opts *o, const double *rhs,
         ba.tank_cta = h->tank_cta;
         ba.tprm = h->tprm;
         ba.infos = info_dev;
-        ba.tco = h->tco;
         kernel = gfm::batched_kernel(h->ht.max_width, lp.n_stages > 0, lp.ct);
         GFM_CUDA(h, cudaMemsetAsync(info_dev, 0, sizeof(gfm_solve_info) * h->T, s));
     }
@@ -697,11 +687,8 @@ gfm_status alloc_upload(gfm_ctx *h, cudaStream_t s)
     A(dinv32, np);
     A(stage_alpha, n); A(stage_phi, F); A(stage_p, n);
     A(prm, 1); A(bar, 1); A(err, 1); A(partials, 2 * (size_t)h->max_grid * gfm::kMaxReduce); A(dinfo, 1);
-    h->max_cross = (int)std::min<long long>((long long)F, std::max<long long>(65536, (long long)F / 8));
-    A(cc_parent, n); A(cc_size, n); A(cc_cand, gfm::kMaxCandidates); A(cc_counters, 2);
-    A(cc_bcount, (F + 255) / 256); A(cc_boff, (F + 255) / 256);
-    A(cc_epart, (size_t)gfm::kCoarseEParts * gfm::kMaxCoarse * gfm::kMaxCoarse);
-    A(comp, np); A(cross, h->max_cross); A(coarse, 1);
+    A(cc_parent, n); A(cc_size, n); A(cc_cand, gfm::kMaxCandidates); A(cc_counters, 1);
+    A(coarse, 1);
 #undef A
     if (e != cudaSuccess)
         return fail(h, e == cudaErrorMemoryAllocation ? GFM_ERR_NOMEM : GFM_ERR_CUDA,
@@ -718,8 +705,6 @@ gfm_status alloc_upload(gfm_ctx *h, cudaStream_t s)
     double *zero_d[] = {h->b, h->diag, h->dinv, h->x64, h->r64, h->p64, h->q64, h->rhs};
     for (double *zp : zero_d)
         if (e == cudaSuccess) e = cudaMemsetAsync(zp, 0, sizeof(double) * np, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->comp, 0xff, np, s);  // -1: no coarse region
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->coarse, 0, sizeof(gfm::Coarse), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->UP0, 0, sizeof(float2) * np, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->UP1, 0, sizeof(float2) * np, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->Q0, 0, sizeof(float4) * np, s);
@@ -943,31 +928,20 @@ gfm::CoarseArgs coarse_args(gfm_ctx *h)
     gfm::CoarseArgs co{};
     co.n = h->n;
     co.F = h->F;
-    co.n_pad = h->ht.n_pad;
     co.owner = h->owner;
     co.neighbour = h->neighbour;
-    co.perm = h->perm;
     co.kind = h->kind;
-    co.gamma = h->gamma;
     co.ref = h->ref_internal;
     co.max_k = h->asm_max;
     co.min_size = h->asm_min_size;
-    co.max_cross = h->max_cross;
-    co.prm = h->prm;
     co.parent = h->cc_parent;
     co.csize = h->cc_size;
     co.cand = h->cc_cand;
     co.counters = h->cc_counters;
-    co.bcount = h->cc_bcount;
-    co.boff = h->cc_boff;
-    co.epart = h->cc_epart;
-    co.comp = h->comp;
-    co.cross = h->cross;
     co.coarse = h->coarse;
-    if (h->batched) {  // one coarse space per tank
+    if (h->batched) {  // counted per tank
         co.T = h->T;
         co.coff = h->tcoff;
-        co.ioff = h->tioff;
         co.tprm = h->tprm;
         co.tco = h->tco;
         co.max_k = std::min(h->asm_max, gfm::kTankCoarse);
@@ -1280,9 +1254,8 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
     // c_f / rho of the phase, i.e. without a face Rhie-Chow coefficient
     const bool use_ct = h->ct_ok && !h->rau_set;
     // A pinned system is preconditioned by multigrid, whose coarse levels
-    // follow from gamma; the one-phase regions are then only reported
-    // (gfm_get_coarse finds them).  Unpinned systems and gfm_set_coarse(0)
-    // take the Jacobi forms, the only ones that read the compact table.
+    // follow from gamma.  Unpinned systems and gfm_set_coarse(0) take the
+    // Jacobi forms, the only ones that read the compact table.
     const bool use_mg = h->ref_internal >= 0 && h->coarse_max > 0;
     int launched = 2;
     if (use_ct && !use_mg) {
@@ -1361,8 +1334,6 @@ gfm_status gfm_assemble(gfm_handle h, const double *alpha, const double *phi, co
             }
         }
         h->mg_valid = true;
-    } else {
-        GFM_CUDA(h, gfm::launch_coarse(coarse_args(h), s, &launched));
     }
     if (h->ref_internal < 0) {  // only an unpinned system needs sum(b) for its compatibility test
         GFM_CUDA(h, gfm::launch_bsums(h->b, h->n, h->prm, s));
@@ -1920,10 +1891,16 @@ gfm_status gfm_set_coarse(gfm_handle h, int32_t max_vectors, int32_t min_size)
 gfm_status gfm_get_coarse(gfm_handle h, int32_t *n_vectors, int32_t *n_regions, int32_t *sizes, gfm_stream stream)
 {
     if (!h) return GFM_ERR_ARG;
-    gfm::Coarse co;
+    gfm::Coarse co{};
     cudaStream_t s = (cudaStream_t)stream;
-    // a multigrid solve does not need the regions: find those of the last assembly
-    if (h->mg_valid) GFM_CUDA(h, gfm::launch_coarse(coarse_args(h), s, nullptr));
+    if (!h->assembled) {
+        if (n_vectors) *n_vectors = 0;
+        if (n_regions) *n_regions = 0;
+        if (sizes) std::fill_n(sizes, gfm::kMaxCoarse, 0);
+        return GFM_OK;
+    }
+    // no solver needs the regions: find those of the last assembly
+    GFM_CUDA(h, gfm::launch_coarse(coarse_args(h), s));
     GFM_CUDA(h, cudaMemcpyAsync(&co, h->coarse, sizeof co, cudaMemcpyDeviceToHost, s));
     if (h->batched) {  // vectors summed over the tanks; sizes of the first tanks' vectors
         std::vector<gfm::TankCoarse> tc((size_t)h->T);

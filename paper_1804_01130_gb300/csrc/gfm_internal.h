@@ -10,11 +10,10 @@
 namespace gfm {
 
 constexpr int kSlice = 32;  // cells per sliced-ELL slice (one warp, one lane per cell)
-constexpr int kMaxCoarse = 8;         // coarse vectors of the two-level preconditioner
-constexpr int kMaxCandidates = 4096;  // components examined when choosing them
+constexpr int kMaxCoarse = 8;         // one-phase regions gfm_get_coarse lists
+constexpr int kMaxCandidates = 4096;  // regions examined when choosing them
 constexpr int kMaxTanks = 128;        // tanks of one batched solve
 constexpr int kMaxStages = 4;         // shared-memory stages of streamed slice tables
-constexpr int kCoarseEParts = 128;    // blocks summing E = Z^T A Z
 
 // Physics of one tank of a batch (device copy of gfm_phys, ref internal).
 struct TankPhys {
@@ -24,45 +23,21 @@ struct TankPhys {
     int32_t pad;
 };
 
-// Two-level preconditioner data, rebuilt by every assembly.  The coarse space
-// is spanned by the indicator vectors of the largest connected regions of one
-// phase (cells joined by non-interface faces); E = Z^T A Z and its inverse.
-// Faces whose two cells lie in different coarse regions (or one in none) are
-// listed so that Z^T (A v) can be formed from them exactly.
+// The connected one-phase regions of an assembled system (cells joined by
+// non-interface faces) as gfm_get_coarse reports them.
 struct Coarse {
-    int32_t K;       // coarse vectors in use (0 = Jacobi only)
+    int32_t K;       // regions counted, the largest
     int32_t n_cand;  // regions of at least min_size cells
-    int32_t n_cross; // listed cross faces
-    int32_t ref_comp;  // coarse region of the pinned cell, -1 = none
-    int32_t roots[kMaxCoarse];
     int32_t sizes[kMaxCoarse];
-    double E[kMaxCoarse * kMaxCoarse];
-    double Einv[kMaxCoarse * kMaxCoarse];
 };
-
-// Coarse space of one tank of a batch: its up-to-kTankCoarse largest
-// one-phase regions (typically the water body and the air above it), E =
-// Z^T A Z of those regions and its inverse, and the tank's stretch
-// [x0, x1) of the face-ordered cross-face list.
-constexpr int kTankCoarse = 2;
-constexpr int kMaxReduce = 16;  // most values one grid all-reduce of a single mesh sums
-constexpr int kBatchNR = 3 + kTankCoarse;  // most values one batched all-reduce sums
-constexpr int kLaneSum = 8;                // tanks with more CTAs are summed by a warp
+constexpr int kTankCoarse = 2;  // most regions counted per tank of a batch
 struct TankCoarse {
-    int32_t K, ref_comp, x0, x1;
-    int32_t roots[kTankCoarse], sizes[kTankCoarse];
-    double E[kTankCoarse * kTankCoarse];
-    double Einv[kTankCoarse * kTankCoarse];
+    int32_t K;
+    int32_t sizes[kTankCoarse];
 };
-
-// One face between two coarse regions: internal cell indices, coefficient,
-// and the regions (a of cell o, b of cell v; -1 = not in a coarse region).
-struct CrossFace {
-    int32_t o, v;
-    int8_t a, b;
-    float g32;
-    double g64;
-};
+constexpr int kMaxReduce = 5;   // most values one grid all-reduce of a single mesh sums
+constexpr int kBatchNR = 3;     // most values one batched all-reduce sums
+constexpr int kLaneSum = 8;     // tanks with more CTAs are summed by a warp
 
 // Written on the device by the assembly, read by the solver kernels, so that
 // assembling and solving need no host round trip.
@@ -113,16 +88,13 @@ struct SolveArgs {
     float2 *UP0, *UP1;     // MIXED: (u, p) pairs, double-buffered (gathered)
     float *R32, *S32, *E;  // MIXED: scaled residual, s = A p, FP32 correction
     float *P32;            // MIXED: this iteration's direction p (written whole, read by the update pass)
-    float4 *Q0, *Q1;       // MIXED, fused form: (q, t, p, region) per cell, double-buffered (gathered)
+    float4 *Q0, *Q1;       // MIXED, fused form: (q, t, p, 0) per cell, double-buffered (gathered)
     const float *dinv32;   // MIXED: 1 / (float)diag
     const int32_t *iperm;  // [n] internal -> caller index
     double *p_user;        // caller-order x0 in / solution out
     double rtol, inner_rtol;
     int32_t max_iters, max_refine, use_x0;
     unsigned long long budget_ns;
-    const Coarse *coarse;  // two-level preconditioner (K = 0: Jacobi only)
-    const int8_t *comp;    // [n_pad] coarse region of each internal cell, -1 none
-    const CrossFace *cross;  // [coarse->n_cross]
     const int32_t *n_per_tank;  // batched: real cells of each tank (else nullptr)
     int32_t cache_cap;     // slots of a CTA's slice tables staged in shared memory
     int32_t meta_slots;    // slice-metadata entries reserved in shared memory
@@ -210,27 +182,20 @@ cudaError_t launch_dict(const DictArgs &a, cudaStream_t s);
 cudaError_t launch_bsums(const double *b, int32_t n, DevParams *prm, cudaStream_t s);
 
 struct CoarseArgs {
-    int32_t n, F, n_pad;
-    const int32_t *owner, *neighbour, *perm;
+    int32_t n, F;
+    const int32_t *owner, *neighbour;
     const int8_t *kind;
-    const double *gamma;
     int32_t ref;  // internal index of the pinned cell, -1 none
-    int32_t max_k, min_size, max_cross;
-    const DevParams *prm;
-    int32_t *parent, *csize, *cand, *counters;  // counters[0] = candidates, [1] = cross faces
-    int32_t *bcount, *boff;  // [ceil(F / 256)] cross faces per face block, and their offsets
-    double *epart;           // [kCoarseEParts][kMaxCoarse^2] partial sums of E
-    int8_t *comp;  // internal order
-    CrossFace *cross;
+    int32_t max_k, min_size;
+    int32_t *parent, *csize, *cand, *counters;  // counters[0] = candidates
     Coarse *coarse;
-    // batched handles (T > 0): coarse regions are chosen per tank (region ids
-    // in comp are tank-local)
+    // batched handles (T > 0): regions are counted per tank
     int32_t T;
-    const int32_t *coff, *ioff;  // [T+1] caller / internal cell offsets of the tanks
-    const DevParams *tprm;       // [T] pinned cell and pin of each tank
+    const int32_t *coff;         // [T+1] caller cell offsets of the tanks
+    const DevParams *tprm;       // [T] pinned cell of each tank
     TankCoarse *tco;             // [T]
 };
-cudaError_t launch_coarse(const CoarseArgs &a, cudaStream_t s, int *launches);
+cudaError_t launch_coarse(const CoarseArgs &a, cudaStream_t s);
 
 cudaError_t launch_corrected_flux(int32_t F, const int32_t *owner, const int32_t *neighbour, const double *gamma,
                                   const double *jump, const double *phi, const double *p, double *out,
@@ -320,7 +285,6 @@ struct BatchArgs {
     const int2 *tank_cta;
     const DevParams *tprm;
     gfm_solve_info *infos;  // [T]
-    const TankCoarse *tco;  // [T] coarse space of each tank
 };
 const void *batched_kernel(int max_width, bool streamed = false, bool compact = false);
 

@@ -68,18 +68,6 @@ struct Shared {
     double warp_d[32][kMaxNR];
     double out[kMaxNR];
     Ctl ctl;
-    double y[kMaxCoarse];    // thread 0: Z^T r (coarse components of the residual)
-    double c64[kMaxCoarse];  // coarse correction E^{-1} Z^T r, broadcast
-    float c32[kMaxCoarse];
-    float cz[kMaxCoarse + 1];  // fused form: 0, then the FP32 coarse correction of each region
-    float zb32[kMaxCoarse];  // this CTA's Z^T (A p) in a pass
-    double zb64[kMaxCoarse];
-    float zbw32[16][kMaxCoarse];  // the same per warp, summed in warp order
-    double zbw64[16][kMaxCoarse];
-    float zpin32;  // the pinned cell's share, when this CTA holds it
-    double zpin64;
-    double Einv[kMaxCoarse * kMaxCoarse];  // staged copy of the coarse inverse
-    float Einv32[kMaxCoarse * kMaxCoarse];  // the same in FP32 (the FP32 iterations' coarse correction)
     int flag;
     int flag2;  // a reduction's error check, published with its sums
     int ring_fail;  // a streamed-table stage did not arrive within the budget
@@ -756,133 +744,10 @@ __device__ void record_abort(const SolveArgs &a)
 
 enum Action : int { kGo = 0, kConverged = 1, kCheck = 2, kNotConverged = 3, kBreakdown = 4, kUpdate = 5, kRestart = 6 };
 
-// Warp 0, all lanes: c = E^{-1} y (y in shared memory), lane i forming row
-// i, published in shared memory in FP64 and FP32.  An FP64 instruction takes
-// the same pipe time on GB300 whether one lane or 32 are active, so rows in
-// parallel cost K instructions where one thread doing all of them cost K^2.
-__device__ __forceinline__ void coarse_solve_warp(int K, Shared &sh)
-{
-    __syncwarp();
-    const int i = threadIdx.x & 31;
-    if (i < K) {
-        double t = 0.0;
-#pragma unroll
-        for (int j = 0; j < kMaxCoarse; ++j)
-            if (j < K) t = fma(sh.Einv[i * kMaxCoarse + j], sh.y[j], t);
-        sh.c64[i] = t;
-        sh.c32[i] = (float)t;
-    }
-    __syncwarp();
-}
-
-// Copy E^{-1} into shared memory once per solve.
-__device__ __forceinline__ void stage_coarse(const Coarse *co, Shared &sh)
-{
-    for (int q = threadIdx.x; q < kMaxCoarse * kMaxCoarse; q += blockDim.x) {
-        sh.Einv[q] = co->Einv[q];
-        sh.Einv32[q] = (float)co->Einv[q];
-    }
-}
-
-// One warp, all lanes: lane k < K returns c_k = sum_j E^{-1}_kj y_j in FP32,
-// y_j taken from lane j's y (lanes >= K return 0).  The FP32 iterations only
-// need the correction in FP32, and on GB300 a chain of K dependent FP64
-// multiply-adds costs several times this shuffle-and-FMA form.
-__device__ __forceinline__ float coarse32_lane(int K, double y_lane, const Shared &sh)
-{
-    const int k = threadIdx.x & 31;
-    const float yl = (float)y_lane;
-    float c = 0.0f;
-#pragma unroll
-    for (int j = 0; j < kMaxCoarse; ++j) {
-        const float yj = __shfl_sync(0xffffffffu, yl, j);
-        if (j < K && k < K) c = fmaf(sh.Einv32[k * kMaxCoarse + j], yj, c);
-    }
-    return c;
-}
-
-__device__ __forceinline__ void zero_bins(Shared &sh)
-{
-    if (threadIdx.x < kMaxCoarse) {
-        sh.zb32[threadIdx.x] = 0.0f;
-        sh.zb64[threadIdx.x] = 0.0;
-    }
-    if (threadIdx.x == 0) {
-        sh.zpin32 = 0.0f;
-        sh.zpin64 = 0.0;
-    }
-}
-
-// Z^T (A p) over this CTA's share of the faces between coarse regions:
-// val(face) = gamma_f (p_own - p_nb) is added to the owner's region and
-// subtracted from the neighbour's.  Sums stay in registers per thread (one
-// per region), then per warp into wbins[warp], which finish_bins adds in
-// warp order: the same result at every run, and no shared-memory atomics
-// serialised on the two words of the water/air region pair.
-template <typename T, typename ValFn>
-__device__ __forceinline__ void cross_sums_range(const CrossFace *cross, int f0, int f1, int K,
-                                                 T (*wbins)[kMaxCoarse], ValFn val)
-{
-    T acc[kMaxCoarse];
-#pragma unroll
-    for (int k = 0; k < kMaxCoarse; ++k) acc[k] = T(0);
-    // taken by the CTA's last threads first, whose warps hold the fewest slices
-    const int t0 = f0 + (int)(blockDim.x - 1 - threadIdx.x);
-    for (int t = t0; t < f1; t += blockDim.x) {
-        const CrossFace cf = cross[t];
-        const T v = val(cf);
-        if constexpr (sizeof(T) == 4) {
-            // FP32: selects are cheaper than a local-memory bin
-#pragma unroll
-            for (int k = 0; k < kMaxCoarse; ++k) acc[k] += (cf.a == k ? v : T(0)) - (cf.b == k ? v : T(0));
-        } else {
-            // FP64: two adds into a (local-memory) bin instead of 16 FP64 selects and adds
-            if (cf.a >= 0) acc[cf.a] += v;
-            if (cf.b >= 0) acc[cf.b] -= v;
-        }
-    }
-    const bool any = __any_sync(0xffffffffu, t0 < f1);  // a warp without faces adds nothing
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < kMaxCoarse; ++k) {
-        if (k >= K) break;  // K is the same in every thread
-        T x = acc[k];
-        if (any) {
-#pragma unroll
-            for (int off = 16; off; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-        }
-        if (lane == 0) wbins[warp][k] = any ? x : T(0);
-    }
-}
-
-// The CTA's even share of all n_cross cross faces.
-template <typename T, typename ValFn>
-__device__ __forceinline__ void cross_sums(const CrossFace *cross, int n_cross, int K, T (*wbins)[kMaxCoarse],
-                                           ValFn val)
-{
-    const int f0 = (int)(((long long)n_cross * blockIdx.x) / gridDim.x);
-    const int f1 = (int)(((long long)n_cross * (blockIdx.x + 1)) / gridDim.x);
-    cross_sums_range<T>(cross, f0, f1, K, wbins, val);
-}
-
-// Warp 0, after a CTA barrier that follows cross_sums: bins[k] = the warps'
-// sums in warp order plus the pinned cell's share.
-template <typename T>
-__device__ __forceinline__ void finish_bins(const T (*wbins)[kMaxCoarse], T pin, int rc, int K, int nw, T *bins)
-{
-    const int k = threadIdx.x & 31;
-    if (k < K) {
-        T x = (k == rc) ? pin : T(0);
-        for (int w = 0; w < nw; ++w) x += wbins[w][k];
-        bins[k] = x;
-    }
-    __syncwarp();
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// FP64 Jacobi(+coarse)-PCG
+// FP64 Jacobi-PCG
 // ---------------------------------------------------------------------------
 template <int CH>
 __global__ void __launch_bounds__(512, 1) k_solve_fp64(SolveArgs a)
@@ -894,23 +759,17 @@ __global__ void __launch_bounds__(512, 1) k_solve_fp64(SolveArgs a)
     extern __shared__ __align__(16) unsigned char dsm[];
     Grid g{a.bar, a.err, a.partials, a.budget_ns, 0u, (int)gridDim.x, 0};
     const Range R = my_range(a.m.n_slices);
-    stage_coarse(a.coarse, sh);
     const Tab<double> tab = stage_tables<double>(a.m, a.m.val64, R, a.cache_cap, a.meta_slots, dsm);
     const int n = a.m.n;
     const int ref = a.prm->ref;
-    const int K = a.coarse->K;
-    const int rc = a.coarse->ref_comp;
     const double pin64 = a.prm->pin64;
-    const int nx = a.coarse->n_cross;
     double *x = a.x64;  // gathered by the true-residual pass
     double *__restrict__ r = a.r64;
     double *p = a.p64;  // gathered by the SpMV: read by other CTAs, no nc loads
     double *__restrict__ q = a.q64;
     const double *__restrict__ dinv = a.dinv64;
-    const int8_t *__restrict__ comp = a.comp;
-    // thread-0 scalar state (rr_ref: ||r||^2 when Z^T r was last summed exactly;
-    // best: smallest true relative residual seen at a check)
-    double bnorm = 1.0, rz = 0.0, rr_ref = 0.0, best = 1e300;
+    // thread-0 scalar state (best: smallest true relative residual seen at a check)
+    double bnorm = 1.0, rz = 0.0, best = 1e300;
     int checks = 0, stall = 0;
 
     if (a.use_x0) {
@@ -920,13 +779,9 @@ __global__ void __launch_bounds__(512, 1) k_solve_fp64(SolveArgs a)
         }
         if (!grid_sync(g, sh)) { record_abort(a); return; }
     }
-    // r = b - A x, p = z = M^{-1} r; with a coarse space the Jacobi part is
-    // written first and the coarse part added once Z^T r is known.
+    // r = b - A x, p = z = D^{-1} r
     {
         double v3[3] = {0.0, 0.0, 0.0};  // b.b, r.r, r.(D^{-1} r)
-        double zb[kMaxCoarse];
-#pragma unroll
-        for (int k = 0; k < kMaxCoarse; ++k) zb[k] = 0.0;
         for (int s = R.s0 + R.warp; s < R.s1; s += R.nw) {
             const int i = s * kSlice + R.lane;
             if (i < n) {
@@ -940,51 +795,24 @@ __global__ void __launch_bounds__(512, 1) k_solve_fp64(SolveArgs a)
                 v3[0] += bi * bi;
                 v3[1] += ri * ri;
                 v3[2] += ri * zi;
-                if (K > 0) {
-                    const int cm = comp[i];
-#pragma unroll
-                    for (int k = 0; k < kMaxCoarse; ++k) zb[k] += (cm == k) ? ri : 0.0;
-                }
             }
         }
         block_sum_f64<3>(sh, v3);
-        block_sum_f64<kMaxCoarse>(sh, zb);
-        double t3[3 + kMaxCoarse];
-        {
-            double blk[3 + kMaxCoarse];
-            blk[0] = v3[0]; blk[1] = v3[1]; blk[2] = v3[2];
-            for (int k = 0; k < kMaxCoarse; ++k) blk[3 + k] = zb[k];
-            if (!grid_allreduce<3 + kMaxCoarse>(g, sh, blk, t3, 3 + K)) { record_abort(a); return; }
-        }
-        if (threadIdx.x < 32) {
-            if (threadIdx.x == 0) {
-                bnorm = (t3[0] > 0.0) ? sqrt(t3[0]) : 1.0;
-                rz = t3[2];
-                rr_ref = t3[1];
-                for (int k = 0; k < K; ++k) sh.y[k] = t3[3 + k];
-            }
-            coarse_solve_warp(K, sh);
-            if (threadIdx.x == 0) {
-                for (int k = 0; k < K; ++k) rz = fma(sh.c64[k], sh.y[k], rz);
-                sh.ctl.action = (sqrt(t3[1]) / bnorm <= a.rtol) ? kConverged : kGo;
-            }
+        double t3[3];
+        if (!grid_allreduce<3>(g, sh, v3, t3)) { record_abort(a); return; }
+        if (threadIdx.x == 0) {
+            bnorm = (t3[0] > 0.0) ? sqrt(t3[0]) : 1.0;
+            rz = t3[2];
+            sh.ctl.action = (sqrt(t3[1]) / bnorm <= a.rtol) ? kConverged : kGo;
         }
         __syncthreads();
-        if (K > 0) {
-            for (int s = R.s0 + R.warp; s < R.s1; s += R.nw) {
-                const int i = s * kSlice + R.lane;
-                if (i < n && comp[i] >= 0) p[i] += sh.c64[comp[i]];
-            }
-        }
     }
     int action = sh.ctl.action;
     int iters = 0, status = GFM_OK;
     while (action != kConverged) {
         if (iters >= a.max_iters) { status = GFM_ERR_NOT_CONVERGED; break; }
         if (!grid_sync(g, sh)) { record_abort(a); return; }  // p complete
-        zero_bins(sh);
-        __syncthreads();
-        // pass 1: q = A p, p.q; Z^T q from the faces between coarse regions
+        // pass 1: q = A p, p.q
         double v1[1] = {0.0};
         for (int sb = R.s0 + R.warp; sb < R.s1; sb += U * R.nw) {
             int ii[U], base[U], w[U];
@@ -1032,40 +860,23 @@ __global__ void __launch_bounds__(512, 1) k_solve_fp64(SolveArgs a)
                 if (sb + u * R.nw < R.s1 && ii[u] < n) {
                     q[ii[u]] = acc[u];
                     v1[0] = fma(pi[u], acc[u], v1[0]);
-                    if (ii[u] == ref && rc >= 0 && K > 0) sh.zpin64 = pin64 * pi[u];  // pin term of Z^T A p
                 }
             }
         }
-        if (K > 0)  // each CTA takes an even share of the cross faces
-            cross_sums<double>(a.cross, nx, K, sh.zbw64,
-                               [&](const CrossFace &cf) { return cf.g64 * (p[cf.o] - p[cf.v]); });
         block_sum_f64<1>(sh, v1);
-        if (K > 0 && threadIdx.x < 32) finish_bins<double>(sh.zbw64, sh.zpin64, rc, K, R.nw, sh.zb64);
-        double t1[1 + kMaxCoarse];
-        {
-            double blk[1 + kMaxCoarse];
-            blk[0] = v1[0];
-            for (int k = 0; k < kMaxCoarse; ++k) blk[1 + k] = sh.zb64[k];
-            if (K > 0) {
-                if (!grid_allreduce<1 + kMaxCoarse>(g, sh, blk, t1, 1 + K)) { record_abort(a); return; }
-            } else {
-                double b1[1] = {blk[0]}, o1[1];
-                if (!grid_allreduce<1>(g, sh, b1, o1)) { record_abort(a); return; }
-                t1[0] = o1[0];
-            }
-        }
+        double t1[1];
+        if (!grid_allreduce<1>(g, sh, v1, t1)) { record_abort(a); return; }
         if (threadIdx.x == 0) {
             const double pq = t1[0];
             const bool ok = pq > 0.0 && isfinite(pq);
             const double alpha = ok ? rz / pq : 0.0;
             sh.ctl.alpha = alpha;
             sh.ctl.action = ok ? kGo : kBreakdown;
-            for (int k = 0; k < K; ++k) sh.y[k] = fma(-alpha, t1[1 + k], sh.y[k]);
         }
         __syncthreads();
         if (sh.ctl.action == kBreakdown) { status = GFM_ERR_BREAKDOWN; break; }
         const double alpha = sh.ctl.alpha;
-        // pass 2: x += alpha p, r -= alpha q, z = M^{-1} r; r.z, r.r
+        // pass 2: x += alpha p, r -= alpha q, z = D^{-1} r; r.z, r.r
         double v2[2] = {0.0, 0.0};
         for (int s = R.s0 + R.warp; s < R.s1; s += R.nw) {
             const int i = s * kSlice + R.lane;
@@ -1073,7 +884,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_fp64(SolveArgs a)
                 x[i] = fma(alpha, p[i], x[i]);
                 const double ri = fma(-alpha, q[i], r[i]);
                 r[i] = ri;
-                v2[0] = fma(ri, dinv[i] * ri, v2[0]);  // r.(D^{-1} r); the coarse part is added below
+                v2[0] = fma(ri, dinv[i] * ri, v2[0]);  // r.(D^{-1} r)
                 v2[1] = fma(ri, ri, v2[1]);
             }
         }
@@ -1081,72 +892,21 @@ __global__ void __launch_bounds__(512, 1) k_solve_fp64(SolveArgs a)
         double t2[2];
         if (!grid_allreduce<2>(g, sh, v2, t2)) { record_abort(a); return; }
         ++iters;
-        if (threadIdx.x < 32) {
-            if (threadIdx.x == 0) {
-                if (sqrt(t2[1]) / bnorm <= a.rtol) {
-                    sh.ctl.action = kCheck;
-                } else if (K > 0 && t2[1] <= 1e-2 * rr_ref) {
-                    // the residual fell a decade since Z^T r was last summed:
-                    // sum it exactly again so the recurrence cannot drift
-                    sh.ctl.xavg = t2[0];
-                    rr_ref = t2[1];
-                    sh.ctl.action = kUpdate;
-                } else {
-                    sh.ctl.action = kGo;
-                }
-            }
-            __syncwarp();
-            if (sh.ctl.action == kGo) {
-                // z = D^{-1} r + Z E^{-1} y:  r.z = r.D^{-1}r + y.E^{-1}y
-                coarse_solve_warp(K, sh);
-                if (threadIdx.x == 0) {
-                    double rzn = t2[0];
-                    for (int k = 0; k < K; ++k) rzn = fma(sh.c64[k], sh.y[k], rzn);
-                    sh.ctl.beta = rzn / rz;
-                    rz = rzn;
-                }
+        if (threadIdx.x == 0) {
+            if (sqrt(t2[1]) / bnorm <= a.rtol) {
+                sh.ctl.action = kCheck;
+            } else {
+                sh.ctl.action = kGo;
+                sh.ctl.beta = t2[0] / rz;
+                rz = t2[0];
             }
         }
         __syncthreads();
         action = sh.ctl.action;
-        if (action == kUpdate) {
-            double zb[kMaxCoarse];
-#pragma unroll
-            for (int k = 0; k < kMaxCoarse; ++k) zb[k] = 0.0;
-            for (int s = R.s0 + R.warp; s < R.s1; s += R.nw) {
-                const int i = s * kSlice + R.lane;
-                if (i < n) {
-                    const int cm = comp[i];
-                    const double ri = r[i];
-#pragma unroll
-                    for (int k = 0; k < kMaxCoarse; ++k) zb[k] += (cm == k) ? ri : 0.0;
-                }
-            }
-            block_sum_f64<kMaxCoarse>(sh, zb);
-            double ty[kMaxCoarse];
-            if (!grid_allreduce<kMaxCoarse>(g, sh, zb, ty, K)) { record_abort(a); return; }
-            if (threadIdx.x < 32) {
-                if (threadIdx.x == 0)
-                    for (int k = 0; k < K; ++k) sh.y[k] = ty[k];
-                coarse_solve_warp(K, sh);
-                if (threadIdx.x == 0) {
-                    double rzn = sh.ctl.xavg;
-                    for (int k = 0; k < K; ++k) rzn = fma(sh.c64[k], sh.y[k], rzn);
-                    sh.ctl.beta = rzn / rz;
-                    rz = rzn;
-                    sh.ctl.action = kGo;
-                }
-            }
-            __syncthreads();
-            action = sh.ctl.action;
-        }
         if (action == kCheck) {
             // confirm with the true residual; restart from it on a miss
             if (!grid_sync(g, sh)) { record_abort(a); return; }  // x complete
             double vt[2] = {0.0, 0.0};
-            double zb[kMaxCoarse];
-#pragma unroll
-            for (int k = 0; k < kMaxCoarse; ++k) zb[k] = 0.0;
             for (int s = R.s0 + R.warp; s < R.s1; s += R.nw) {
                 const int i = s * kSlice + R.lane;
                 if (i < n) {
@@ -1159,33 +919,14 @@ __global__ void __launch_bounds__(512, 1) k_solve_fp64(SolveArgs a)
                     p[i] = zi;
                     vt[0] += ri * zi;
                     vt[1] += ri * ri;
-                    if (K > 0) {
-                        const int cm = comp[i];
-#pragma unroll
-                        for (int k = 0; k < kMaxCoarse; ++k) zb[k] += (cm == k) ? ri : 0.0;
-                    }
                 }
             }
             block_sum_f64<2>(sh, vt);
-            block_sum_f64<kMaxCoarse>(sh, zb);
-            double tt[2 + kMaxCoarse];
-            {
-                double blk[2 + kMaxCoarse];
-                blk[0] = vt[0]; blk[1] = vt[1];
-                for (int k = 0; k < kMaxCoarse; ++k) blk[2 + k] = zb[k];
-                if (!grid_allreduce<2 + kMaxCoarse>(g, sh, blk, tt, 2 + K)) { record_abort(a); return; }
-            }
-            if (threadIdx.x < 32) {
-                if (threadIdx.x == 0) {
-                    ++checks;
-                    rz = tt[0];
-                    rr_ref = tt[1];
-                    for (int k = 0; k < K; ++k) sh.y[k] = tt[2 + k];
-                }
-                coarse_solve_warp(K, sh);
-            }
+            double tt[2];
+            if (!grid_allreduce<2>(g, sh, vt, tt)) { record_abort(a); return; }
             if (threadIdx.x == 0) {
-                for (int k = 0; k < K; ++k) rz = fma(sh.c64[k], sh.y[k], rz);
+                ++checks;
+                rz = tt[0];
                 const double rel = sqrt(tt[1]) / bnorm;
                 if (rel < 0.5 * best) { best = rel; stall = 0; }
                 else ++stall;
@@ -1195,12 +936,6 @@ __global__ void __launch_bounds__(512, 1) k_solve_fp64(SolveArgs a)
             __syncthreads();
             action = sh.ctl.action;
             if (action == kNotConverged) { status = GFM_ERR_NOT_CONVERGED; break; }
-            if (action == kGo && K > 0) {
-                for (int s = R.s0 + R.warp; s < R.s1; s += R.nw) {
-                    const int i = s * kSlice + R.lane;
-                    if (i < n && comp[i] >= 0) p[i] += sh.c64[comp[i]];
-                }
-            }
             continue;
         }
         const double beta = sh.ctl.beta;
@@ -1208,9 +943,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_fp64(SolveArgs a)
         for (int s = R.s0 + R.warp; s < R.s1; s += R.nw) {
             const int i = s * kSlice + R.lane;
             if (i < n) {
-                double zi = dinv[i] * r[i];
-                if (K > 0 && comp[i] >= 0) zi += sh.c64[comp[i]];
-                p[i] = fma(beta, p[i], zi);
+                p[i] = fma(beta, p[i], dinv[i] * r[i]);
             }
         }
     }
@@ -1226,17 +959,14 @@ namespace {
 
 // Residual replacement.  When `fold`, first x += e / sc in FP64 (e = 0).
 // Then r = b - A x in FP64 (difference form), r32 = (float)(r sc) and the
-// preconditioned residual u = r32 / D + (Z E^{-1} Z^T r32) into up.x; with
-// `zero_p` the kept direction up.y is cleared.  Thread 0 gets
-// t = (||r||^2 in FP64, r32.u, r32.r32) and sh.y = Z^T r32.
+// preconditioned residual u = r32 / D into up.x; with `zero_p` the kept
+// direction up.y is cleared.  Thread 0 gets t = (||r||^2 in FP64, r32.u, r32.r32).
 template <int CH>
 __device__ __noinline__ bool replace_residual(const SolveArgs &a, Grid &g, Shared &sh, const Range &R, float2 *up,
-                                              double sc, double isc, bool fold, bool zero_p, double (&t)[3],
-                                              double &y_lane)
+                                              double sc, double isc, bool fold, bool zero_p, double (&t)[3])
 {
     const int n = a.m.n;
     const int ref = a.prm->ref;
-    const int K = a.coarse->K;
     const double pin64 = a.prm->pin64;
     double *x = a.x64;
     if (fold) {
@@ -1250,8 +980,7 @@ __device__ __noinline__ bool replace_residual(const SolveArgs &a, Grid &g, Share
         if (!grid_sync(g, sh)) return false;  // x complete
     }
     double vr[1] = {0.0};
-    FF acc[2 + kMaxCoarse];
-    for (int k = 0; k < 2 + kMaxCoarse; ++k) acc[k] = FF{0.f, 0.f};
+    FF acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
     for (int s = R.s0 + R.warp; s < R.s1; s += R.nw) {
         const int i = s * kSlice + R.lane;
         if (i < n) {
@@ -1265,58 +994,30 @@ __device__ __noinline__ bool replace_residual(const SolveArgs &a, Grid &g, Share
             else up[i].x = u;
             ff_add(acc[0], r32 * u);
             ff_add(acc[1], r32 * r32);
-            const int cm = a.comp[i];
-#pragma unroll
-            for (int k = 0; k < kMaxCoarse; ++k) ff_add(acc[2 + k], (cm == k) ? r32 : 0.0f);
         }
     }
     block_sum_f64<1>(sh, vr);
-    double ffo[2 + kMaxCoarse];
-    block_sum_ff<2 + kMaxCoarse>(sh, acc, ffo);
-    double blk[3 + kMaxCoarse], tt[3 + kMaxCoarse];
-    blk[0] = vr[0];
-    for (int k = 0; k < 2 + kMaxCoarse; ++k) blk[1 + k] = ffo[k];
-    if (!grid_allreduce<3 + kMaxCoarse>(g, sh, blk, tt, 3 + K)) return false;
-    if (threadIdx.x < 32) {
-        if (threadIdx.x == 0)
-            for (int k = 0; k < K; ++k) sh.y[k] = tt[3 + k];
-        coarse_solve_warp(K, sh);  // c in FP64, for r.u below
-        // warp 0's register copy of y, and the FP32 correction the FP32
-        // iterations apply (the same form as in every iteration)
-        y_lane = (R.lane < K) ? tt[3 + R.lane] : 0.0;
-        const float c = coarse32_lane(K, y_lane, sh);
-        if (R.lane < K) sh.c32[R.lane] = c;
-    }
-    if (threadIdx.x == 0) {
-        double gam = tt[1];
-        for (int k = 0; k < K; ++k) gam = fma(sh.c64[k], sh.y[k], gam);
-        t[0] = tt[0];
-        t[1] = gam;
-        t[2] = tt[2];
-        sh.ctl.gam32 = (float)gam;
-    }
+    double ffo[2];
+    block_sum_ff<2>(sh, acc, ffo);
+    const double blk[3] = {vr[0], ffo[0], ffo[1]};
+    // also the barrier after which the next pass gathers the new u
+    if (!grid_allreduce<3>(g, sh, blk, t)) return false;
+    if (threadIdx.x == 0) sh.ctl.gam32 = (float)t[1];
     __syncthreads();
-    if (K > 0) {
-        for (int s = R.s0 + R.warp; s < R.s1; s += R.nw) {
-            const int i = s * kSlice + R.lane;
-            if (i < n && a.comp[i] >= 0) up[i].x += sh.c32[a.comp[i]];
-        }
-        if (!grid_sync(g, sh)) return false;  // u complete before it is gathered
-    }
     return true;
 }
 
 // One group of the mixed operator pass: slices sb, sb + nw, ... (U of them,
 // those before s_end): p = u + beta p for the cell and, from the gathered
 // (u, p) pairs, for its neighbours; s = A p in difference form; p into P32,
-// s into S32, p.s into acc (and the pin's share of Z^T A p).  The tables are
+// s into S32, p.s into acc.  The tables are
 // in shared memory (cached or a streamed stage): neighbour indices and
 // coefficients are read where they are used, so only the gathered pairs
 // occupy registers and all U x CH gathers of a chunk are in flight at once.
 template <int CH, int U, typename TabT>
 __device__ __forceinline__ void mixed_op_group(const TabT &tab, int sb, int s_end, const Range &R, int n,
                                                const float2 *cur, float *P32, float *S32, float be, int ref,
-                                               float pin32, int rc, int K, Shared &sh, FF &acc)
+                                               float pin32, FF &acc)
 {
     int ii[U], base[U], w[U];
     float2 v[U];
@@ -1374,7 +1075,6 @@ __device__ __forceinline__ void mixed_op_group(const TabT &tab, int sb, int s_en
             __stcs(P32 + ii[u], pn[u]);  // read once, by the update pass
             __stcs(S32 + ii[u], si[u]);
             ff_add(acc, pn[u] * si[u]);
-            if (ii[u] == ref && rc >= 0 && K > 0) sh.zpin32 = pin32 * pn[u];  // pin term of Z^T A p
         }
     }
 }
@@ -1387,7 +1087,7 @@ __device__ __forceinline__ void mixed_op_group(const TabT &tab, int sb, int s_en
 template <int CH, int U, typename TabT>
 __device__ __forceinline__ void mixed_op_group_hoisted(const TabT &tab, int sb, int s_end, const Range &R, int n,
                                                        const float2 *cur, float *P32, float *S32, float be, int ref,
-                                                       float pin32, int rc, int K, Shared &sh, FF &acc)
+                                                       float pin32, FF &acc)
 {
     int ii[U], base[U], w[U];
     float2 v[U];
@@ -1438,7 +1138,6 @@ __device__ __forceinline__ void mixed_op_group_hoisted(const TabT &tab, int sb, 
             __stcs(P32 + ii[u], pn[u]);  // read once, by the update pass
             __stcs(S32 + ii[u], si[u]);
             ff_add(acc, pn[u] * si[u]);
-            if (ii[u] == ref && rc >= 0 && K > 0) sh.zpin32 = pin32 * pn[u];  // pin term of Z^T A p
         }
     }
 }
@@ -1463,7 +1162,6 @@ __global__ void __launch_bounds__(512, 1) k_solve_mixed(SolveArgs a)
     extern __shared__ __align__(16) unsigned char dsm[];
     Grid g{a.bar, a.err, a.partials, a.budget_ns, 0u, (int)gridDim.x, 0};
     const Range R = my_range(a.m.n_slices);
-    stage_coarse(a.coarse, sh);
     const Tab<float> tab = stage_tables<float>(a.m, a.m.val32, R, a.cache_cap, a.meta_slots, dsm);
     Ring ring{};
     if constexpr (STREAM) ring = make_ring(a, R, tab.meta, dsm, sh, CT);
@@ -1476,15 +1174,11 @@ __global__ void __launch_bounds__(512, 1) k_solve_mixed(SolveArgs a)
     const int n = a.m.n;
     const int ref = a.prm->ref;
     const float pin32 = a.prm->pin32;
-    const int K = a.coarse->K;
-    const int rc = a.coarse->ref_comp;
-    const int nx = a.coarse->n_cross;
     float *__restrict__ E = a.E;
     float *__restrict__ R32 = a.R32;
     float *__restrict__ S32 = a.S32;
     float *__restrict__ P32 = a.P32;
     const float *__restrict__ dinv = a.dinv32;
-    const int8_t *__restrict__ comp = a.comp;
 
     // prologue: x0, e = 0, no direction yet, ||b||
     double vb[1] = {0.0};
@@ -1534,8 +1228,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_mixed(SolveArgs a)
     float2 *cur = a.UP0, *nxt = a.UP1;  // cur holds (u, p_old) for the next pass A
     int iters = 0, updates = 0, status = GFM_OK;
     double t[3];
-    double y_lane = 0.0;  // warp 0: Z^T r (lane k: component k)
-    if (!replace_residual<CH>(a, g, sh, R, cur, sc, isc, false, true, t, y_lane)) { bail(); return; }
+    if (!replace_residual<CH>(a, g, sh, R, cur, sc, isc, false, true, t)) { bail(); return; }
     ++updates;
     if (threadIdx.x == 0) {
         best_rel2 = t[0] / (bnorm * bnorm);
@@ -1550,8 +1243,6 @@ __global__ void __launch_bounds__(512, 1) k_solve_mixed(SolveArgs a)
         if (threadIdx.x == 0) ring_prefetch(ring);
     while (action != kConverged) {
         const float be = sh.ctl.be;
-        zero_bins(sh);
-        __syncthreads();
         // pass A: p = u + beta p (own and, redundantly, neighbours), s = A p, p.s
         FF accA[1] = {{0.f, 0.f}};
         if constexpr (STREAM) {
@@ -1562,13 +1253,11 @@ __global__ void __launch_bounds__(512, 1) k_solve_mixed(SolveArgs a)
                     if constexpr (CT) {
                         const StageTabCT st = ring_stage_ct(ring, r);
                         for (int sb = sr0 + R.warp; sb < sr1; sb += US * R.nw)
-                            mixed_op_group<CH, US>(st, sb, sr1, R, n, cur, P32, S32, be, ref, pin32, rc, K, sh,
-                                                   accA[0]);
+                            mixed_op_group<CH, US>(st, sb, sr1, R, n, cur, P32, S32, be, ref, pin32, accA[0]);
                     } else {
                         const StageTab st = ring_stage(ring, r);
                         for (int sb = sr0 + R.warp; sb < sr1; sb += US * R.nw)
-                            mixed_op_group<CH, US>(st, sb, sr1, R, n, cur, P32, S32, be, ref, pin32, rc, K, sh,
-                                                   accA[0]);
+                            mixed_op_group<CH, US>(st, sb, sr1, R, n, cur, P32, S32, be, ref, pin32, accA[0]);
                     }
                 } else {
                     sh.ring_fail = 1;
@@ -1590,57 +1279,26 @@ __global__ void __launch_bounds__(512, 1) k_solve_mixed(SolveArgs a)
             // to global memory, so the group's loads carry no branches
             const StageTab ft{tab.meta, tab.col, tab.val, tab.s0, tab.base0};
             for (int sb = R.s0 + R.warp; sb < R.s1; sb += U * R.nw)
-                mixed_op_group<CH, U>(ft, sb, R.s1, R, n, cur, P32, S32, be, ref, pin32, rc, K, sh, accA[0]);
+                mixed_op_group<CH, U>(ft, sb, R.s1, R, n, cur, P32, S32, be, ref, pin32, accA[0]);
         } else {
             for (int sb = R.s0 + R.warp; sb < R.s1; sb += U * R.nw)
-                mixed_op_group<CH, U>(tab, sb, R.s1, R, n, cur, P32, S32, be, ref, pin32, rc, K, sh, accA[0]);
+                mixed_op_group<CH, U>(tab, sb, R.s1, R, n, cur, P32, S32, be, ref, pin32, accA[0]);
         }
-        if (K > 0)  // Z^T (A p) from the faces between coarse regions (the pin's share is added above)
-            cross_sums<float>(a.cross, nx, K, sh.zbw32, [&](const CrossFace &cf) {
-                const float2 vo = cur[cf.o], vv = cur[cf.v];
-                return cf.g32 * (fmaf(be, vo.y, vo.x) - fmaf(be, vv.y, vv.x));
-            });
-        double tA[1 + kMaxCoarse];
+        double tA[1];
         float2 blkA[1];
         block_sum_ff2<1>(sh, accA, blkA);
-        if (K > 0) {
-            float2 b9[1 + kMaxCoarse];
-            b9[0] = blkA[0];
-            if (threadIdx.x < 32) finish_bins<float>(sh.zbw32, sh.zpin32, rc, K, R.nw, sh.zb32);
-            for (int k = 0; k < kMaxCoarse; ++k) b9[1 + k] = make_float2(sh.zb32[k], 0.0f);
-            if (!grid_allreduce_ff<1 + kMaxCoarse>(g, sh, b9, tA, 1 + K)) { bail(); return; }
-        } else {
-            double o1[1];
-            if (!grid_allreduce_ff<1>(g, sh, blkA, o1)) { bail(); return; }
-            tA[0] = o1[0];
-        }
-        if (threadIdx.x < 32) {
-            // warp 0: alpha in FP32 (the vectors use it in FP32), lane k
-            // updates y_k (FP64) and the warp forms the FP32 coarse
-            // correction; FP64 work stays in this one warp (GB300's FP64 pipe
-            // would serialise it across all warps of the SM)
+        if (!grid_allreduce_ff<1>(g, sh, blkA, tA)) { bail(); return; }
+        if (threadIdx.x == 0) {
+            // alpha in FP32: the vectors use it in FP32
             const float ps32 = (float)tA[0], gam32 = sh.ctl.gam32;
             const bool ok = ps32 > 0.0f && isfinite(ps32) && gam32 > 0.0f;
-            const float al0 = ok ? gam32 / ps32 : 0.0f;
-            if (threadIdx.x == 0) {
-                sh.ctl.al = al0;
-                sh.ctl.action = ok ? kGo : kRestart;
-            }
-            double zk = 0.0;  // this lane's (Z^T A p)_k, picked without indexing the array at run time
-#pragma unroll
-            for (int k = 0; k < kMaxCoarse; ++k)
-                if (k == R.lane) zk = tA[1 + k];
-            if (R.lane < K) {
-                y_lane = fma(-(double)al0, zk, y_lane);
-                sh.y[R.lane] = y_lane;
-            }
-            const float c = coarse32_lane(K, y_lane, sh);
-            if (R.lane < K) sh.c32[R.lane] = c;
+            sh.ctl.al = ok ? gam32 / ps32 : 0.0f;
+            sh.ctl.action = ok ? kGo : kRestart;
         }
         __syncthreads();
         if (sh.ctl.action == kRestart) {
             // breakdown of the FP32 recurrence: restart from the true residual
-            if (!replace_residual<CH>(a, g, sh, R, cur, sc, isc, true, true, t, y_lane)) { bail(); return; }
+            if (!replace_residual<CH>(a, g, sh, R, cur, sc, isc, true, true, t)) { bail(); return; }
             ++updates;
             if (threadIdx.x == 0) {
                 const double rel2 = t[0] / (bnorm * bnorm);
@@ -1656,13 +1314,12 @@ __global__ void __launch_bounds__(512, 1) k_solve_mixed(SolveArgs a)
             continue;
         }
         const float al = sh.ctl.al;
-        // pass B: e += alpha p, r -= alpha s, u = M^{-1} r; r.u, r.r
+        // pass B: e += alpha p, r -= alpha s, u = D^{-1} r; r.u, r.r
         FF accB[2] = {{0.f, 0.f}, {0.f, 0.f}};
         for (int sb = R.s0 + R.warp; sb < R.s1; sb += UB * R.nw) {
             int ii[UB];
             bool act[UB];
             float pi[UB], si[UB], ri[UB], ei[UB], di[UB];
-            int cm[UB];
 #pragma unroll
             for (int u = 0; u < UB; ++u) {
                 ii[u] = (sb + u * R.nw) * kSlice + R.lane;
@@ -1674,7 +1331,6 @@ __global__ void __launch_bounds__(512, 1) k_solve_mixed(SolveArgs a)
                 ri[u] = act[u] ? __ldcs(R32 + ii[u]) : 0.f;
                 ei[u] = act[u] ? __ldcs(E + ii[u]) : 0.f;
                 di[u] = act[u] ? __ldcs(dinv + ii[u]) : 0.f;
-                cm[u] = (act[u] && K > 0) ? (int)comp[ii[u]] : -1;
             }
 #pragma unroll
             for (int u = 0; u < UB; ++u) {
@@ -1682,8 +1338,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_mixed(SolveArgs a)
                     __stcs(E + ii[u], fmaf(al, pi[u], ei[u]));
                     const float rn = fmaf(-al, si[u], ri[u]);
                     __stcs(R32 + ii[u], rn);
-                    float un = rn * di[u];
-                    if (cm[u] >= 0) un += sh.c32[cm[u]];
+                    const float un = rn * di[u];
                     nxt[ii[u]] = make_float2(un, pi[u]);
                     ff_add(accB[0], rn * un);
                     ff_add(accB[1], rn * rn);
@@ -1720,7 +1375,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_mixed(SolveArgs a)
         if (action == kUpdate || action == kNotConverged) {
             // fold e into x (FP64) and replace r by the true residual; the
             // direction p is kept
-            if (!replace_residual<CH>(a, g, sh, R, cur, sc, isc, true, false, t, y_lane)) { bail(); return; }
+            if (!replace_residual<CH>(a, g, sh, R, cur, sc, isc, true, false, t)) { bail(); return; }
             ++updates;
             if (threadIdx.x == 0) {
                 const double rel2 = t[0] / (bnorm * bnorm);
@@ -1757,28 +1412,26 @@ __global__ void __launch_bounds__(512, 1) k_solve_mixed(SolveArgs a)
 // The two-pass iteration needs two grid-wide all-reduces (p.s, then r.u),
 // and on a mesh whose vectors stay in L2 those cost more than the passes.
 // Here the update of iteration k is folded into the operator pass of
-// iteration k + 1.  Each cell keeps the state (q, t, p, region), with
-// q = D^{-1} r the Jacobi part of the preconditioned residual and
-// t = D^{-1} s, s = A p.  Given alpha_k, beta_{k+1} and the coarse
-// correction c_{k+1} = E^{-1} Z^T r_{k+1}, one pass forms, for the cell and,
-// from their gathered state, for its neighbours,
-//     q' = q - alpha t,   u' = q' + c[region],   p' = u' + beta p,
+// iteration k + 1.  Each cell keeps the state (q, t, p), with
+// q = D^{-1} r the preconditioned residual and t = D^{-1} s, s = A p.  Given
+// alpha_k and beta_{k+1}, one pass forms, for the cell and, from their
+// gathered state, for its neighbours,
+//     q' = q - alpha t,   p' = q' + beta p,
 // then s' = A p' (difference form), t' = s' / D and e += alpha p.  Its
 // partial sums are p'.s' (for alpha), q'.D q' = r'.D^{-1} r' (for r'.u'),
 // t'.D q' and t'.D t' (so that r''.D^{-1} r'' after the next step, and with
-// it beta, follows from alpha without another all-reduce), r'.r' (the
-// stopping and replacement tests) and Z^T A p' (the coarse recurrence).  A
+// it beta, follows from alpha without another all-reduce) and r'.r' (the
+// stopping and replacement tests).  A
 // neighbour's p' is recomputed with the same operations as its owner's, so
 // both sides of a face use the same bits.  Residual replacement, restarts
 // and the stopping rules are those of the two-pass form.
 // ---------------------------------------------------------------------------
 namespace {
 
-// p' of a cell from its stored state (q, t, p, region bits).
-__device__ __forceinline__ float fused_pnew(float4 v, float al, float be, const Shared &sh)
+// p' of a cell from its stored state (q, t, p, unused).
+__device__ __forceinline__ float fused_pnew(float4 v, float al, float be)
 {
-    const float qn = fmaf(-al, v.y, v.x);
-    return fmaf(be, v.z, __fadd_rn(qn, sh.cz[__float_as_int(v.w) + 1]));
+    return fmaf(be, v.z, fmaf(-al, v.y, v.x));
 }
 
 // One group of the fused pass: slices sb, sb + nw, ... (U of them, those
@@ -1787,7 +1440,7 @@ template <int CH, int U, typename TabT>
 __device__ __forceinline__ void fused_group(const TabT &tab, int sb, int s_end, const Range &R, int n,
                                             const float4 *__restrict__ cur, float4 *__restrict__ nxt,
                                             float *__restrict__ E, const float *__restrict__ dinv, float al, float be,
-                                            int ref, float pin32, int rc, int K, Shared &sh, FF (&acc)[5])
+                                            int ref, float pin32, FF (&acc)[5])
 {
     int ii[U], base[U], w[U];
     float4 v[U];
@@ -1806,14 +1459,14 @@ __device__ __forceinline__ void fused_group(const TabT &tab, int sb, int s_end, 
             w[u] = rw.w;
         }
         // the cell's own loads all in flight together, before the gathers
-        v[u] = act ? cur[ii[u]] : make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+        v[u] = act ? cur[ii[u]] : make_float4(0.f, 0.f, 0.f, 0.f);
         di[u] = act ? __ldcs(dinv + ii[u]) : 0.0f;
         ei[u] = act ? __ldcs(E + ii[u]) : 0.0f;
         wmax = max(wmax, w[u]);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        pn[u] = fused_pnew(v[u], al, be, sh);
+        pn[u] = fused_pnew(v[u], al, be);
         si[u] = (ii[u] == ref) ? pin32 * pn[u] : 0.0f;
     }
     for (int k0 = 0; k0 < wmax; k0 += CH) {
@@ -1830,7 +1483,7 @@ __device__ __forceinline__ void fused_group(const TabT &tab, int sb, int s_end, 
 #pragma unroll
             for (int c = 0; c < CH; ++c) {
                 const float gm = (k0 + c < w[u]) ? tab.v(base[u] + (k0 + c) * kSlice + R.lane) : 0.0f;
-                si[u] = fmaf(gm, pn[u] - fused_pnew(vj[u][c], al, be, sh), si[u]);
+                si[u] = fmaf(gm, pn[u] - fused_pnew(vj[u][c], al, be), si[u]);
             }
     }
 #pragma unroll
@@ -1838,7 +1491,7 @@ __device__ __forceinline__ void fused_group(const TabT &tab, int sb, int s_end, 
         if (sb + u * R.nw < s_end && ii[u] < n) {
             const float qn = fmaf(-al, v[u].y, v[u].x);
             const float tn = si[u] * di[u];
-            nxt[ii[u]] = make_float4(qn, tn, pn[u], v[u].w);
+            nxt[ii[u]] = make_float4(qn, tn, pn[u], 0.0f);
             __stcs(E + ii[u], fmaf(al, v[u].z, ei[u]));
             const float rn = qn * __frcp_rn(di[u]);  // r' = D q'
             ff_add(acc[0], pn[u] * si[u]);
@@ -1846,7 +1499,6 @@ __device__ __forceinline__ void fused_group(const TabT &tab, int sb, int s_end, 
             ff_add(acc[2], si[u] * qn);
             ff_add(acc[3], si[u] * tn);
             ff_add(acc[4], rn * rn);
-            if (ii[u] == ref && rc >= 0 && K > 0) sh.zpin32 = pin32 * pn[u];  // pin term of Z^T A p'
         }
     }
 }
@@ -1854,16 +1506,13 @@ __device__ __forceinline__ void fused_group(const TabT &tab, int sb, int s_end, 
 // Residual replacement of the fused form.  When `fold`, first x += e / sc in
 // FP64 (e = 0).  Then r = b - A x in FP64, r32 = (float)(r sc) and
 // q = r32 / D into the state; with `zero_p` the kept direction p and its t
-// are cleared.  Every thread gets t = (||r||^2 in FP64, q.D q, t.D q, r32.r32)
-// and lane k of warp 0 the k-th component of Z^T r32.
+// are cleared.  Every thread gets t = (||r||^2 in FP64, q.D q, t.D q, r32.r32).
 template <int CH>
 __device__ __noinline__ bool replace_fused(const SolveArgs &a, Grid &g, Shared &sh, const Range &R, float4 *qd,
-                                           double sc, double isc, bool fold, bool zero_p, double (&t)[4],
-                                           double &y_lane)
+                                           double sc, double isc, bool fold, bool zero_p, double (&t)[4])
 {
     const int n = a.m.n;
     const int ref = a.prm->ref;
-    const int K = a.coarse->K;
     const double pin64 = a.prm->pin64;
     double *x = a.x64;
     if (fold) {
@@ -1877,8 +1526,7 @@ __device__ __noinline__ bool replace_fused(const SolveArgs &a, Grid &g, Shared &
         if (!grid_sync(g, sh)) return false;  // x complete
     }
     double vr[1] = {0.0};
-    FF acc[3 + kMaxCoarse];
-    for (int k = 0; k < 3 + kMaxCoarse; ++k) acc[k] = FF{0.f, 0.f};
+    FF acc[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
     for (int s = R.s0 + R.warp; s < R.s1; s += R.nw) {
         const int i = s * kSlice + R.lane;
         if (i < n) {
@@ -1887,88 +1535,42 @@ __device__ __noinline__ bool replace_fused(const SolveArgs &a, Grid &g, Shared &
             vr[0] = fma(ri, ri, vr[0]);
             const float r32 = (float)(ri * sc);
             const float q = r32 * a.dinv32[i];
-            const int cm = a.comp[i];
-            float4 v = zero_p ? make_float4(q, 0.0f, 0.0f, __int_as_float(cm)) : qd[i];
+            float4 v = zero_p ? make_float4(q, 0.0f, 0.0f, 0.0f) : qd[i];
             v.x = q;
             qd[i] = v;
             ff_add(acc[0], r32 * q);
             ff_add(acc[1], v.y * r32);
             ff_add(acc[2], r32 * r32);
-#pragma unroll
-            for (int k = 0; k < kMaxCoarse; ++k) ff_add(acc[3 + k], (cm == k) ? r32 : 0.0f);
         }
     }
     block_sum_f64<1>(sh, vr);
-    double ffo[3 + kMaxCoarse];
-    block_sum_ff<3 + kMaxCoarse>(sh, acc, ffo);
-    double blk[4 + kMaxCoarse], tt[4 + kMaxCoarse];
-    blk[0] = vr[0];
-    for (int k = 0; k < 3 + kMaxCoarse; ++k) blk[1 + k] = ffo[k];
+    double ffo[3];
+    block_sum_ff<3>(sh, acc, ffo);
+    const double blk[4] = {vr[0], ffo[0], ffo[1], ffo[2]};
     // also the barrier after which the next pass gathers the new q
-    if (!grid_allreduce<4 + kMaxCoarse>(g, sh, blk, tt, 4 + K)) return false;
-    for (int k = 0; k < 4; ++k) t[k] = tt[k];  // every thread: the all-reduced values
-    if (threadIdx.x < 32) {
-        double yl = 0.0;  // lane k's component, picked without indexing the array at run time
-#pragma unroll
-        for (int k = 0; k < kMaxCoarse; ++k)
-            if (k == R.lane && k < K) yl = tt[4 + k];
-        y_lane = yl;
-    }
-    return true;
+    return grid_allreduce<4>(g, sh, blk, t);  // every thread: the all-reduced values
 }
 
-// Warp 0, K <= 8: y.c = sum over lanes k < K of y_k c_k in FP32 (lanes >= K
-// hold zeros, so three butterfly steps sum lanes 0..7), from lane 0 to all.
-__device__ __forceinline__ float coarse_dot8(int K, double y_lane, float c)
-{
-    float yc = ((threadIdx.x & 31) < K) ? (float)y_lane * c : 0.0f;
-    yc += __shfl_xor_sync(0xffffffffu, yc, 4);
-    yc += __shfl_xor_sync(0xffffffffu, yc, 2);
-    yc += __shfl_xor_sync(0xffffffffu, yc, 1);
-    return __shfl_sync(0xffffffffu, yc, 0);
-}
-
-// Warp 0: r.u of the state, q.D q plus the coarse part y.c with c = E^{-1} y
-// in FP32 (the correction the vectors use).  All lanes return the same value.
-__device__ __forceinline__ double fused_gamma(int K, double qdq, double y_lane, const Shared &sh)
-{
-    static_assert(kMaxCoarse <= 8, "coarse_dot8 sums at most 8 lanes");
-    return qdq + (double)coarse_dot8(K, y_lane, coarse32_lane(K, y_lane, sh));
-}
-
-// Warp 0: one step of the recurrences from state k (gam = r_k.u_k, ps, qdq,
-// tdq, tdt = the all-reduced p.s, q.D q, t.D q, t.D t of state k, zk_lane =
-// (Z^T A p_k)_lane): alpha_k = gam / p.s in FP32 (the vectors' precision, as
-// in the two-pass form), y_{k+1} = y_k - alpha_k Z^T A p_k (FP64),
-// c_{k+1} = E^{-1} y_{k+1} into sh.cz, r_{k+1}.u_{k+1} =
-// q.D q - 2 alpha t.D q + alpha^2 t.D t + y_{k+1}.c_{k+1} (FP64, where the
+// Thread 0: one step of the recurrences from state k (gam = r_k.u_k, ps, qdq,
+// tdq, tdt = the all-reduced p.s, q.D q, t.D q, t.D t of state k): alpha_k =
+// gam / p.s in FP32 (the vectors' precision, as in the two-pass form),
+// r_{k+1}.u_{k+1} = q.D q - 2 alpha t.D q + alpha^2 t.D t (FP64, where the
 // terms cancel) and beta_{k+1} = r_{k+1}.u_{k+1} / gam into sh.ctl.  With
 // `restart`, alpha = beta = 0 (the next direction is the preconditioned
 // residual).  A non-positive expanded r.u (rounding at a steep drop) also
-// sets beta = 0.  FP64 work is kept to a few instructions: GB300's FP64 pipe
-// makes each one cost as much as a long FP32 sequence.
-__device__ __forceinline__ void fused_advance(int K, double gam, double ps, double qdq, double tdq, double tdt,
-                                              double zk_lane, double &y_lane, bool restart, Shared &sh)
+// sets beta = 0.
+__device__ __forceinline__ void fused_advance(double gam, double ps, double qdq, double tdq, double tdt, bool restart,
+                                              Shared &sh)
 {
-    const int lane = threadIdx.x & 31;
     float al = 0.0f, be = 0.0f;
     if (!restart) {
         al = (float)gam / (float)ps;
-        if (lane < K) y_lane = fma(-(double)al, zk_lane, y_lane);
-    }
-    const float c = coarse32_lane(K, y_lane, sh);
-    if (!restart) {
         const double ad = (double)al;
-        const double gn = fma(ad, fma(ad, tdt, -2.0 * tdq), qdq) + (double)coarse_dot8(K, y_lane, c);
+        const double gn = fma(ad, fma(ad, tdt, -2.0 * tdq), qdq);
         be = (gn > 0.0 && isfinite(gn)) ? (float)gn / (float)gam : 0.0f;
     }
-    if (lane < kMaxCoarse) sh.cz[1 + lane] = (lane < K) ? c : 0.0f;
-    if (lane == 0) {
-        sh.cz[0] = 0.0f;
-        sh.ctl.al = al;
-        sh.ctl.be = be;
-    }
-    __syncwarp();
+    sh.ctl.al = al;
+    sh.ctl.be = be;
 }
 
 }  // namespace
@@ -1993,7 +1595,6 @@ __global__ void __launch_bounds__(512, 1) k_solve_fused(SolveArgs a)
     extern __shared__ __align__(16) unsigned char dsm[];
     Grid g{a.bar, a.err, a.partials, a.budget_ns, 0u, (int)gridDim.x, 0};
     const Range R = my_range(a.m.n_slices);
-    stage_coarse(a.coarse, sh);
     const Tab<float> tab = stage_tables<float>(a.m, a.m.val32, R, a.cache_cap, a.meta_slots, dsm);
     Ring ring{};
     if constexpr (STREAM) ring = make_ring(a, R, tab.meta, dsm, sh, false);
@@ -2005,9 +1606,6 @@ __global__ void __launch_bounds__(512, 1) k_solve_fused(SolveArgs a)
     const int n = a.m.n;
     const int ref = a.prm->ref;
     const float pin32 = a.prm->pin32;
-    const int K = a.coarse->K;
-    const int rc = a.coarse->ref_comp;
-    const int nx = a.coarse->n_cross;
     float *__restrict__ E = a.E;
     const float *__restrict__ dinv = a.dinv32;
 
@@ -2046,28 +1644,21 @@ __global__ void __launch_bounds__(512, 1) k_solve_fused(SolveArgs a)
     float4 *cur = a.Q0, *nxt = a.Q1;  // cur: the state the next pass reads
     int iters = 0, updates = 0, status = GFM_OK;
     double t[4];
-    double y_lane = 0.0;   // warp 0: Z^T r of the current state (lane k: component k)
-    double zk_lane = 0.0;  // warp 0: Z^T A p of the current state
-    if (!replace_fused<CH>(a, g, sh, R, cur, sc, isc, false, true, t, y_lane)) { bail(); return; }
+    if (!replace_fused<CH>(a, g, sh, R, cur, sc, isc, false, true, t)) { bail(); return; }
     ++updates;
-    if (threadIdx.x < 32) {
-        const double gam = fused_gamma(K, t[1], y_lane, sh);
-        if (threadIdx.x == 0) {
-            fs.best_rel2 = t[0] / (fs.bnorm * fs.bnorm);
-            fs.gam = gam;
-            fs.rho_max = t[3];
-            sh.ctl.action = (fs.best_rel2 <= a.rtol * a.rtol) ? kConverged : kGo;
-        }
-        fused_advance(K, gam, 0.0, 0.0, 0.0, 0.0, 0.0, y_lane, true, sh);
-        zero_bins(sh);
+    if (threadIdx.x == 0) {
+        fs.best_rel2 = t[0] / (fs.bnorm * fs.bnorm);
+        fs.gam = t[1];
+        fs.rho_max = t[3];
+        sh.ctl.action = (fs.best_rel2 <= a.rtol * a.rtol) ? kConverged : kGo;
+        fused_advance(t[1], 0.0, 0.0, 0.0, 0.0, true, sh);
     }
     __syncthreads();
     int action = sh.ctl.action;
     if constexpr (STREAM)
         if (threadIdx.x == 0) ring_prefetch(ring);
     while (action != kConverged) {
-        // al, be, sh.cz and the cleared coarse bins were published by warp 0
-        // before the CTA barrier that ended the last scalar step
+        // published by thread 0 before the CTA barrier that ended the last scalar step
         const float al = sh.ctl.al, be = sh.ctl.be;
         // the fused pass: the update of the last step and s' = A p' of this one
         FF acc[5];
@@ -2080,7 +1671,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_fused(SolveArgs a)
                     const int sr1 = min(R.s1, sr0 + ring.stage_slices);
                     const StageTab st = ring_stage(ring, r);
                     for (int sb = sr0 + R.warp; sb < sr1; sb += US * R.nw)
-                        fused_group<CH, US>(st, sb, sr1, R, n, cur, nxt, E, dinv, al, be, ref, pin32, rc, K, sh, acc);
+                        fused_group<CH, US>(st, sb, sr1, R, n, cur, nxt, E, dinv, al, be, ref, pin32, acc);
                 } else {
                     sh.ring_fail = 1;
                 }
@@ -2098,57 +1689,39 @@ __global__ void __launch_bounds__(512, 1) k_solve_fused(SolveArgs a)
         } else if (tab.full) {
             const StageTab ft{tab.meta, tab.col, tab.val, tab.s0, tab.base0};
             for (int sb = R.s0 + R.warp; sb < R.s1; sb += U * R.nw)
-                fused_group<CH, U>(ft, sb, R.s1, R, n, cur, nxt, E, dinv, al, be, ref, pin32, rc, K, sh, acc);
+                fused_group<CH, U>(ft, sb, R.s1, R, n, cur, nxt, E, dinv, al, be, ref, pin32, acc);
         } else {
             for (int sb = R.s0 + R.warp; sb < R.s1; sb += U * R.nw)
-                fused_group<CH, U>(tab, sb, R.s1, R, n, cur, nxt, E, dinv, al, be, ref, pin32, rc, K, sh, acc);
+                fused_group<CH, U>(tab, sb, R.s1, R, n, cur, nxt, E, dinv, al, be, ref, pin32, acc);
         }
-        if (K > 0)  // Z^T (A p') from the faces between coarse regions (the pin's share is added above)
-            cross_sums<float>(a.cross, nx, K, sh.zbw32, [&](const CrossFace &cf) {
-                return cf.g32 * (fused_pnew(cur[cf.o], al, be, sh) - fused_pnew(cur[cf.v], al, be, sh));
-            });
-        double tP[5 + kMaxCoarse];
+        double tP[5];
         {
-            float2 blk[5], b[5 + kMaxCoarse];
+            float2 blk[5];
             block_sum_ff2<5>(sh, acc, blk);
-            for (int k = 0; k < 5; ++k) b[k] = blk[k];
-            if (K > 0 && threadIdx.x < 32) finish_bins<float>(sh.zbw32, sh.zpin32, rc, K, R.nw, sh.zb32);
-            for (int k = 0; k < kMaxCoarse; ++k) b[5 + k] = make_float2((K > 0) ? sh.zb32[k] : 0.0f, 0.0f);
             // also the barrier after which the next pass gathers the new state
-            if (!grid_allreduce_ff<5 + kMaxCoarse>(g, sh, b, tP, 5 + K)) { bail(); return; }
+            if (!grid_allreduce_ff<5>(g, sh, blk, tP)) { bail(); return; }
         }
         ++iters;
         { float4 *tmp = cur; cur = nxt; nxt = tmp; }
-        if (threadIdx.x < 32) {
-            zero_bins(sh);  // this pass's bins were read before the all-reduce
-            double zl = 0.0;
-#pragma unroll
-            for (int k = 0; k < kMaxCoarse; ++k)
-                if (k == R.lane && k < K) zl = tP[5 + k];
-            zk_lane = zl;
-            const double gam = fused_gamma(K, tP[1], y_lane, sh);
-            if (threadIdx.x == 0) {
-                const double ps = tP[0], rho = tP[4];
-                fs.gam = gam;
-                fs.ps = ps;
-                fs.tdt = tP[3];
-                if (rho > fs.rho_max) fs.rho_max = rho;
-                if (iters >= a.max_iters) {
-                    sh.ctl.action = kNotConverged;
-                } else if (!(ps > 0.0) || !isfinite(ps) || !(gam > 0.0)) {
-                    sh.ctl.action = kRestart;  // breakdown of the FP32 recurrence
-                } else if (rho <= 1e-2 * fs.rho_max || rho <= fs.rho_stop || iters - fs.last_upd >= 1000) {
-                    // replacement when the FP32 residual fell a decade, claims
-                    // convergence, or has not fallen a decade for 1000 iterations
-                    sh.ctl.action = kUpdate;
-                    fs.last_upd = iters;
-                } else {
-                    sh.ctl.action = kGo;
-                }
+        if (threadIdx.x == 0) {
+            const double ps = tP[0], gam = tP[1], rho = tP[4];
+            fs.gam = gam;
+            fs.ps = ps;
+            fs.tdt = tP[3];
+            if (rho > fs.rho_max) fs.rho_max = rho;
+            if (iters >= a.max_iters) {
+                sh.ctl.action = kNotConverged;
+            } else if (!(ps > 0.0) || !isfinite(ps) || !(gam > 0.0)) {
+                sh.ctl.action = kRestart;  // breakdown of the FP32 recurrence
+            } else if (rho <= 1e-2 * fs.rho_max || rho <= fs.rho_stop || iters - fs.last_upd >= 1000) {
+                // replacement when the FP32 residual fell a decade, claims
+                // convergence, or has not fallen a decade for 1000 iterations
+                sh.ctl.action = kUpdate;
+                fs.last_upd = iters;
+            } else {
+                sh.ctl.action = kGo;
+                fused_advance(gam, ps, tP[1], tP[2], tP[3], false, sh);
             }
-            __syncwarp();
-            if (sh.ctl.action == kGo)
-                fused_advance(K, gam, tP[0], tP[1], tP[2], tP[3], zk_lane, y_lane, false, sh);
         }
         __syncthreads();
         action = sh.ctl.action;
@@ -2156,14 +1729,13 @@ __global__ void __launch_bounds__(512, 1) k_solve_fused(SolveArgs a)
         // fold e into x (FP64) and replace r by the true residual; the
         // direction is kept, or cleared on a restart
         const bool restart = action == kRestart;
-        if (!replace_fused<CH>(a, g, sh, R, cur, sc, isc, true, restart, t, y_lane)) { bail(); return; }
+        if (!replace_fused<CH>(a, g, sh, R, cur, sc, isc, true, restart, t)) { bail(); return; }
         ++updates;
-        if (threadIdx.x < 32) {
+        if (threadIdx.x == 0) {
             // r.u of the state before the replacement: the recurrences' own
             // value, which the step along the kept direction keeps using
             const double gam_pre = fs.gam;
-            __syncwarp();
-            if (threadIdx.x == 0) {
+            {
                 const double rel2 = t[0] / (fs.bnorm * fs.bnorm);
                 if (rel2 <= a.rtol * a.rtol) {
                     sh.ctl.action = kConverged;
@@ -2183,7 +1755,6 @@ __global__ void __launch_bounds__(512, 1) k_solve_fused(SolveArgs a)
                 }
                 if (sh.ctl.action == kGo) fs.rho_max = t[3];
             }
-            __syncwarp();
             if (sh.ctl.action == kGo) {
                 // Residual replacement keeps the recurrences' step: alpha from
                 // the pre-replacement r.u and the kept direction's p.s, and beta
@@ -2196,7 +1767,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_fused(SolveArgs a)
                 // cleared), or when the kept direction cannot give a step, the
                 // next direction is the preconditioned residual (alpha = beta = 0).
                 const bool fresh = restart || !(fs.ps > 0.0 && gam_pre > 0.0);
-                fused_advance(K, gam_pre, fs.ps, t[1], t[2], fs.tdt, zk_lane, y_lane, fresh, sh);
+                fused_advance(gam_pre, fs.ps, t[1], t[2], fs.tdt, fresh, sh);
             }
         }
         __syncthreads();
@@ -2228,10 +1799,6 @@ struct TankState {
     double rho_max[kMaxTanks], best[kMaxTanks], rho_stop[kMaxTanks], xavg[kMaxTanks];
     double tot[6][kMaxTanks];
     float al[kMaxTanks], be[kMaxTanks];
-    // each tank's coarse space: K vectors, region of the pinned cell, stretch
-    // [x0, x1) of the cross-face list, E^{-1}; y = Z^T r (FP64 recurrence)
-    // and the correction c = E^{-1} y (FP32, added to u)
-    int K[kMaxTanks], rc[kMaxTanks], x0[kMaxTanks], x1[kMaxTanks];
     // CTAs of each tank [first, last + 1), re-planned when tanks finish, and
     // each tank's slices [sfirst, sfirst + nslc) and end of its real cells
     int2 tcta[kMaxTanks];
@@ -2241,10 +1808,6 @@ struct TankState {
     int wide[kMaxTanks];
     int n_wide;
     unsigned ring_used;  // thread 0's count of consumed stages after a drain
-    double Einv[kTankCoarse * kTankCoarse][kMaxTanks];
-    float Einv32[kTankCoarse * kTankCoarse][kMaxTanks];  // the same in FP32 (the FP32 iterations' correction)
-    double y[kTankCoarse][kMaxTanks];
-    float c32[kTankCoarse][kMaxTanks];
     int act[kMaxTanks];   // kGo while iterating, else kConverged / kNotConverged / kBreakdown
     int flag[kMaxTanks];  // replacement in this iteration: 0, kUpdate, kRestart, kNotConverged
     // a replacement a tank asked for while it can still iterate (kUpdate):
@@ -2379,40 +1942,6 @@ __device__ __forceinline__ void list_wide(TankState &ts, int T)
     ts.n_wide = n;
 }
 
-// One lane, one tank: c = E^{-1} y into ts.c32 (K <= 2); returns y.c.
-// The FP32 iterations' form: c = E^{-1} y from the FP32 inverse and the
-// rounded y (the vectors apply c in FP32; a chain of FP64 multiply-adds per
-// tank costs far more on GB300's FP64 pipe).
-__device__ __forceinline__ void tank_coarse_solve32(TankState &ts, int t)
-{
-    const int K = ts.K[t];
-    float yf[kTankCoarse];
-#pragma unroll
-    for (int j = 0; j < kTankCoarse; ++j) yf[j] = (j < K) ? (float)ts.y[j][t] : 0.0f;
-#pragma unroll
-    for (int i = 0; i < kTankCoarse; ++i) {
-        if (i >= K) break;
-        float c = 0.0f;
-#pragma unroll
-        for (int j = 0; j < kTankCoarse; ++j)
-            if (j < K) c = fmaf(ts.Einv32[i * kTankCoarse + j][t], yf[j], c);
-        ts.c32[i][t] = c;
-    }
-}
-
-__device__ __forceinline__ double tank_coarse_solve(TankState &ts, int t)
-{
-    const int K = ts.K[t];
-    double yc = 0.0;
-    for (int i = 0; i < K; ++i) {
-        double c = 0.0;
-        for (int j = 0; j < K; ++j) c = fma(ts.Einv[i * kTankCoarse + j][t], ts.y[j][t], c);
-        ts.c32[i][t] = (float)c;
-        yc = fma(c, ts.y[i][t], yc);
-    }
-    return yc;
-}
-
 // Residual replacement for the tanks with a pending flag (or all, `all`):
 // x += e / sc (FP64, when `fold`), r = b - A x (FP64, difference form),
 // r32 = (float)(r sc), u = r32 / D into up (direction cleared on restart).
@@ -2453,13 +1982,13 @@ __device__ bool batch_replace(const SolveArgs &a, const BatchArgs &bt, Grid &g, 
         if (!grid_sync(g, sh)) return false;  // x complete
     }
     double vr[1] = {0.0};
-    FF acc[2 + kTankCoarse] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+    FF acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
     if (work) {
         // two slices per warp at a time: the residual pass is a chain of
         // dependent loads per row (slice table, slots, neighbours)
         constexpr int UR = 2;
         for (int sb = R.s0 + R.warp; sb < R.s1; sb += UR * R.nw) {
-            int ii[UR], cm[UR];
+            int ii[UR];
             bool act[UR];
             Row rw[UR];
             double xi[UR], bi[UR], pin[UR], ax[UR];
@@ -2473,7 +2002,6 @@ __device__ bool batch_replace(const SolveArgs &a, const BatchArgs &bt, Grid &g, 
                 xi[u] = act[u] ? x[ii[u]] : 0.0;
                 bi[u] = act[u] ? a.b[ii[u]] : 0.0;
                 di[u] = act[u] ? a.dinv32[ii[u]] : 0.0f;
-                cm[u] = act[u] ? (int)a.comp[ii[u]] : -1;
                 pin[u] = (act[u] && ii[u] == ref) ? pin64 : 0.0;
             }
             apply64_diff_multi<CH, UR>(a.m, rw, R.lane, x, xi, pin, ax);
@@ -2490,52 +2018,14 @@ __device__ bool batch_replace(const SolveArgs &a, const BatchArgs &bt, Grid &g, 
                 else up[i].x = uu;
                 ff_add(acc[0], r32 * uu);
                 ff_add(acc[1], r32 * r32);
-#pragma unroll
-                for (int k = 0; k < kTankCoarse; ++k) ff_add(acc[2 + k], (cm[u] == k) ? r32 : 0.0f);
             }
         }
     }
     block_sum_f64<1>(sh, vr);
-    double ffo[2 + kTankCoarse];
-    block_sum_ff<2 + kTankCoarse>(sh, acc, ffo);
-    const double blk[3 + kTankCoarse] = {vr[0], ffo[0], ffo[1], ffo[2], ffo[3]};
-    if (!batch_allreduce<3 + kTankCoarse>(g, sh, ts, bt, blk)) return false;
-    // replaced tanks: y = Z^T r exactly, c = E^{-1} y, r.z gains y.c, and the
-    // coarse correction joins u
-    int any_coarse = 0;
-    if (threadIdx.x < 32) {
-        for (int t = threadIdx.x; t < bt.T; t += 32) {
-            if (!(all || ts.flag[t] != 0) || ts.K[t] == 0) continue;
-            for (int k = 0; k < ts.K[t]; ++k) ts.y[k][t] = ts.tot[3 + k][t];
-            ts.tot[1][t] += tank_coarse_solve(ts, t);
-            any_coarse = 1;
-        }
-        any_coarse = __any_sync(0xffffffffu, any_coarse);
-        if (threadIdx.x == 0) sh.flag = any_coarse;
-    }
-    __syncthreads();
-    if (sh.flag == 0) return true;  // the same in every CTA
-    __syncthreads();
-    if (work && ts.K[tank] > 0) {
-        constexpr int UF = 4;  // four slices per warp at a time, their loads in flight together
-        for (int sb = R.s0 + R.warp; sb < R.s1; sb += UF * R.nw) {
-            int cm[UF];
-            float ux[UF];
-#pragma unroll
-            for (int u = 0; u < UF; ++u) {
-                const int i = (sb + u * R.nw) * kSlice + R.lane;
-                const bool act = sb + u * R.nw < R.s1 && i < cend;
-                cm[u] = act ? (int)a.comp[i] : -1;
-                ux[u] = act ? up[i].x : 0.0f;
-            }
-#pragma unroll
-            for (int u = 0; u < UF; ++u) {
-                const int i = (sb + u * R.nw) * kSlice + R.lane;
-                if (cm[u] >= 0) up[i].x = ux[u] + ts.c32[cm[u]][tank];
-            }
-        }
-    }
-    return grid_sync(g, sh);  // u complete before it is gathered
+    double ffo[2];
+    block_sum_ff<2>(sh, acc, ffo);
+    const double blk[3] = {vr[0], ffo[0], ffo[1]};
+    return batch_allreduce<3>(g, sh, ts, bt, blk);  // also the barrier before u is gathered
 }
 
 // Warp 0 of every CTA: split the grid among the tanks that take part (those
@@ -2836,19 +2326,6 @@ __global__ void __launch_bounds__(512, 1) k_solve_batched(SolveArgs a, BatchArgs
             ts.iters[t] = ts.updates[t] = ts.stall[t] = ts.last_upd[t] = ts.restarts[t] = 0;
             ts.be[t] = 0.0f;
             ts.gam_prev[t] = 1.0;
-            const TankCoarse &tc = bt.tco[t];
-            ts.K[t] = tc.K;
-            ts.rc[t] = tc.ref_comp;
-            ts.x0[t] = tc.x0;
-            ts.x1[t] = tc.x1;
-            for (int q = 0; q < kTankCoarse * kTankCoarse; ++q) {
-                ts.Einv[q][t] = tc.Einv[q];
-                ts.Einv32[q][t] = (float)tc.Einv[q];
-            }
-            for (int k = 0; k < kTankCoarse; ++k) {
-                ts.y[k][t] = 0.0;
-                ts.c32[k][t] = 0.0f;
-            }
         }
     }
     __syncthreads();
@@ -2877,17 +2354,12 @@ __global__ void __launch_bounds__(512, 1) k_solve_batched(SolveArgs a, BatchArgs
         ts.n_active = T;  // re-plan as soon as any tank is done
         if constexpr (STREAM) ring_prefetch(ring);
     }
-    if (threadIdx.x < 32) zero_bins(sh);
     // tanks that the start already solves give their CTAs away at once
     if (!replan_if_finished()) { bail(); return; }
     while (ts.any_active) {
         const bool work = ts.act[tank] == kGo && ts.wait[tank] == 0;
         const float be = ts.be[tank];
-        // pass A: p = u + beta p (own and, redundantly, neighbours), s = A p, p.s,
-        // and the tank's Z^T (A p) from its faces between coarse regions
-        const int Kt = ts.K[tank];
-        // the coarse bins were cleared by warp 0 in the last alpha step (or
-        // before the loop), ahead of a CTA barrier
+        // pass A: p = u + beta p (own and, redundantly, neighbours), s = A p, p.s
         FF accA[1] = {{0.f, 0.f}};
         if constexpr (STREAM) {
             // every stage is waited for, so the ring stays in step even when
@@ -2901,12 +2373,12 @@ __global__ void __launch_bounds__(512, 1) k_solve_batched(SolveArgs a, BatchArgs
                             const StageTabCT st = ring_stage_ct(ring, r);
                             for (int sb = sr0 + R.warp; sb < sr1; sb += US * R.nw)
                                 mixed_op_group<CH, US>(st, sb, sr1, R, cend, cur, P32, S32, be, ref, pin32,
-                                                       ts.rc[tank], Kt, sh, accA[0]);
+                                                       accA[0]);
                         } else {
                             const StageTab st = ring_stage(ring, r);
                             for (int sb = sr0 + R.warp; sb < sr1; sb += US * R.nw)
                                 mixed_op_group<CH, US>(st, sb, sr1, R, cend, cur, P32, S32, be, ref, pin32,
-                                                       ts.rc[tank], Kt, sh, accA[0]);
+                                                       accA[0]);
                         }
                     }
                 } else {
@@ -2925,34 +2397,14 @@ __global__ void __launch_bounds__(512, 1) k_solve_batched(SolveArgs a, BatchArgs
             // the next pass's first stages load during the rest of the iteration
             if (threadIdx.x == 0) ring_prefetch(ring);
         }
-        if (work) {
-            if constexpr (!STREAM)
+        if constexpr (!STREAM)
+            if (work)
                 for (int sb = R.s0 + R.warp; sb < R.s1; sb += U * R.nw)
-                    mixed_op_group_hoisted<CH, U>(tab, sb, R.s1, R, cend, cur, P32, S32, be, ref, pin32, ts.rc[tank],
-                                                  Kt, sh, accA[0]);
-            if (Kt > 0) {
-                // this CTA's share of the tank's cross faces
-                const int2 tr = ts.tcta[tank];
-                const long long q = blockIdx.x - tr.x, nq = tr.y - tr.x, span = ts.x1[tank] - ts.x0[tank];
-                cross_sums_range<float>(a.cross, ts.x0[tank] + (int)(span * q / nq),
-                                        ts.x0[tank] + (int)(span * (q + 1) / nq), Kt, sh.zbw32,
-                                        [&](const CrossFace &cf) {
-                                            const float2 vo = cur[cf.o], vv = cur[cf.v];
-                                            return cf.g32 * (fmaf(be, vo.y, vo.x) - fmaf(be, vv.y, vv.x));
-                                        });
-            }
-        }
-        float2 blkA[1 + kTankCoarse];
-        {
-            float2 b1[1];
-            block_sum_ff2<1>(sh, accA, b1);
-            blkA[0] = b1[0];
-        }
-        if (work && Kt > 0 && threadIdx.x < 32) finish_bins<float>(sh.zbw32, sh.zpin32, ts.rc[tank], Kt, R.nw, sh.zb32);
-        for (int k = 0; k < kTankCoarse; ++k) blkA[1 + k] = make_float2((work && k < Kt) ? sh.zb32[k] : 0.0f, 0.0f);
-        if (!batch_allreduce_ff<1 + kTankCoarse>(g, sh, ts, bt, blkA)) { bail(); return; }
+                    mixed_op_group_hoisted<CH, U>(tab, sb, R.s1, R, cend, cur, P32, S32, be, ref, pin32, accA[0]);
+        float2 blkA[1];
+        block_sum_ff2<1>(sh, accA, blkA);
+        if (!batch_allreduce_ff<1>(g, sh, ts, bt, blkA)) { bail(); return; }
         if (threadIdx.x < 32) {
-            zero_bins(sh);  // this pass's bins were read before the all-reduce
             for (int t = threadIdx.x; t < T; t += 32) {
                 if (ts.act[t] != kGo || ts.wait[t]) continue;
                 const double ps = ts.tot[0][t];
@@ -2962,10 +2414,6 @@ __global__ void __launch_bounds__(512, 1) k_solve_batched(SolveArgs a, BatchArgs
                 const float al = ok ? (float)ts.gam[t] / (float)ps : 0.0f;
                 ts.al[t] = al;
                 ts.flag[t] = ok ? 0 : kRestart;
-                if (ok && ts.K[t] > 0) {  // y -= alpha Z^T A p (FP64), c = E^{-1} y (FP32)
-                    for (int k = 0; k < ts.K[t]; ++k) ts.y[k][t] = fma(-(double)al, ts.tot[1 + k][t], ts.y[k][t]);
-                    tank_coarse_solve32(ts, t);
-                }
             }
         }
         __syncthreads();
@@ -2974,7 +2422,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_batched(SolveArgs a, BatchArgs
         FF accB[2] = {{0.f, 0.f}, {0.f, 0.f}};
         if (work && ts.flag[tank] == 0) {
             for (int sb = R.s0 + R.warp; sb < R.s1; sb += UB * R.nw) {
-                int ii[UB], cm[UB];
+                int ii[UB];
                 bool act[UB];
                 float pi[UB], si[UB], ri[UB], ei[UB], di[UB];
 #pragma unroll
@@ -2987,7 +2435,6 @@ __global__ void __launch_bounds__(512, 1) k_solve_batched(SolveArgs a, BatchArgs
                     ri[u] = act[u] ? __ldcs(R32 + ii[u]) : 0.f;
                     ei[u] = act[u] ? __ldcs(E + ii[u]) : 0.f;
                     di[u] = act[u] ? __ldcs(dinv + ii[u]) : 0.f;
-                    cm[u] = (act[u] && Kt > 0) ? (int)a.comp[ii[u]] : -1;
                 }
 #pragma unroll
                 for (int u = 0; u < UB; ++u) {
@@ -2995,8 +2442,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_batched(SolveArgs a, BatchArgs
                         __stcs(E + ii[u], fmaf(al, pi[u], ei[u]));
                         const float rn = fmaf(-al, si[u], ri[u]);
                         __stcs(R32 + ii[u], rn);
-                        float un = rn * di[u];
-                        if (cm[u] >= 0) un += ts.c32[cm[u]][tank];
+                        const float un = rn * di[u];
                         nxt[ii[u]] = make_float2(un, pi[u]);
                         ff_add(accB[0], rn * un);
                         ff_add(accB[1], rn * rn);
