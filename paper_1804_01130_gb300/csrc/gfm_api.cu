@@ -1485,8 +1485,11 @@ gfm_status gfm_gradient(gfm_handle h, const double *p, const double *V, const do
     if (grad && !h->assembled) return fail(h, GFM_ERR_STATE, "gradient before assemble");
     clear_stale_error();
     cudaStream_t s = (cudaStream_t)stream;
-    const gfm_status st = need_grad_rec(h);
-    if (st != GFM_OK) return st;
+    const bool small = h->F < gfm::kGradSmallFaces;
+    if (!small) {
+        const gfm_status st = need_grad_rec(h);
+        if (st != GFM_OK) return st;
+    }
     gfm::GradArgs a{};
     a.n = h->n;
     a.F = h->F;
@@ -1509,12 +1512,12 @@ gfm_status gfm_gradient(gfm_handle h, const double *p, const double *V, const do
     a.inv_a = known_inverse(a.rho_a);
     a.ftank = h->batched ? h->ftank : nullptr;
     a.tphys = h->batched ? h->tphys : nullptr;
-    a.rec = h->grad_rec;
+    a.rec = small ? nullptr : h->grad_rec;
     a.grad = grad;
     a.U = U;
     GFM_CUDA(h, gfm::launch_gradient(a, s));
-    h->prof.launches = 2;
-    h->prof.launches_total += 2;
+    h->prof.launches = small ? 1 : 2;
+    h->prof.launches_total += small ? 1 : 2;
     return GFM_OK;
 }
 

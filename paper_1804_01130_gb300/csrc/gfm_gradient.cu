@@ -56,6 +56,26 @@ __device__ __forceinline__ double4 load_record(const double4 *p)
     return v;
 }
 
+// S.(x_f - x_own) / S.d of a face with a given centre.
+__device__ __forceinline__ double face_weight(const GradArgs &a, int f, int o, double S0, double S1, double S2,
+                                              double x0, double x1, double x2)
+{
+    const size_t n = (size_t)a.n;
+    const double2 sd = a.sd[f];
+    return div_known(S0 * (x0 - a.C[o]) + S1 * (x1 - a.C[n + o]) + S2 * (x2 - a.C[2 * n + o]), sd.x, sd.y);
+}
+
+// The densities of a face's tank and their inverses as div_known takes them.
+struct Densities {
+    double w, a, inv_w, inv_a;
+};
+__device__ __forceinline__ Densities densities(const GradArgs &a, int f)
+{
+    if (!a.ftank) return Densities{a.rho_w, a.rho_a, a.inv_w, a.inv_a};
+    const TankPhys *tp = a.tphys + a.ftank[f];
+    return Densities{tp->rho_w, tp->rho_a, tp->inv_w, tp->inv_a};
+}
+
 template <bool G, bool U>
 __global__ void __launch_bounds__(256) k_grad_faces(GradArgs a)
 {
@@ -70,21 +90,17 @@ __global__ void __launch_bounds__(256) k_grad_faces(GradArgs a)
     const int o = on ? a.owner[f] : 0, nb = on ? a.neighbour[f] : 0;
     double q = 0.0;
     if (G) {
-        double rho_w = a.rho_w, rho_a = a.rho_a, inv_w = a.inv_w, inv_a = a.inv_a;
         bool iface = false;
         if (on) {
             const int8_t kind = a.kind[f];
-            if (a.ftank) {
-                const TankPhys *tp = a.tphys + a.ftank[f];
-                rho_w = tp->rho_w;
-                rho_a = tp->rho_a;
-                inv_w = tp->inv_w;
-                inv_a = tp->inv_a;
-            }
             iface = kind > 1;  // 0: both cells dry, 1: both wet
             q = a.p[nb] - a.p[o];
-            if (iface) q -= a.jump[f];
-            else q = div_known(q, kind ? rho_w : rho_a, kind ? inv_w : inv_a);
+            if (iface) {
+                q -= a.jump[f];
+            } else {
+                const Densities rho = densities(a, f);
+                q = div_known(q, kind ? rho.w : rho.a, kind ? rho.inv_w : rho.inv_a);
+            }
         }
         const unsigned m = __ballot_sync(0xffffffffu, iface);
         if (lane == 0) wcount[warp] = __popc(m);
@@ -105,11 +121,8 @@ __global__ void __launch_bounds__(256) k_grad_faces(GradArgs a)
             if ((int)threadIdx.x < total) {
                 const int e = list[threadIdx.x];
                 const double lam = a.lambda[e];
-                if (a.ftank) {
-                    rho_w = a.tphys[a.ftank[e]].rho_w;
-                    rho_a = a.tphys[a.ftank[e]].rho_a;
-                }
-                val[threadIdx.x] = val[threadIdx.x] / (lam * rho_w + (1.0 - lam) * rho_a);
+                const Densities rho = densities(a, e);
+                val[threadIdx.x] = val[threadIdx.x] / (lam * rho.w + (1.0 - lam) * rho.a);
             }
             __syncthreads();
             if (iface) q = val[at];
@@ -126,11 +139,7 @@ __global__ void __launch_bounds__(256) k_grad_faces(GradArgs a)
     }
     if (G) {
         const double S0 = a.Sf[f], S1 = a.Sf[F + f], S2 = a.Sf[2 * F + f];
-        double fac = 0.5;
-        if (!mid) {
-            const double2 sd = a.sd[f];
-            fac = div_known(S0 * (x0 - a.C[o]) + S1 * (x1 - a.C[n + o]) + S2 * (x2 - a.C[2 * n + o]), sd.x, sd.y);
-        }
+        const double fac = mid ? 0.5 : face_weight(a, f, o, S0, S1, S2, x0, x1, x2);
         store_record(rec, q * S0, q * S1, q * S2, fac);
     }
     if (U) {
@@ -145,6 +154,88 @@ __global__ void __launch_bounds__(256) k_grad_faces(GradArgs a)
             store_record(rec + (int)G, x0, x1, x2, ph);
         }
     }
+}
+
+// Both passes in one launch, for small meshes: a block takes a slice of 32
+// cells, eight lanes a cell.  Each lane evaluates one face as k_grad_faces does
+// (a face is evaluated for both its cells, but all faces of a cell at once), and
+// six threads a cell, one a component, sum the faces in ascending order as
+// k_grad_cells does: the same bits.  Such a call is bound by the host's launches
+// and the passes' latency.  Gradient and velocity, us on the device, two
+// launches and one: 10.0 and 5.2 (800 cells), 13.8 and 10.7 (24x18x12), 11.0 and
+// 9.8 (200x60), 16.3 and 15.2 (30x24x20: 41,400 faces), 12.1 and 17.1 (300x90:
+// 53,610 faces), where evaluating every face twice costs more; called from
+// Python one after another 33 and 29.  The line lies at 45,056 faces.
+template <bool G, bool U>
+__global__ void __launch_bounds__(256) k_grad_small(GradArgs a)
+{
+    __shared__ double part[8][8][33];  // [slot][weight, q S; flux, x][cell]
+    __shared__ int code[8][32];
+    const size_t n = (size_t)a.n, F = (size_t)a.F;
+    const int base = a.cf.ptr[blockIdx.x], w = (a.cf.ptr[blockIdx.x + 1] - base) >> 5;
+    const int c = threadIdx.x >> 3, k = threadIdx.x & 7;
+    const int comp = threadIdx.x >> 5, lane = threadIdx.x & 31, cell = blockIdx.x * 32 + lane;
+    const bool sums = cell < a.n && ((G && comp < 3) || (U && comp >= 3 && comp < 6));
+    double acc = 0.0, xP = 0.0, iv = 0.0;
+    if (sums) {
+        iv = 1.0 / a.V[cell];
+        if (comp >= 3 && a.xf) xP = a.C[(size_t)(comp - 3) * n + cell];
+    }
+    for (int k0 = 0; k0 < w; k0 += 8) {
+        const int fo = k0 + k < w && (int)blockIdx.x * 32 + c < a.n ? a.cf.face[base + (k0 + k) * kSlice + c] : 0;
+        code[k][c] = fo;
+        if (fo != 0) {
+            const int f = (fo > 0 ? fo : -fo) - 1, o = a.owner[f], nb = a.neighbour[f];
+            double x0 = 0.0, x1 = 0.0, x2 = 0.0;
+            if (a.xf) {
+                x0 = a.xf[f];
+                x1 = a.xf[F + f];
+                x2 = a.xf[2 * F + f];
+            }
+            if (G) {
+                const int8_t kind = a.kind[f];
+                const Densities rho = densities(a, f);
+                double q = a.p[nb] - a.p[o];
+                if (kind > 1) {
+                    const double lam = a.lambda[f];
+                    q -= a.jump[f];
+                    q = q / (lam * rho.w + (1.0 - lam) * rho.a);
+                } else {
+                    q = div_known(q, kind ? rho.w : rho.a, kind ? rho.inv_w : rho.inv_a);
+                }
+                const double S0 = a.Sf[f], S1 = a.Sf[F + f], S2 = a.Sf[2 * F + f];
+                const double fac = a.xf ? face_weight(a, f, o, S0, S1, S2, x0, x1, x2) : 0.5;
+                part[k][0][c] = fo > 0 ? fac : 1.0 - fac;
+                part[k][1][c] = q * S0;
+                part[k][2][c] = q * S1;
+                part[k][3][c] = q * S2;
+            }
+            if (U) {
+                const double ph = a.phi[f];
+                if (a.xf) {
+                    part[k][4][c] = fo > 0 ? ph : -ph;
+                    part[k][5][c] = x0;
+                    part[k][6][c] = x1;
+                    part[k][7][c] = x2;
+                } else {
+                    const double h = 0.5 * ph;
+                    part[k][5][c] = h * (a.C[nb] - a.C[o]);
+                    part[k][6][c] = h * (a.C[n + nb] - a.C[n + o]);
+                    part[k][7][c] = h * (a.C[2 * n + nb] - a.C[2 * n + o]);
+                }
+            }
+        }
+        __syncthreads();
+        if (sums)
+            for (int q = 0; q < 8; ++q) {
+                if (code[q][lane] == 0) continue;
+                if (comp < 3) acc = fma(part[q][0][lane], part[q][1 + comp][lane], acc);
+                else if (a.xf) acc = fma(part[q][4][lane], part[q][2 + comp][lane] - xP, acc);
+                else acc += part[q][2 + comp][lane];
+            }
+        __syncthreads();
+    }
+    if (sums) (comp < 3 ? a.grad : a.U)[(size_t)(comp % 3) * n + cell] = acc * iv;
 }
 
 template <bool G, bool U>
@@ -260,6 +351,10 @@ cudaError_t launch_nonorth(const NonorthArgs &a, cudaStream_t s)
 template <bool G, bool U>
 static cudaError_t gradient(const GradArgs &a, cudaStream_t s)
 {
+    if (!a.rec) {
+        k_grad_small<G, U><<<(a.n + 31) / 32, 256, 0, s>>>(a);
+        return cudaGetLastError();
+    }
     k_grad_faces<G, U><<<(a.F + 255) / 256, 256, 0, s>>>(a);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -231,9 +231,10 @@ struct GradArgs {
     double rho_w, rho_a, inv_w, inv_a;
     const int32_t *ftank;              // batched: tank of each face (else nullptr)
     const TankPhys *tphys;             // batched: densities per tank
-    double4 *rec;                      // [2 F] scratch: the faces' records
+    double4 *rec;                      // [2 F] scratch: the faces' records (nullptr: one launch without them)
     double *grad, *U;                  // [3][n] caller order, either nullable
 };
+constexpr int kGradSmallFaces = 45056;  // meshes of fewer faces: one launch (k_grad_small)
 cudaError_t launch_gradient(const GradArgs &a, cudaStream_t s);
 
 // Explicit non-orthogonal correction: corr_f = rau_f k_f . G_f from the
