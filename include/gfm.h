@@ -280,8 +280,8 @@ gfm_status gfm_solve_host(gfm_handle h, const double *alpha_host, const double *
  *   xf [3][F]  face centres, or NULL for the midpoints of the two cell centres
  *              (exact on uniform hex meshes).
  * Works on batched handles (densities per tank).  FP64.  The first gradient
- * (of meshes of 45,056 faces or more) or correction on a handle allocates 64
- * bytes of workspace per face.
+ * or correction on a handle of more than 262,144 faces allocates 64 bytes of
+ * workspace per face (smaller handles hold it from gfm_create on).
  * Errors: GFM_ERR_ARG (NULL p or V, both outputs NULL, U without phi),
  * GFM_ERR_STATE (grad before gfm_assemble), GFM_ERR_NOMEM, GFM_ERR_CUDA.
  */

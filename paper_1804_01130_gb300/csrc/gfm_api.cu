@@ -216,7 +216,9 @@ struct LaunchPlan {
 // The gradient's face records (64 bytes a face), allocated at the first gradient
 // or correction: a handle that only solves or advects has no use for them.
 // That call may be under stream capture, where cudaMalloc is allowed to a
-// thread in relaxed mode.
+// thread in relaxed mode.  Up to kEagerRecFaces (16 MiB) they come with the
+// handle: cudaMalloc takes 60 to 100 us, as much as a small mesh's first call.
+constexpr int kEagerRecFaces = 262144;
 gfm_status need_grad_rec(gfm_ctx *h)
 {
     if (h->grad_rec) return GFM_OK;
@@ -689,6 +691,7 @@ gfm_status alloc_upload(gfm_ctx *h, cudaStream_t s)
     A(prm, 1); A(bar, 1); A(err, 1); A(partials, 2 * (size_t)h->max_grid * gfm::kMaxReduce); A(dinfo, 1);
     A(cc_parent, n); A(cc_size, n); A(cc_cand, gfm::kMaxCandidates); A(cc_counters, 1);
     A(coarse, 1);
+    if (F <= kEagerRecFaces) A(grad_rec, 2 * (size_t)F);
 #undef A
     if (e != cudaSuccess)
         return fail(h, e == cudaErrorMemoryAllocation ? GFM_ERR_NOMEM : GFM_ERR_CUDA,

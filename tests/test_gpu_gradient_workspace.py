@@ -1,5 +1,6 @@
-"""The gradient's workspace: allocated by the first gradient, not by every
-handle, and that first call may be the one a graph captures."""
+"""The gradient's workspace: on meshes of more than 262,144 faces allocated by
+the first gradient, not by every handle, and that first call may be the one a
+graph captures."""
 import numpy as np
 import pytest
 import torch
@@ -43,7 +44,7 @@ def test_first_gradient_allocates_its_workspace():
 def test_first_call_under_capture(call):
     """Gradient: the first call on the handle is the captured one.  Correction:
     its own workspace comes with an earlier call, the records with a gradient."""
-    c = cases.box_case(60, 44, 1, seed=2)
+    c = cases.box_case(400, 400, 1, seed=2)
     a = _inputs(c)
     if call == "gradient":
         ref = [t.clone() for t in _handle(c).gradient(**a)]
