@@ -19,10 +19,8 @@ All use rho_w = 1000, rho_a = 1, g = (0, -9.81, 0), one pinned cell per mesh.
 
 A step = one pass of the hot path on device-resident inputs: assemble the
 GFM system (interface fraction, face coefficients, jump source, cell sums),
-solve it with the mixed-precision persistent solver (FP32 inner PCG inside
-FP64 reliable updates, two-level preconditioner: up to 8 one-phase regions on
-a single mesh, the 2 largest of each tank in a batch), and, on single
-meshes, compute the corrected face flux.  The L2 is flushed (a 512
+solve it with the mixed-precision persistent solver (FP32 CG preconditioned by
+a multigrid V-cycle, inside FP64 residual replacement), and, on single meshes, compute the corrected face flux.  The L2 is flushed (a 512
 MiB write) before every step.
 
 Metric: cell-iterations per second (sum over meshes of cells x CG
@@ -39,7 +37,7 @@ the box and the batch stream ~1.2-1.5 GB per V-cycle through HBM and L2.
 
 Iterations are not alike on the two sides: a GPU iteration is one FP32 PCG
 step preconditioned by a multigrid V-cycle (some five operator passes over the
-mesh, and 20 to 60 iterations a solve); an oracle iteration is one FP64
+mesh, and 16 to 30 iterations a solve here); an oracle iteration is one FP64
 Jacobi-PCG step (one pass, 1 700 to 4 800 iterations).  cpu_baseline therefore
 reports both the oracle's fixed-count rate and its time to the workload's
 tolerance, and ms_per_step and speedup are the figures to compare.

@@ -8,9 +8,10 @@
 // polynomial on [0.35, 2] (the spectrum of D^{-1} A is in [0, 2]) in mirrored
 // order, piecewise constant transfers, and the coarse operator formed by
 // every assembly from the assembled face coefficients (k_mg_level).  The
-// iteration count hardly depends on the mesh size: 20-40 V-cycles for a
-// relative residual of 1e-12 where Jacobi with the deflated one-phase
-// regions took 270 (64x32 tank) to 4300 (1024x512 tank).
+// iteration count hardly depends on the mesh size: 22-52 V-cycles for a
+// relative residual of 1e-12 on tanks up to 20 times as long as deep, where
+// Jacobi iterations number 184 to 6600.  On longer, shallower tanks the merged
+// cells mix water and air: up to 315 V-cycles (529x13 cells, 120 depths long).
 //
 // A V-cycle on the mesh level is five passes over the rows (two sweeps, the
 // residual, two sweeps), all of them gathers of ONE vector, against the one
@@ -1212,13 +1213,13 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
         if (!mg_allreduce<1, A>(c)) { bail(); return; }
         // A tank asks for a residual replacement when its residual claims
         // convergence, can no longer be trusted in FP32 (three decades below
-        // the last true one), has gone kMgCheck32 or kMgCheck64 iterations without one, or
-        // cannot go on.  In a batch a tank that claims convergence idles until
-        // the round, which comes when no tank is left iterating or some tank
-        // must not wait.  In FP64 each claim that the true residual refuted
-        // halves the next one's target: near the rounding floor the true
-        // residual is the recurrence's and x's rounding added up, so a claim
-        // just below the tolerance would be refuted again and again.
+        // the last true one), has gone kMgCheck32 or kMgCheck64 iterations
+        // without one, or cannot go on.  In a batch a tank that claims
+        // convergence idles until the round, which comes when no tank is left
+        // iterating or some tank must not wait.  In FP64 each claim that the
+        // true residual refuted halves the next one's target: near the
+        // rounding floor the true residual is the recurrence's and x's
+        // rounding added up.
         if (threadIdx.x < 32) {
             bool now = false, asked = false, going = false, waits = false;
             for (int t = threadIdx.x; t < T_; t += 32) {
@@ -1241,7 +1242,8 @@ __global__ void __launch_bounds__(NT, 1) k_solve_mg(MgArgs a)
                     sh.flag[t] = kFlagUpdate;
                     sh.wait[t] = 1;
                     asked = waits = true;
-                } else if ((kMixed && rho <= 1e-6 * sh.rho_max[t]) || it - sh.last_rep[t] >= (kMixed ? kMgCheck32 : kMgCheck64)) {
+                } else if ((kMixed && rho <= 1e-6 * sh.rho_max[t]) ||
+                           it - sh.last_rep[t] >= (kMixed ? kMgCheck32 : kMgCheck64)) {
                     sh.flag[t] = kFlagUpdate;
                     sh.wait[t] = 1;
                     asked = waits = true;
