@@ -1,4 +1,4 @@
-"""FP64 multigrid solves whose tolerance lies near the rounding floor: the
+"""Multigrid solves whose tolerance lies near the rounding floor: the
 adjoint of a two-gauge pressure difference (its right-hand side's residual
 cannot be brought below about 6e-13 at 256x128) on many free surfaces, and
 long shallow or tall tanks.  Every solve ends, and with status 0 wherever the
@@ -64,3 +64,15 @@ def test_long_and_tall_tanks_end(nx, ny, aspect):
             assert mg.status == 0 and mg.rel_res_l2 <= 1e-12 and mg.iters < 400, (mg, jacobi)
         else:
             assert mg.status in (0, NOT_CONVERGED) and mg.iters < 2000, (mg, jacobi)
+
+
+def test_mixed_adjoint_just_above_the_floor():
+    """24x18 cells, a band across the surface: the rounding of x leaves about
+    1.0e-13, the Jacobi form ends at 1.6e-13; asked for 1e-13."""
+    c = cases.box_case(24, 18, 1, seed=3, nwaves=2, lx=2.0, ly=1.0, ka=0.05)
+    s = _g().GFM.from_case(c)
+    _assemble(s, c)
+    p, _, _ = s.solve(mode="mixed", rtol=1e-13)
+    w = torch.as_tensor(np.where(np.abs(c.C[1] - 0.5) < 0.15, c.V, 0.0))
+    _, _, _, i = s.adjoint(p, w, mode="mixed", rtol=1e-13, raise_on_error=False)
+    assert i.status == 0 and i.rel_res_l2 <= 1e-13 and i.iters < 100, i
