@@ -135,9 +135,10 @@ def _cores() -> int:
 
 def _traffic_record(workload: str, kernel: str):
     """DRAM bytes per launch of the solver kernel from a committed ncu summary,
-    valid only while the kernel source is unchanged and the capture is of the
-    kernel the bench ran (else None)."""
-    src = os.path.join(ROOT, "paper_1804_01130_gb300", "csrc", "gfm_solve.cu")
+    valid only while the kernel's source file is unchanged and the capture is
+    of the kernel the bench ran (else None)."""
+    unit = "gfm_mg.cu" if "k_solve_mg" in kernel else "gfm_solve.cu"
+    src = os.path.join(ROOT, "paper_1804_01130_gb300", "csrc", unit)
     with open(src, "rb") as fh:
         sha = hashlib.sha256(fh.read()).hexdigest()[:16]
     path = os.path.join(ROOT, "profiles", "ncu_traffic.json")
